@@ -18,16 +18,32 @@
 // rolling resistance M^r = -mu_r R_e |f^n| w_rel/|w_rel|; M^t = r_i n x f^t.
 // The box faces are walls of infinite mass and radius.
 //
-// GPU layout.  One thread per particle, in cell order.  A cell list (edge
-// >= 2 r_max) is rebuilt by counting sort every sub-step; each particle
-// gathers its overlapping partners from the 27 cells around it into a list
-// sorted by partner index (capacity C per particle), merges it with its
-// previous list to carry d_t, and sums its contacts in that order, then the
-// six walls, gravity and the fluid force -- so the forces do not depend on
-// the order in which the cell list was filled, and no atomics touch a
-// force.  Each particle keeps its own copy of a pair's d_t (the partner's is
-// its negative), so i and j never write the same word.  The state is FP64;
-// the contact arithmetic is FP64 or, on the mixed path, FP32.
+// GPU layout.  Four launches per sub-step: the cell ranges, the scatter of
+// the state into cell order, the contact forces, and the rest with the
+// integration.  In the contact kernel eight lanes work on one particle: they
+// walk the rows of its 27 cells in parallel (FP32 screen), sort the partners
+// by index, take one contact each, and add the contacts' forces up in that
+// order -- so the forces do not depend on the order in which the cells were
+// filled, and no atomics touch a force; the six walls follow, a lane each.
+// It reads the cell-ordered copies only.  The last kernel has one thread per
+// particle: gravity and the fluid force, the closing half kick of this
+// sub-step, the opening kick and drift of the next, and the particle's next
+// cell.  (Left to the eight lanes those FP64 instructions took 70 of 132 us:
+// one costs a warp 16 cycles however few of its lanes it serves.)
+//
+// One thread per particle (the form before) left every lane to its own
+// serial chain of 6 to 12 contacts of ~300 dependent operations, and a bed of
+// 5,000 spheres 157 warps for 152 SMs.  Per sub-step, 100,000 spheres on the
+// mixed path 154 -> 90 us (contact kernel 120 -> 63 us, now bound by the
+// latency of its gathers at 64 % of the warps), 5,003 spheres in FP64 190 ->
+// 60 us (181 -> 43 us, bound by the FP64 pipe).
+//
+// Each particle keeps its own copy of a pair's d_t (the partner's is its
+// negative), so i and j never write the same word.  The state is FP64; the
+// contact arithmetic is FP64 or, on the mixed path, FP32 on differences of
+// double-float positions and velocities (FP64 instructions, conversions
+// among them, issue at 1/64 of the FP32 rate here).
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdint>
@@ -46,146 +62,136 @@ namespace {
 constexpr int kDemMaxCap = 64;
 
 struct DemDev {
-  double rho, Y, nu, e, mus, mur;       // particles
-  double Yw, nuw, ew, musw, murw;       // walls
+  double rho;
   double g[3], lo[3], hi[3];
   double rmax;
   int nc[3];                            // cells per axis
-  double inv_ce[3];                     // 1 / cell edge
+  float inv_ce[3];                      // 1 / cell edge
+  df64 ext[3];                          // hi - lo
   int cap;                              // contacts per particle
-  // host-computed constants: -2 sqrt(5/6) beta(e) for particle pairs and
-  // walls, effective Young's and shear moduli of particle-particle and
-  // particle-wall contacts
-  double c56, c56w, Ye, Ge, Yew, Gew;
 };
 
-__device__ __forceinline__ double d_dot(const double* a, const double* b) {
-  return a[0] * b[0] + a[1] * b[1] + a[2] * b[2];
-}
-
-// one contact's force (added to F) and torque (added to T) on particle i,
-// advancing the carried tangential displacement th in place; T = double
-// (FP64 path) or float (mixed path: the overlap arrives from an FP64
-// difference, the rest of the contact in FP32)
+// The constants of a kind of contact (particle-particle, particle-wall):
+// effective Young's and shear moduli, -2 sqrt(5/6) beta(e) sqrt(2 Y_e) and
+// ... sqrt(8 G_e), so that eta_n and eta_t share one root, the friction
+// coefficients, and the mass of a particle of radius 1.  Kept in the type of
+// the arithmetic: converting a kernel argument from FP64 is an FP64-pipe
+// instruction of its own.
 template <typename R>
-__device__ void dem_contact(const R* n, R dn, const R* vrel, const R* wrel, R ri, R me, R Re,
-                            R Ye, R Ge, R c56, R mus, R mur, R dt, R* th, R* F, R* Tq) {
+struct Contact {
+  R Ye, Ge, en, et, mus, mur, mass1;
+};
+
+// One contact's force F and torque Tq on particle i, advancing the carried
+// tangential displacement th in place; T = double (FP64 path) or float
+// (mixed path).  sq = sqrt(R_e d_n); |f^n| is the magnitude of its one
+// component along n.
+template <typename R>
+__device__ __forceinline__ void dem_contact(const R* n, R dn, const R* vrel, const R* wrel, R ri,
+                                            R me, R Re, const Contact<R>& k, R dt, R* th, R* F,
+                                            R* Tq) {
   const R vn = n[0] * vrel[0] + n[1] * vrel[1] + n[2] * vrel[2];
-  R vrn[3], vrt[3];
-  for (int a = 0; a < 3; ++a) {
-    vrn[a] = vn * n[a];
-    vrt[a] = vrel[a] - vrn[a];
-  }
+  R vrt[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) vrt[a] = vrel[a] - vn * n[a];
   const R sq = t_sqrt<R>(Re * dn);
-  const R kn = (R)(4.0 / 3.0) * Ye * sq;
-  const R kt = (R)8 * Ge * sq;
-  const R Sn = (R)2 * Ye * sq;
-  const R St = (R)8 * Ge * sq;
-  const R etan = c56 * t_sqrt<R>(Sn * me);
-  const R etat = c56 * t_sqrt<R>(St * me);
+  const R root = t_sqrt<R>(sq * me);
+  const R etan = k.en * root, etat = k.et * root;
+  const R kn = (R)(4.0 / 3.0) * k.Ye * sq;
+  const R kt = (R)8 * k.Ge * sq;
   const R hn = th[0] * n[0] + th[1] * n[1] + th[2] * n[2];
-  for (int a = 0; a < 3; ++a) th[a] = th[a] - hn * n[a] + vrt[a] * dt;
-  R fn[3], ft[3];
+  const R fnn = kn * dn + etan * vn;  // f^n = -fnn n
+  const R fnm = fabs(fnn);
+  R ft[3];
+#pragma unroll
   for (int a = 0; a < 3; ++a) {
-    fn[a] = -(kn * dn) * n[a] - etan * vrn[a];
+    th[a] = th[a] - hn * n[a] + vrt[a] * dt;
     ft[a] = -kt * th[a] - etat * vrt[a];
   }
-  const R fnm = t_sqrt<R>(fn[0] * fn[0] + fn[1] * fn[1] + fn[2] * fn[2]);
   const R ftm = t_sqrt<R>(ft[0] * ft[0] + ft[1] * ft[1] + ft[2] * ft[2]);
-  if (ftm > mus * fnm) {
-    const R sc = mus * fnm / ftm;
+  if (ftm > k.mus * fnm) {
+    const R sc = k.mus * fnm / ftm, ikt = (R)1 / kt;
+#pragma unroll
     for (int a = 0; a < 3; ++a) {
       ft[a] = ft[a] * sc;
-      th[a] = -(ft[a] + etat * vrt[a]) / kt;
+      th[a] = -(ft[a] + etat * vrt[a]) * ikt;
     }
   }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) F[a] = ft[a] - fnn * n[a];
   // (r_i n) x f^t
-  const R mt[3] = {ri * (n[1] * ft[2] - n[2] * ft[1]), ri * (n[2] * ft[0] - n[0] * ft[2]),
-                   ri * (n[0] * ft[1] - n[1] * ft[0])};
-  const R wm = t_sqrt<R>(wrel[0] * wrel[0] + wrel[1] * wrel[1] + wrel[2] * wrel[2]);
-  for (int a = 0; a < 3; ++a) {
-    F[a] += fn[a] + ft[a];
-    Tq[a] += mt[a];
-    if (wm > (R)0) Tq[a] += -mur * Re * fnm * wrel[a] / wm;
+  Tq[0] = ri * (n[1] * ft[2] - n[2] * ft[1]);
+  Tq[1] = ri * (n[2] * ft[0] - n[0] * ft[2]);
+  Tq[2] = ri * (n[0] * ft[1] - n[1] * ft[0]);
+  if (k.mur > (R)0) {
+    const R wm = t_sqrt<R>(wrel[0] * wrel[0] + wrel[1] * wrel[1] + wrel[2] * wrel[2]);
+    if (wm > (R)0) {
+      const R c = k.mur * Re * fnm / wm;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) Tq[a] -= c * wrel[a];
+    }
   }
 }
 
-__device__ __forceinline__ int cell_axis(double x, double lo, double inv_ce, int nc) {
-  int c = (int)floor((x - lo) * inv_ce);
-  return c < 0 ? 0 : (c > nc - 1 ? nc - 1 : c);
+// cell along one axis, in FP32: a cell is at least 2 r_max (1 + 2^-9) wide and
+// there are at most 4096, so the rounding of the quotient (4 x 2^-24 x 4096)
+// cannot put touching particles two cells apart
+__device__ __forceinline__ int cell_axis(double x, double lo, float inv_ce, int nc) {
+  const float t = (float)(x - lo) * inv_ce;
+  return t >= 1.0f ? (t < (float)nc ? (int)t : nc - 1) : 0;  // NaN to 0
 }
 
-// The Velocity Verlet updates, with explicit FMAs so that the fused kernel
-// below gives the same bits as the two it replaces.
+// The Velocity Verlet updates, with explicit FMAs so that the forces' kernel
+// and the one below give the same bits.
 __device__ __forceinline__ void half_kick(double hdt, double a, double& v) { v = fma(hdt, a, v); }
 
-// first half kick and drift
-__global__ void k_dem_kick_drift(int64_t n, double dt, double* __restrict__ x,
-                                 double* __restrict__ v, double* __restrict__ w,
-                                 const double* __restrict__ acc,
-                                 const double* __restrict__ alpha) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= 3 * n) return;
-  double vt = v[t], wt = w[t];
-  half_kick(0.5 * dt, acc[t], vt);
-  half_kick(0.5 * dt, alpha[t], wt);
-  v[t] = vt;
-  w[t] = wt;
-  x[t] = fma(dt, vt, x[t]);
+// cell of a position (cell_axis per axis)
+__device__ __forceinline__ int cell_of_axes(const DemDev& p, int cx, int cy, int cz) {
+  return cx + p.nc[0] * (cy + p.nc[1] * cz);
 }
 
-// second half kick
-__global__ void k_dem_kick(int64_t n, double dt, double* __restrict__ v, double* __restrict__ w,
-                           const double* __restrict__ acc, const double* __restrict__ alpha) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= 3 * n) return;
-  double vt = v[t], wt = w[t];
-  half_kick(0.5 * dt, acc[t], vt);
-  half_kick(0.5 * dt, alpha[t], wt);
-  v[t] = vt;
-  w[t] = wt;
-}
-
-// the second half kick of one sub-step and the first half kick and drift of
-// the next, in one pass
-__global__ void k_dem_kick_kick_drift(int64_t n, double dt, double* __restrict__ x,
-                                      double* __restrict__ v, double* __restrict__ w,
-                                      const double* __restrict__ acc,
-                                      const double* __restrict__ alpha) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= 3 * n) return;
-  const double a = acc[t], al = alpha[t];
-  double vt = v[t], wt = w[t];
-  half_kick(0.5 * dt, a, vt);
-  half_kick(0.5 * dt, al, wt);
-  half_kick(0.5 * dt, a, vt);
-  half_kick(0.5 * dt, al, wt);
-  v[t] = vt;
-  w[t] = wt;
-  x[t] = fma(dt, vt, x[t]);
-}
-
-// cell of every particle and its slot in the cell (counting sort, pass 1);
-// a radius above the stated maximum raises the flag
-__global__ void k_dem_cell_count(int64_t n, DemDev p, const double* __restrict__ x,
-                                 const double* __restrict__ r, int32_t* __restrict__ cell_of,
-                                 int32_t* __restrict__ slot, int32_t* __restrict__ count,
-                                 int* __restrict__ flags) {
+// the start of a call: with `kick` (the accelerations of the last call are
+// there) the first half kick and drift; then the cell of every particle and
+// its slot in the cell, and its inverse mass and moment of inertia; a radius
+// above the stated maximum raises the flag
+__global__ void k_dem_begin(int64_t n, DemDev p, double dt, int kick, double* __restrict__ x,
+                            double* __restrict__ v, double* __restrict__ w,
+                            const double* __restrict__ r, const double* __restrict__ acc,
+                            const double* __restrict__ alpha, int32_t* __restrict__ cell_of,
+                            int32_t* __restrict__ slot, int32_t* __restrict__ count,
+                            double2* __restrict__ inv, int* __restrict__ flags) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const int cx = cell_axis(x[3 * i], p.lo[0], p.inv_ce[0], p.nc[0]);
-  const int cy = cell_axis(x[3 * i + 1], p.lo[1], p.inv_ce[1], p.nc[1]);
-  const int cz = cell_axis(x[3 * i + 2], p.lo[2], p.inv_ce[2], p.nc[2]);
-  const int c = cx + p.nc[0] * (cy + p.nc[1] * cz);
-  cell_of[i] = c;
-  slot[i] = atomicAdd(count + c, 1);
-  if (!(r[i] <= p.rmax)) atomicOr(flags, 2);
+  int c[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const int64_t t = 3 * i + a;
+    double xt = x[t];
+    if (kick) {
+      double vt = v[t], wt = w[t];
+      half_kick(0.5 * dt, acc[t], vt);
+      half_kick(0.5 * dt, alpha[t], wt);
+      v[t] = vt;
+      w[t] = wt;
+      x[t] = xt = fma(dt, vt, xt);
+    }
+    c[a] = cell_axis(xt, p.lo[a], p.inv_ce[a], p.nc[a]);
+  }
+  const int cell = cell_of_axes(p, c[0], c[1], c[2]);
+  cell_of[i] = cell;
+  slot[i] = atomicAdd(count + cell, 1);
+  const double ri = r[i];
+  if (!(ri <= p.rmax)) atomicOr(flags, 2);
+  const double mi = p.rho * (4.0 / 3.0 * kPi) * ri * ri * ri;
+  inv[i] = make_double2(1.0 / mi, 1.0 / (0.4 * mi * ri * ri));
 }
 
-// exclusive scan of count[0..nc) into start[0..nc]: tiles of 1024 cells
-// (256 threads x 4) are summed, the tile sums scanned by one block, then
-// every tile scans itself from its offset
-constexpr int kScanTile = 1024;
+// The cells' ranges in cell order.  Only the cells of one x-row have to lie
+// next to each other, so a block takes whole rows (about 2048 cells, at least
+// one row), scans them and reserves its range with one atomic addition: one
+// launch where a scan over all cells takes three.  Also clears the counters
+// of the next sub-step.
+constexpr int kRangeTile = 2048, kRangePer = 16;  // 256 threads x 16 >= 4096 cells
 
 __device__ __forceinline__ int32_t block_excl_scan256(int32_t v, int32_t* sh, int32_t* total) {
   const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
@@ -214,67 +220,88 @@ __device__ __forceinline__ int32_t block_excl_scan256(int32_t v, int32_t* sh, in
 }
 
 __global__ void __launch_bounds__(256)
-k_dem_scan_tiles(int ncells, const int32_t* __restrict__ count, int32_t* __restrict__ tsum) {
-  __shared__ int32_t sh[16];
-  const int base = blockIdx.x * kScanTile + threadIdx.x * 4;
-  int32_t v = 0;
-  for (int q = 0; q < 4; ++q) v += base + q < ncells ? count[base + q] : 0;
-  int32_t tot;
-  block_excl_scan256(v, sh, &tot);
-  if (threadIdx.x == 0) tsum[blockIdx.x] = tot;
-}
-
-__global__ void __launch_bounds__(256)
-k_dem_scan_sums(int ntiles, int32_t* __restrict__ tsum) {  // in place, exclusive; tsum[ntiles] = total
-  __shared__ int32_t sh[16];
-  int32_t run = 0;
-  for (int b0 = 0; b0 < ntiles; b0 += 256) {
-    const int b = b0 + threadIdx.x;
-    const int32_t v = b < ntiles ? tsum[b] : 0;
-    int32_t tot;
-    const int32_t ex = block_excl_scan256(v, sh, &tot);
-    if (b < ntiles) tsum[b] = run + ex;
-    run += tot;
-  }
-  if (threadIdx.x == 0) tsum[ntiles] = run;
-}
-
-__global__ void __launch_bounds__(256)
-k_dem_scan_final(int ncells, const int32_t* __restrict__ count,
-                 const int32_t* __restrict__ tsum, int32_t* __restrict__ start) {
-  __shared__ int32_t sh[16];
-  const int base = blockIdx.x * kScanTile + threadIdx.x * 4;
-  int32_t c[4], v = 0;
-  for (int q = 0; q < 4; ++q) {
-    c[q] = base + q < ncells ? count[base + q] : 0;
+k_dem_ranges(int ncells, int tile, const int32_t* __restrict__ count, int32_t* __restrict__ next,
+             int32_t* __restrict__ total, int32_t* __restrict__ start) {
+  __shared__ int32_t sh[17];
+  const int t0 = blockIdx.x * tile;
+  const int nt = min(tile, ncells - t0);
+  const int per = (tile + 255) / 256;  // <= kRangePer
+  const int c0 = threadIdx.x * per;
+  int32_t c[kRangePer], v = 0;
+#pragma unroll
+  for (int q = 0; q < kRangePer; ++q) {
+    c[q] = q < per && c0 + q < nt ? count[t0 + c0 + q] : 0;
     v += c[q];
   }
   int32_t tot;
-  int32_t run = tsum[blockIdx.x] + block_excl_scan256(v, sh, &tot);
-  for (int q = 0; q < 4; ++q) {
-    if (base + q < ncells) start[base + q] = run;
-    run += c[q];
-  }
-  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) start[ncells] = tsum[gridDim.x];
+  int32_t run = block_excl_scan256(v, sh, &tot);
+  if (threadIdx.x == 0) sh[16] = atomicAdd(total, tot);
+  __syncthreads();
+  run += sh[16];
+#pragma unroll
+  for (int q = 0; q < kRangePer; ++q)
+    if (q < per && c0 + q < nt) {
+      start[t0 + c0 + q] = run;
+      next[t0 + c0 + q] = 0;
+      run += c[q];
+    }
 }
 
-// pass 3: the particle's place in cell order, with an FP32 copy of its
-// position (offset from the box's low corner) and radius at that place;
-// also FP32 copies of its angular velocity and radius by particle index
+// The state in cell order, for the contacts.  xs: FP32 position (offset from
+// the box's low corner) and radius, for the screen and as the high parts on
+// the mixed path.
+struct DemCells {
+  float4* xs;
+  int32_t* perm;   // particle at each place
+  int32_t* cell;   // and its cell
+  // mixed: low parts of position and radius, high and low parts of the
+  // velocity, angular velocity; FP64: position and radius, v, w
+  float4 *xl, *vh, *vl, *wf;
+  double2 *xr, *vw;  // [n][2], [n][3]
+};
+
+template <typename R>
 __global__ void k_dem_cell_scatter(int64_t n, DemDev p, const double* __restrict__ x,
-                                   const double* __restrict__ w, const double* __restrict__ r,
+                                   const double* __restrict__ v, const double* __restrict__ w,
+                                   const double* __restrict__ r,
                                    const int32_t* __restrict__ cell_of,
                                    const int32_t* __restrict__ slot,
-                                   const int32_t* __restrict__ start, int32_t* __restrict__ perm,
-                                   float4* __restrict__ xs, float4* __restrict__ wf) {
+                                   const int32_t* __restrict__ start, DemCells cs,
+                                   int32_t* __restrict__ total) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i == 0) *total = 0;  // for the ranges of the next sub-step
   if (i >= n) return;
-  const int32_t s = start[cell_of[i]] + slot[i];
-  const float rf = (float)r[i];
-  perm[s] = (int32_t)i;
-  xs[s] = make_float4((float)(x[3 * i] - p.lo[0]), (float)(x[3 * i + 1] - p.lo[1]),
-                      (float)(x[3 * i + 2] - p.lo[2]), rf);
-  wf[i] = make_float4((float)w[3 * i], (float)w[3 * i + 1], (float)w[3 * i + 2], rf);
+  const int32_t c = cell_of[i];
+  const int32_t s = start[c] + slot[i];
+  cs.perm[s] = (int32_t)i;
+  cs.cell[s] = c;
+  const double xd[3] = {x[3 * i], x[3 * i + 1], x[3 * i + 2]};
+  const double vd[3] = {v[3 * i], v[3 * i + 1], v[3 * i + 2]};
+  const double wd[3] = {w[3 * i], w[3 * i + 1], w[3 * i + 2]};
+  const double rd = r[i];
+  if (std::is_same<R, double>::value) {
+    cs.xs[s] = make_float4((float)(xd[0] - p.lo[0]), (float)(xd[1] - p.lo[1]),
+                           (float)(xd[2] - p.lo[2]), (float)rd);
+    cs.xr[2 * (int64_t)s] = make_double2(xd[0], xd[1]);
+    cs.xr[2 * (int64_t)s + 1] = make_double2(xd[2], rd);
+    cs.vw[3 * (int64_t)s] = make_double2(vd[0], vd[1]);
+    cs.vw[3 * (int64_t)s + 1] = make_double2(vd[2], wd[0]);
+    cs.vw[3 * (int64_t)s + 2] = make_double2(wd[1], wd[2]);
+  } else {
+    df64 q[4], u[3], om[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      q[a] = df_from_double_int(xd[a] - p.lo[a]);
+      u[a] = df_from_double_int(vd[a]);
+      om[a] = df_from_double_int(wd[a]);
+    }
+    q[3] = df_from_double_int(rd);
+    cs.xs[s] = make_float4(q[0].hi, q[1].hi, q[2].hi, q[3].hi);
+    cs.xl[s] = make_float4(q[0].lo, q[1].lo, q[2].lo, q[3].lo);
+    cs.vh[s] = make_float4(u[0].hi, u[1].hi, u[2].hi, 0.0f);
+    cs.vl[s] = make_float4(u[0].lo, u[1].lo, u[2].lo, 0.0f);
+    cs.wf[s] = make_float4(om[0].hi + om[0].lo, om[1].hi + om[1].lo, om[2].hi + om[2].lo, 0.0f);
+  }
 }
 
 // max |coordinate| of an FP32 position copy
@@ -282,209 +309,412 @@ __device__ __forceinline__ float abs_max3(float4 q) {
   return fmaxf(fabsf(q.x), fmaxf(fabsf(q.y), fabsf(q.z)));
 }
 
-// the FP64 contact test of a screened candidate: d2 < (r_i + r_j)^2, and on
-// the FP64 path also 0 < |d| < r_i + r_j on the root (the oracle's test)
+// a particle at a place of the cell order, as the contacts use it
 template <typename R>
-__device__ __forceinline__ bool dem_touch(const double* __restrict__ x,
-                                          const double* __restrict__ r, int32_t j,
-                                          const double* xi, double ri) {
-  const double d[3] = {x[3 * j] - xi[0], x[3 * j + 1] - xi[1], x[3 * j + 2] - xi[2]};
-  const double d2 = d_dot(d, d);
-  const double rs = ri + r[j];
-  if (!(d2 < rs * rs)) return false;
-  if (std::is_same<R, double>::value) {
-    const double dist = sqrt(d2);
-    return dist < rs && dist > 0.0;
+struct Body;
+template <>
+struct Body<double> {
+  double x[3], r;
+  __device__ __forceinline__ void load(const DemCells& cs, int64_t s) {
+    const double2 a = __ldg(cs.xr + 2 * s), b = __ldg(cs.xr + 2 * s + 1);
+    x[0] = a.x;
+    x[1] = a.y;
+    x[2] = b.x;
+    r = b.y;
   }
-  return d2 > 0.0;
+};
+template <>
+struct Body<float> {
+  df64 x[3], r;
+  __device__ __forceinline__ void load(const DemCells& cs, int64_t s) {
+    const float4 h = __ldg(cs.xs + s), l = __ldg(cs.xl + s);
+    x[0] = df64(h.x, l.x);
+    x[1] = df64(h.y, l.y);
+    x[2] = df64(h.z, l.z);
+    r = df64(h.w, l.w);
+  }
+};
+
+// The contact test of a pair: n from i to j and the overlap.  FP64: |d| > 0
+// and |d| < r_i + r_j on the root.  Mixed: the overlap is (rs^2 - d^2) /
+// (rs + d) with the difference of squares in double-float, so the small
+// overlap keeps its digits.
+__device__ __forceinline__ bool dem_pair(const Body<double>& a, const Body<double>& b, double* nrm,
+                                         double* dn) {
+  const double d[3] = {b.x[0] - a.x[0], b.x[1] - a.x[1], b.x[2] - a.x[2]};
+  const double dist = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
+  const double rs = a.r + b.r;
+  if (!(dist < rs && dist > 0.0)) return false;
+  const double inv = 1.0 / dist;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) nrm[c] = d[c] * inv;
+  *dn = rs - dist;
+  return true;
+}
+__device__ __forceinline__ bool dem_pair(const Body<float>& a, const Body<float>& b, float* nrm,
+                                         float* dn) {
+  const df64 d[3] = {b.x[0] - a.x[0], b.x[1] - a.x[1], b.x[2] - a.x[2]};
+  const df64 d2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+  const df64 rs = a.r + b.r;
+  const df64 over = rs * rs - d2;
+  if (!((over.hi > 0.0f || (over.hi == 0.0f && over.lo > 0.0f)) && d2.hi > 0.0f)) return false;
+  const float dist = sqrtf(d2.hi);
+  const float inv = 1.0f / dist;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) nrm[c] = d[c].hi * inv;
+  *dn = over.hi / (rs.hi + dist);
+  return true;
 }
 
-// forces and torques on every particle; tangential displacements advance by
-// dt (0 for the first evaluation of a fresh state).  Thread t takes the
-// particle at place t of the cell order, so the threads of a warp share
-// most of their 27 cells.  The candidates are screened in FP32 on the
-// cell-ordered copy: a stored coordinate is within 2^-24 of its magnitude
-// of the FP64 offset and the FP32 difference adds 2^-24 |d|, so
-// |d_f - d| <= sqrt(3) 2^-24 (M_i + M_j + |d|) (M = largest |coordinate|);
-// the screen passes |d_f| < (r_i + r_j)(1 + 2^-18) + 2^-18 (M_i + M_j), a
-// bound more than ten times that error plus the rounding of the squares,
-// so no pair the FP64 test accepts is screened out.  The screened
-// candidates are kept sorted by index and the FP64 test (dem_touch) runs
-// on them afterwards, once per candidate, outside the divergent cell walk.
-// The contact arithmetic runs in R (double, or float on the mixed path,
-// where the overlap is (rs^2 - d^2) / (rs + d) with the difference of
-// squares in FP64, so the small overlap keeps its digits, and the carried
-// tangential displacements are stored in FP32).
+// relative velocity v_i - v_j and angular velocities of places s (own) and q
+__device__ __forceinline__ void dem_motion(const DemCells& cs, int64_t s, double* v, double* w) {
+  const double2 a = __ldg(cs.vw + 3 * s), b = __ldg(cs.vw + 3 * s + 1), c = __ldg(cs.vw + 3 * s + 2);
+  v[0] = a.x;
+  v[1] = a.y;
+  v[2] = b.x;
+  w[0] = b.y;
+  w[1] = c.x;
+  w[2] = c.y;
+}
+__device__ __forceinline__ void dem_relative(const DemCells& cs, int64_t s, int64_t q, double* dv,
+                                             double* wi, double* wj) {
+  double vi[3], vj[3];
+  dem_motion(cs, s, vi, wi);
+  dem_motion(cs, q, vj, wj);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) dv[a] = vi[a] - vj[a];
+}
+__device__ __forceinline__ void dem_relative(const DemCells& cs, int64_t s, int64_t q, float* dv,
+                                             float* wi, float* wj) {
+  const float4 hi = __ldg(cs.vh + s), li = __ldg(cs.vl + s), hj = __ldg(cs.vh + q),
+               lj = __ldg(cs.vl + q), a = __ldg(cs.wf + s), b = __ldg(cs.wf + q);
+  dv[0] = (hi.x - hj.x) + (li.x - lj.x);
+  dv[1] = (hi.y - hj.y) + (li.y - lj.y);
+  dv[2] = (hi.z - hj.z) + (li.z - lj.z);
+  wi[0] = a.x;
+  wi[1] = a.y;
+  wi[2] = a.z;
+  wj[0] = b.x;
+  wj[1] = b.y;
+  wj[2] = b.z;
+}
+// own velocity and angular velocity, and the overlap with wall `wl` (x-, x+,
+// y-, ...; positive in contact)
+__device__ __forceinline__ void dem_own(const DemCells& cs, int64_t s, double* v, double* w) {
+  dem_motion(cs, s, v, w);
+}
+__device__ __forceinline__ void dem_own(const DemCells& cs, int64_t s, float* v, float* w) {
+  const float4 h = __ldg(cs.vh + s), l = __ldg(cs.vl + s), a = __ldg(cs.wf + s);
+  v[0] = h.x + l.x;
+  v[1] = h.y + l.y;
+  v[2] = h.z + l.z;
+  w[0] = a.x;
+  w[1] = a.y;
+  w[2] = a.z;
+}
+__device__ __forceinline__ double wall_overlap(const DemDev& p, const Body<double>& b, int wl) {
+  const double xa = wl < 2 ? b.x[0] : (wl < 4 ? b.x[1] : b.x[2]);
+  const double lo = wl < 2 ? p.lo[0] : (wl < 4 ? p.lo[1] : p.lo[2]);
+  const double hi = wl < 2 ? p.hi[0] : (wl < 4 ? p.hi[1] : p.hi[2]);
+  return wl & 1 ? b.r - (hi - xa) : b.r - (xa - lo);
+}
+__device__ __forceinline__ float wall_overlap(const DemDev& p, const Body<float>& b, int wl) {
+  const df64 xa = wl < 2 ? b.x[0] : (wl < 4 ? b.x[1] : b.x[2]);  // from the low corner
+  const df64 ext = wl < 2 ? p.ext[0] : (wl < 4 ? p.ext[1] : p.ext[2]);
+  return (wl & 1 ? b.r - (ext - xa) : b.r - xa).hi;
+}
+__device__ __forceinline__ double body_radius(const Body<double>& b) { return b.r; }
+__device__ __forceinline__ float body_radius(const Body<float>& b) { return b.r.hi + b.r.lo; }
+
+// contact lists of the last and of this evaluation: partners ascending, one -1
+// behind the last (C per particle), and their tangential displacements; the
+// walls' (valid where the particle's bit of wmask is set)
 template <typename R>
-__global__ void __launch_bounds__(128)
-k_dem_forces(int64_t n, DemDev p, double dt, const double* __restrict__ x,
-             const double* __restrict__ v, const double* __restrict__ w,
-             const double* __restrict__ r, const double* __restrict__ f_ext,
-             const int32_t* __restrict__ start, const int32_t* __restrict__ perm,
-             const float4* __restrict__ xs, const float4* __restrict__ wf,
-             const int32_t* __restrict__ hj_old, const R* __restrict__ ht_old,
-             int32_t* __restrict__ hj_new, R* __restrict__ ht_new, double* __restrict__ wh,
-             double* __restrict__ acc, double* __restrict__ alpha, int* __restrict__ flags) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  // the warp's live threads meet again after each divergent loop: without
-  // it they stay split into the groups the cell walk left them in, and every
-  // later instruction issues once per group
-  const unsigned live = __ballot_sync(0xffffffffu, t < n);
-  if (t >= n) return;
-  const int64_t i = perm[t];
+struct DemHist {
+  const int32_t* j_old;
+  const R* t_old;
+  int32_t* j_new;
+  R* t_new;
+  R* wall;
+  unsigned char* wmask;
+};
+
+constexpr int kLanes = 8;                     // lanes per particle
+constexpr int kDemBlock = 128, kDemPer = kDemBlock / kLanes;
+
+// Contact forces and torques of every particle, sums[i][6].  Group g of eight
+// lanes takes the particle at place g of the cell order, so that the lanes of
+// a warp share most of their cells.  The candidates are screened in FP32 on
+// the cell-ordered copy: a stored coordinate is within 2^-23 of its magnitude
+// of the FP64 offset and the FP32 difference adds 2^-24 |d|, so |d_f - d| <=
+// sqrt(3) 2^-23 (M_i + M_j + |d|) (M = largest |coordinate|); the screen
+// passes |d_f| < (r_i + r_j)(1 + 2^-18) + 2^-18 (M_i + M_j), a bound more
+// than ten times that error plus the rounding of the squares, so no touching
+// pair is screened out.  dt: advance of the tangential displacements (0 for
+// the first evaluation of a fresh state).
+template <typename R>
+__global__ void __launch_bounds__(kDemBlock, std::is_same<R, float>::value ? 8 : 5)
+k_dem_forces(int64_t n, DemDev p, Contact<R> k, Contact<R> kw, R dt,
+             const int32_t* __restrict__ start, const int32_t* __restrict__ count, DemCells cs, DemHist<R> h,
+             R* __restrict__ sums, int* __restrict__ flags) {
+  __shared__ int32_t s_j[kDemPer][kDemMaxCap], s_at[kDemPer][kDemMaxCap];
+  __shared__ unsigned char s_ord[kDemPer][kDemMaxCap];
+  __shared__ int32_t s_old[kDemPer][kDemMaxCap];
+  __shared__ int s_n[kDemPer];
+  __shared__ R s_f[kDemPer][kLanes][6];
+  const int lane = threadIdx.x % kLanes, grp = threadIdx.x / kLanes;
+  const int base = (threadIdx.x & 31) - lane;  // the group's first lane in its warp
+  const unsigned below = (1u << lane) - 1u;
+  const int64_t t = blockIdx.x * (int64_t)kDemPer + grp;
+  const bool live = t < n;
+  const int64_t at = live ? t : 0;
+  const int64_t i = cs.perm[at];
   const int C = p.cap;
-  const double xi[3] = {x[3 * i], x[3 * i + 1], x[3 * i + 2]};
-  const double ri = r[i];
-  const float4 qi = xs[t];
+  // the last contact list and its length
+  int len = C;
+  for (int c = lane; c < C; c += kLanes) {
+    const int32_t j = h.j_old[i * C + c];
+    s_old[grp][c] = j;
+    if (j < 0) len = min(len, c);
+  }
+#pragma unroll
+  for (int o = 1; o < kLanes; o <<= 1) len = min(len, __shfl_xor_sync(0xffffffffu, len, o));
+
+  // ---- partners: lane l walks the row l of the nine, all lanes the ninth
+  const float4 qi = __ldg(cs.xs + at);
   const float Mi = abs_max3(qi);
   constexpr float kScreen = 3.814697265625e-06f;  // 2^-18
-  // screened partners, sorted by index (insertion into a list of at most
-  // kDemMaxCap; a full list drops the screened-in pairs the FP64 test
-  // rejects before it takes another)
-  int32_t cand[kDemMaxCap];
-  int nc = 0;
-  const int cx = cell_axis(xi[0], p.lo[0], p.inv_ce[0], p.nc[0]);
-  const int cy = cell_axis(xi[1], p.lo[1], p.inv_ce[1], p.nc[1]);
-  const int cz = cell_axis(xi[2], p.lo[2], p.inv_ce[2], p.nc[2]);
-  for (int dz = -1; dz <= 1; ++dz) {
-    const int z = cz + dz;
-    if (z < 0 || z >= p.nc[2]) continue;
-    for (int dy = -1; dy <= 1; ++dy) {
-      const int y = cy + dy;
-      if (y < 0 || y >= p.nc[1]) continue;
-      // the three cells of a row along x are contiguous in cell order
-      const int row = p.nc[0] * (y + p.nc[1] * z);
-      const int s0 = start[row + (cx > 0 ? cx - 1 : 0)];
-      const int s1 = start[row + (cx < p.nc[0] - 1 ? cx + 2 : p.nc[0])];
-      for (int s = s0; s < s1; ++s) {
-        if (s == t) continue;
-        const float4 qj = xs[s];
-        const float ex = qj.x - qi.x, ey = qj.y - qi.y, ez = qj.z - qi.z;
-        const float M = Mi + abs_max3(qj);
-        const float lim = (qi.w + qj.w) * (1.0f + kScreen) + kScreen * M;
-        // positions beyond FP32 range (M not finite) skip the screen
-        if (!(ex * ex + ey * ey + ez * ez < lim * lim) && M < 3.0e38f) continue;
-        const int32_t j = perm[s];
-        if (nc == kDemMaxCap) {
-          int m = 0;
-          for (int q = 0; q < nc; ++q)
-            if (dem_touch<R>(x, r, cand[q], xi, ri)) cand[m++] = cand[q];
-          nc = m;
-          if (nc == kDemMaxCap) {  // 65 contacts: above any capacity
-            if (dem_touch<R>(x, r, j, xi, ri)) atomicOr(flags, 1);
-            continue;
-          }
-        }
-        int q = nc++;
-        while (q > 0 && cand[q - 1] > j) {
-          cand[q] = cand[q - 1];
-          --q;
-        }
-        cand[q] = j;
+  Body<R> me_b;
+  me_b.load(cs, at);
+  const int cell = cs.cell[at];
+  const int cyz = cell / p.nc[0], cx = cell - cyz * p.nc[0];
+  const int cz = cyz / p.nc[1], cy = cyz - cz * p.nc[1];
+  // range of row q (0..8): places [lo, hi) of its three cells
+  auto row_range = [&](int q, int& lo, int& hi) {
+    const int y = cy + q % 3 - 1, z = cz + q / 3 - 1;
+    lo = hi = 0;
+    if (!live || y < 0 || y >= p.nc[1] || z < 0 || z >= p.nc[2]) return;
+    const int row = p.nc[0] * (y + p.nc[1] * z);
+    const int last = row + (cx < p.nc[0] - 1 ? cx + 1 : cx);
+    lo = start[row + (cx > 0 ? cx - 1 : 0)];
+    hi = start[last] + count[last];
+  };
+  auto screen = [&](int s) {
+    const float4 qj = __ldg(cs.xs + s);
+    const float ex = qj.x - qi.x, ey = qj.y - qi.y, ez = qj.z - qi.z;
+    const float M = Mi + abs_max3(qj);
+    const float lim = (qi.w + qj.w) * (1.0f + kScreen) + kScreen * M;
+    // positions beyond FP32 range (M not finite) skip the screen
+    return ex * ex + ey * ey + ez * ez < lim * lim || !(M < 3.0e38f);
+  };
+  // a candidate joins the group's list; `exact` lets only touching pairs in
+  auto visit = [&](int s, bool exact) {
+    if (s == (int)at || !screen(s)) return;
+    if (exact) {
+      Body<R> o;
+      R nr[3], dn;
+      o.load(cs, s);
+      if (!dem_pair(me_b, o, nr, &dn)) return;
+    }
+    const int q = atomicAdd(&s_n[grp], 1);
+    if (q < kDemMaxCap) {
+      s_j[grp][q] = __ldg(cs.perm + s);
+      s_at[grp][q] = s;
+    }
+  };
+  auto search = [&](bool exact) {
+    int lo, hi;
+    row_range(lane, lo, hi);
+    for (; lo < hi; ++lo) visit(lo, exact);
+    row_range(8, lo, hi);
+    for (lo += lane; lo < hi; lo += kLanes) visit(lo, exact);
+    __syncwarp();
+  };
+  if (lane == 0) s_n[grp] = 0;
+  __syncwarp();
+  search(false);
+  int nc = s_n[grp];
+  if (__any_sync(0xffffffffu, nc > kDemMaxCap)) {
+    // more candidates than the list holds: without the pairs that only pass
+    // the screen; what is too much then is beyond any capacity
+    __syncwarp();
+    if (lane == 0) s_n[grp] = 0;
+    __syncwarp();
+    search(true);
+    nc = s_n[grp];
+    if (nc > kDemMaxCap) {
+      if (lane == 0) atomicOr(flags, 1);
+      nc = kDemMaxCap;
+    }
+  }
+  // ---- sorted by partner index (rank = partners below)
+  for (int q = lane; q < nc; q += kLanes) {
+    const int32_t j = s_j[grp][q];
+    int rank = 0;
+    for (int c = 0; c < nc; ++c) rank += s_j[grp][c] < j;
+    s_ord[grp][rank] = (unsigned char)q;
+  }
+  __syncwarp();
+
+  // ---- contacts, eight at a time; lanes 0..5 add the six components up
+  const R rir = body_radius(me_b);
+  const R mir = k.mass1 * rir * rir * rir;
+  R sum = 0;
+  int m = 0;  // contacts kept
+  const int rounds = __reduce_max_sync(0xffffffffu, (unsigned)nc);
+  for (int c0 = 0; c0 < rounds; c0 += kLanes) {
+    const int c = c0 + lane;
+    bool on = c < nc;
+    int32_t j = 0;
+    int64_t q = 0;
+    R nrm[3], dn = 0;
+    Body<R> o;
+    if (on) {
+      const int l = s_ord[grp][c];
+      j = s_j[grp][l];
+      q = s_at[grp][l];
+      o.load(cs, q);
+      on = dem_pair(me_b, o, nrm, &dn);
+    }
+    const unsigned b = (__ballot_sync(0xffffffffu, on) >> base) & 0xffu;
+    const int pos = m + __popc(b & below);
+    m += __popc(b);
+    if (on && pos >= C) {
+      atomicOr(flags, 1);
+      on = false;
+    }
+    R F[3] = {0, 0, 0}, Tq[3] = {0, 0, 0};
+    if (on) {
+      R th[3] = {0, 0, 0};
+      // the pair's place in the last list: mostly the same as now
+      int old = pos;
+      if (old >= len || s_old[grp][old] != j)
+        for (old = 0; old < len && s_old[grp][old] < j;) ++old;
+      if (old < len && s_old[grp][old] == j)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) th[a] = h.t_old[(i * C + old) * 3 + a];
+      R wi[3], wj[3], vrel[3];
+      dem_relative(cs, at, q, vrel, wi, wj);
+      const R rj = body_radius(o);
+      const R mj = k.mass1 * rj * rj * rj;
+      const R me = mir * mj / (mir + mj);
+      const R Re = rir * rj / (rir + rj);
+      const R ws[3] = {rir * wi[0] + rj * wj[0], rir * wi[1] + rj * wj[1],
+                       rir * wi[2] + rj * wj[2]};
+      vrel[0] += ws[1] * nrm[2] - ws[2] * nrm[1];
+      vrel[1] += ws[2] * nrm[0] - ws[0] * nrm[2];
+      vrel[2] += ws[0] * nrm[1] - ws[1] * nrm[0];
+      const R wrel[3] = {wi[0] - wj[0], wi[1] - wj[1], wi[2] - wj[2]};
+      dem_contact<R>(nrm, dn, vrel, wrel, rir, me, Re, k, dt, th, F, Tq);
+      if (live) {
+        h.j_new[i * C + pos] = j;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) h.t_new[(i * C + pos) * 3 + a] = th[a];
       }
     }
-  }
-  __syncwarp(live);
-  const double mi = p.rho * (4.0 / 3.0 * kPi) * ri * ri * ri;
-  const double Ii = 0.4 * mi * ri * ri;
-  const R rir = (R)ri, mir = (R)mi;
-  const R mcoef = (R)(p.rho * (4.0 / 3.0 * kPi));
-  R F[3] = {0, 0, 0}, Tq[3] = {0, 0, 0};
-  const R wi[3] = {(R)w[3 * i], (R)w[3 * i + 1], (R)w[3 * i + 2]};
-  int o = 0;  // cursor in the previous (sorted) list
-  int m = 0;  // contacts kept
-  for (int c = 0; c < nc; ++c) {
-    const int32_t j = cand[c];
-    const double d[3] = {x[3 * j] - xi[0], x[3 * j + 1] - xi[1], x[3 * j + 2] - xi[2]};
-    const double d2 = d_dot(d, d);
-    const double rjd = r[j];
-    const double rs = ri + rjd;
-    if (!(d2 < rs * rs)) continue;
-    R nrm[3], dn;
-    if (std::is_same<R, double>::value) {
-      const double dist = sqrt(d2);
-      if (!(dist < rs && dist > 0.0)) continue;
-      for (int a = 0; a < 3; ++a) nrm[a] = (R)(d[a] / dist);
-      dn = (R)(rs - dist);
-    } else {
-      if (!(d2 > 0.0)) continue;
-      const R dist = t_sqrt<R>((R)d2);
-      const R inv = (R)1 / dist;
-      for (int a = 0; a < 3; ++a) nrm[a] = (R)d[a] * inv;
-      dn = (R)(rs * rs - d2) / ((R)rs + dist);
-    }
-    if (m == C) {
-      atomicOr(flags, 1);
-      continue;
-    }
-    R rj, wj[3];
-    if (std::is_same<R, double>::value) {
-      rj = (R)rjd;
-      for (int a = 0; a < 3; ++a) wj[a] = (R)w[3 * j + a];
-    } else {
-      const float4 q = wf[j];
-      rj = (R)q.w;
-      wj[0] = (R)q.x;
-      wj[1] = (R)q.y;
-      wj[2] = (R)q.z;
-    }
-    const R mj = mcoef * rj * rj * rj;
-    const R me = (R)1 / ((R)1 / mir + (R)1 / mj);
-    const R Re = (R)1 / ((R)1 / rir + (R)1 / rj);
-    const R ws[3] = {rir * wi[0] + rj * wj[0], rir * wi[1] + rj * wj[1], rir * wi[2] + rj * wj[2]};
-    const R wxn[3] = {ws[1] * nrm[2] - ws[2] * nrm[1], ws[2] * nrm[0] - ws[0] * nrm[2],
-                      ws[0] * nrm[1] - ws[1] * nrm[0]};
-    R vrel[3], wrel[3];
+#pragma unroll
     for (int a = 0; a < 3; ++a) {
-      vrel[a] = (R)(v[3 * i + a] - v[3 * j + a]) + wxn[a];
-      wrel[a] = wi[a] - wj[a];
+      s_f[grp][lane][a] = F[a];
+      s_f[grp][lane][3 + a] = Tq[a];
     }
-    R th[3] = {0, 0, 0};
-    while (o < C && hj_old[i * C + o] >= 0 && hj_old[i * C + o] < j) ++o;
-    if (o < C && hj_old[i * C + o] == j)
-      for (int a = 0; a < 3; ++a) th[a] = ht_old[(i * C + o) * 3 + a];
-    dem_contact<R>(nrm, dn, vrel, wrel, rir, me, Re, (R)p.Ye, (R)p.Ge, (R)p.c56, (R)p.mus,
-                   (R)p.mur, (R)dt, th, F, Tq);
-    hj_new[i * C + m] = j;
-    for (int a = 0; a < 3; ++a) ht_new[(i * C + m) * 3 + a] = th[a];
-    ++m;
+    __syncwarp();
+    if (lane < 6)
+#pragma unroll
+      for (int c1 = 0; c1 < kLanes; ++c1) sum += s_f[grp][c1][lane];
+    __syncwarp();
   }
-  for (int c = m; c < C; ++c) hj_new[i * C + c] = -1;
-  __syncwarp(live);
-  // walls x-, x+, y-, y+, z-, z+
-  for (int wl = 0; wl < 6; ++wl) {
-    const int ax = wl / 2;
-    R nrm[3] = {0, 0, 0};
-    double dnd;
-    if (wl % 2 == 0) {
-      nrm[ax] = (R)-1;
-      dnd = ri - (xi[ax] - p.lo[ax]);
-    } else {
-      nrm[ax] = (R)1;
-      dnd = ri - (p.hi[ax] - xi[ax]);
+  if (live && lane == 0 && m < C) h.j_new[i * C + m] = -1;
+
+  // ---- walls x-, x+, y-, y+, z-, z+: a lane each
+  const R dnw = lane < 6 ? wall_overlap(p, me_b, lane) : (R)-1;
+  const bool on = live && dnw > (R)0;
+  const unsigned all = __ballot_sync(0xffffffffu, on);
+  if (all) {
+    const unsigned b = (all >> base) & 0xffu, had = live ? h.wmask[i] : 0u;
+    R F[3] = {0, 0, 0}, Tq[3] = {0, 0, 0};
+    if (on) {
+      const int ax = lane >> 1;
+      const R sg = lane & 1 ? (R)1 : (R)-1;
+      const R nrm[3] = {ax == 0 ? sg : (R)0, ax == 1 ? sg : (R)0, ax == 2 ? sg : (R)0};
+      R vi[3], wi[3];
+      dem_own(cs, at, vi, wi);
+      const R rw[3] = {rir * wi[0], rir * wi[1], rir * wi[2]};
+      const R vrel[3] = {vi[0] + (rw[1] * nrm[2] - rw[2] * nrm[1]),
+                         vi[1] + (rw[2] * nrm[0] - rw[0] * nrm[2]),
+                         vi[2] + (rw[0] * nrm[1] - rw[1] * nrm[0])};
+      R* tw = h.wall + (i * 6 + lane) * 3;
+      R th[3] = {0, 0, 0};
+      if (had >> lane & 1u)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) th[a] = tw[a];
+      dem_contact<R>(nrm, dnw, vrel, wi, rir, mir, rir, kw, dt, th, F, Tq);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) tw[a] = th[a];
     }
-    double* th = wh + (i * 6 + wl) * 3;
-    if (!(dnd > 0.0)) {
-      th[0] = th[1] = th[2] = 0.0;
-      continue;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      s_f[grp][lane][a] = F[a];
+      s_f[grp][lane][3 + a] = Tq[a];
     }
-    const R rw[3] = {rir * wi[0], rir * wi[1], rir * wi[2]};
-    const R wxn[3] = {rw[1] * nrm[2] - rw[2] * nrm[1], rw[2] * nrm[0] - rw[0] * nrm[2],
-                      rw[0] * nrm[1] - rw[1] * nrm[0]};
-    const R vrel[3] = {(R)v[3 * i] + wxn[0], (R)v[3 * i + 1] + wxn[1], (R)v[3 * i + 2] + wxn[2]};
-    R t3[3] = {(R)th[0], (R)th[1], (R)th[2]};
-    dem_contact<R>(nrm, (R)dnd, vrel, wi, rir, mir, rir, (R)p.Yew, (R)p.Gew, (R)p.c56w,
-                   (R)p.musw, (R)p.murw, (R)dt, t3, F, Tq);
-    th[0] = t3[0];
-    th[1] = t3[1];
-    th[2] = t3[2];
+    __syncwarp();
+    if (lane < 6)
+#pragma unroll
+      for (int c1 = 0; c1 < 6; ++c1) sum += s_f[grp][c1][lane];
+    if (live && lane == 0) h.wmask[i] = (unsigned char)b;
+  } else if (live && lane == 0 && h.wmask[i]) {
+    h.wmask[i] = 0;
   }
-  // two FP64 divisions instead of six (each is a chain on the FP64 pipe)
-  const double inv_mi = 1.0 / mi, inv_Ii = 1.0 / Ii;
+  if (live && lane < 6) sums[6 * i + lane] = sum;
+}
+
+// what k_dem_advance does with the accelerations
+struct DemTurn {
+  double step;   // sub-step length
+  int close;     // the closing half kick of this sub-step
+  int open;      // the next sub-step's opening kick and drift, and its cells
+};
+
+// gravity, the fluid force and the integration
+template <typename R>
+__global__ void __launch_bounds__(128)
+k_dem_advance(int64_t n, DemDev p, DemTurn turn, const R* __restrict__ sums,
+              const double2* __restrict__ inv, double* __restrict__ x, double* __restrict__ v,
+              double* __restrict__ w, const double* __restrict__ f_ext,
+              int32_t* __restrict__ cell_of, int32_t* __restrict__ slot,
+              int32_t* __restrict__ count_next, double* __restrict__ acc,
+              double* __restrict__ alpha) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const double2 im = inv[i];
+  int c[3];
+#pragma unroll
   for (int a = 0; a < 3; ++a) {
-    const double fa = (double)F[a] + mi * p.g[a] + (f_ext ? f_ext[3 * i + a] : 0.0);
-    acc[3 * i + a] = fa * inv_mi;
-    alpha[3 * i + a] = (double)Tq[a] * inv_Ii;
+    const int64_t q = 3 * i + a;
+    double f = (double)sums[6 * i + a];
+    if (f_ext) f += f_ext[q];
+    const double ac = fma(f, im.x, p.g[a]), al = (double)sums[6 * i + 3 + a] * im.y;
+    double vt = v[q], wt = w[q];
+    if (turn.close) {
+      half_kick(0.5 * turn.step, ac, vt);
+      half_kick(0.5 * turn.step, al, wt);
+    }
+    if (turn.open) {
+      half_kick(0.5 * turn.step, ac, vt);
+      half_kick(0.5 * turn.step, al, wt);
+      const double xt = fma(turn.step, vt, x[q]);
+      x[q] = xt;
+      c[a] = cell_axis(xt, p.lo[a], p.inv_ce[a], p.nc[a]);
+    } else {
+      acc[q] = ac;
+      alpha[q] = al;
+    }
+    v[q] = vt;
+    w[q] = wt;
+  }
+  if (turn.open) {
+    const int cell = cell_of_axes(p, c[0], c[1], c[2]);
+    cell_of[i] = cell;
+    slot[i] = atomicAdd(count_next + cell, 1);
   }
 }
 
@@ -499,16 +729,21 @@ struct cfdem_dem {
   cfdem_dem_params prm{};
   bool have_prm = false;
   DemDev dd{};
+  Contact<double> pp{}, pw{};  // particle-particle, particle-wall
   int64_t n = -1;        // particle count the state belongs to
   int have_acc = 0;
   int cur = 0;           // which history buffer holds the last lists
   int64_t cap_n = 0, cap_cells = 0, cap_h = 0;
   double *acc = nullptr, *alpha = nullptr, *ht[2] = {nullptr, nullptr}, *wh = nullptr;
+  double* sums = nullptr;    // contact force and torque (FP32 on the mixed path)
+  double2* inv = nullptr;    // inverse mass and moment of inertia
+  unsigned char* wmask = nullptr;
   int32_t *hj[2] = {nullptr, nullptr};
-  int32_t *cell_of = nullptr, *slot = nullptr, *perm = nullptr, *count = nullptr,
-          *start = nullptr, *tsum = nullptr;
-  float4* xs = nullptr;  // cell-ordered FP32 positions and radii
-  float4* wf = nullptr;  // FP32 angular velocities and radii by particle
+  int32_t *cell_of = nullptr, *slot = nullptr, *perm = nullptr, *pcell = nullptr;
+  int32_t* count = nullptr;  // running total of the ranges, then two sets of cell counts
+  int32_t* start = nullptr;
+  float4* xs = nullptr;      // cell-ordered FP32 positions and radii
+  float4* body = nullptr;    // the rest of the cell-ordered state, 80 bytes a particle
   int* flags = nullptr;
   std::string err;
 };
@@ -531,6 +766,11 @@ cfdem_status dcuda(cfdem_dem_t d, cudaError_t e, const char* where) {
   if (e == cudaErrorMemoryAllocation)
     return dfail(d, CFDEM_ENOMEM, "%s: out of device memory", where);
   return dfail(d, CFDEM_ECUDA, "%s: %s", where, cudaGetErrorString(e));
+}
+
+Contact<float> in_float(const Contact<double>& k) {
+  return Contact<float>{(float)k.Ye, (float)k.Ge, (float)k.en, (float)k.et, (float)k.mus,
+                        (float)k.mur, (float)k.mass1};
 }
 
 #define DCK(expr, where)                                  \
@@ -602,7 +842,8 @@ cfdem_status cfdem_dem_destroy(cfdem_dem_t d) {
   if (d->stream) cudaStreamSynchronize(d->stream);
   else cudaDeviceSynchronize();
   void* ps[] = {d->acc, d->alpha, d->ht[0], d->ht[1], d->wh, d->hj[0], d->hj[1], d->cell_of,
-                d->slot, d->perm, d->count, d->start, d->tsum, d->flags, d->xs, d->wf};
+                d->slot, d->perm, d->count, d->start, d->flags, d->xs, d->body, d->wmask,
+                d->sums, d->pcell, d->inv};
   for (void* p : ps)
     if (p) cudaFree(p);
   delete d;
@@ -632,38 +873,38 @@ cfdem_status cfdem_dem_set_params(cfdem_dem_t d, const cfdem_dem_params* p) {
       return dfail(d, CFDEM_EINVAL, "box: hi must exceed lo on every axis");
   DemDev& q = d->dd;
   q.rho = p->rho_p;
-  q.Y = p->youngs;
-  q.nu = p->poisson;
-  q.e = p->restitution;
-  q.mus = p->friction;
-  q.mur = p->rolling_friction;
-  q.Yw = p->wall_youngs;
-  q.nuw = p->wall_poisson;
-  q.ew = p->wall_restitution;
-  q.musw = p->wall_friction;
-  q.murw = p->wall_rolling_friction;
   q.rmax = p->max_radius;
   auto c56 = [](double e) {
     const double le = std::log(e);
     return -2.0 * std::sqrt(5.0 / 6.0) * (le / std::sqrt(le * le + kPi * kPi));
   };
-  q.c56 = c56(p->restitution);
-  q.c56w = c56(p->wall_restitution);
   const double nu = p->poisson, nuw = p->wall_poisson;
-  q.Ye = 1.0 / ((1.0 - nu * nu) / p->youngs + (1.0 - nu * nu) / p->youngs);
-  q.Ge = 1.0 / (2.0 * (2.0 - nu) * (1.0 + nu) / p->youngs + 2.0 * (2.0 - nu) * (1.0 + nu) / p->youngs);
-  q.Yew = 1.0 / ((1.0 - nu * nu) / p->youngs + (1.0 - nuw * nuw) / p->wall_youngs);
-  q.Gew = 1.0 / (2.0 * (2.0 - nu) * (1.0 + nu) / p->youngs +
-                 2.0 * (2.0 - nuw) * (1.0 + nuw) / p->wall_youngs);
+  auto contact = [&](double Y2, double nu2, double e, double mus, double mur) {
+    Contact<double> k{};
+    k.Ye = 1.0 / ((1.0 - nu * nu) / p->youngs + (1.0 - nu2 * nu2) / Y2);
+    k.Ge = 1.0 / (2.0 * (2.0 - nu) * (1.0 + nu) / p->youngs +
+                  2.0 * (2.0 - nu2) * (1.0 + nu2) / Y2);
+    k.en = c56(e) * std::sqrt(2.0 * k.Ye);
+    k.et = c56(e) * std::sqrt(8.0 * k.Ge);
+    k.mus = mus;
+    k.mur = mur;
+    k.mass1 = p->rho_p * (4.0 / 3.0 * kPi);
+    return k;
+  };
+  d->pp = contact(p->youngs, nu, p->restitution, p->friction, p->rolling_friction);
+  d->pw = contact(p->wall_youngs, nuw, p->wall_restitution, p->wall_friction,
+                  p->wall_rolling_friction);
   int64_t tot = 1;
   for (int a = 0; a < 3; ++a) {
     q.g[a] = p->g[a];
     q.lo[a] = p->lo[a];
     q.hi[a] = p->hi[a];
-    double f = std::floor((p->hi[a] - p->lo[a]) / (2.0 * p->max_radius));
+    const double ext = p->hi[a] - p->lo[a];
+    q.ext[a] = df64((float)ext, (float)(ext - (double)(float)ext));
+    double f = std::floor(ext / (2.0 * p->max_radius * (1.0 + 1.0 / 512.0)));
     int nc = f < 1.0 ? 1 : (f > 4096.0 ? 4096 : (int)f);
     q.nc[a] = nc;
-    q.inv_ce[a] = nc / (p->hi[a] - p->lo[a]);
+    q.inv_ce[a] = (float)(nc / ext);
     tot *= nc;
   }
   if (tot > ((int64_t)1 << 28)) return dfail(d, CFDEM_EINVAL, "too many cells");
@@ -700,13 +941,18 @@ cfdem_status cfdem_dem_step(cfdem_dem_t d, int64_t n, double* x, double* v, doub
   const int64_t ncells = (int64_t)d->dd.nc[0] * d->dd.nc[1] * d->dd.nc[2];
   if (n != d->n) {  // a new particle set: fresh state
     if (n > d->cap_n || (int64_t)n * C > d->cap_h) {
-      void* old[] = {d->acc, d->alpha, d->wh, d->cell_of, d->slot, d->perm,
-                     d->hj[0], d->hj[1], d->ht[0], d->ht[1], d->xs, d->wf};
+      void* old[] = {d->acc, d->alpha, d->wh, d->cell_of, d->slot, d->perm, d->wmask,
+                     d->hj[0], d->hj[1], d->ht[0], d->ht[1], d->xs, d->body, d->sums,
+                     d->pcell, d->inv};
       for (void* q : old)
         if (q) cudaFree(q);
       d->acc = d->alpha = d->wh = d->ht[0] = d->ht[1] = nullptr;
       d->cell_of = d->slot = d->perm = d->hj[0] = d->hj[1] = nullptr;
-      d->xs = d->wf = nullptr;
+      d->xs = d->body = nullptr;
+      d->wmask = nullptr;
+      d->sums = nullptr;
+      d->inv = nullptr;
+      d->pcell = nullptr;
       d->cap_n = d->cap_h = 0;
       const int64_t cap = n + n / 4 + 256;
       DCK(cudaMalloc(&d->acc, sizeof(double) * 3 * cap), "dem arena");
@@ -716,7 +962,11 @@ cfdem_status cfdem_dem_step(cfdem_dem_t d, int64_t n, double* x, double* v, doub
       DCK(cudaMalloc(&d->slot, sizeof(int32_t) * cap), "dem arena");
       DCK(cudaMalloc(&d->perm, sizeof(int32_t) * cap), "dem arena");
       DCK(cudaMalloc(&d->xs, sizeof(float4) * cap), "dem arena");
-      DCK(cudaMalloc(&d->wf, sizeof(float4) * cap), "dem arena");
+      DCK(cudaMalloc(&d->body, sizeof(float4) * 5 * cap), "dem arena");
+      DCK(cudaMalloc(&d->wmask, cap), "dem arena");
+      DCK(cudaMalloc(&d->sums, sizeof(double) * 6 * cap), "dem arena");
+      DCK(cudaMalloc(&d->inv, sizeof(double2) * cap), "dem arena");
+      DCK(cudaMalloc(&d->pcell, sizeof(int32_t) * cap), "dem arena");
       DCK(cudaMalloc(&d->hj[0], sizeof(int32_t) * cap * C), "dem arena");
       DCK(cudaMalloc(&d->hj[1], sizeof(int32_t) * cap * C), "dem arena");
       DCK(cudaMalloc(&d->ht[0], sizeof(double) * 3 * cap * C), "dem arena");
@@ -725,7 +975,7 @@ cfdem_status cfdem_dem_step(cfdem_dem_t d, int64_t n, double* x, double* v, doub
       d->cap_h = cap * C;
     }
     DCK(cudaMemsetAsync(d->hj[0], 0xff, sizeof(int32_t) * n * C, s), "dem reset");
-    DCK(cudaMemsetAsync(d->wh, 0, sizeof(double) * 18 * n, s), "dem reset");
+    DCK(cudaMemsetAsync(d->wmask, 0, n, s), "dem reset");
     d->cur = 0;
     d->n = n;
     d->have_acc = 0;
@@ -733,57 +983,75 @@ cfdem_status cfdem_dem_step(cfdem_dem_t d, int64_t n, double* x, double* v, doub
   if (ncells + 1 > d->cap_cells) {
     if (d->count) cudaFree(d->count);
     if (d->start) cudaFree(d->start);
-    if (d->tsum) cudaFree(d->tsum);
-    d->count = d->start = d->tsum = nullptr;
+    d->count = d->start = nullptr;
     d->cap_cells = 0;
-    DCK(cudaMalloc(&d->count, sizeof(int32_t) * ncells), "dem cells");
-    DCK(cudaMalloc(&d->start, sizeof(int32_t) * (ncells + 1)), "dem cells");
-    DCK(cudaMalloc(&d->tsum, sizeof(int32_t) * (ncells / kScanTile + 2)), "dem cells");
+    DCK(cudaMalloc(&d->count, sizeof(int32_t) * (2 * ncells + 1)), "dem cells");
+    DCK(cudaMalloc(&d->start, sizeof(int32_t) * ncells), "dem cells");
     d->cap_cells = ncells + 1;
   }
-  const unsigned nb = (unsigned)((n + 127) / 128), nb3 = (unsigned)((3 * n + 255) / 256);
-  auto forces = [&](double hdt) -> cudaError_t {
-    cudaError_t e = cudaMemsetAsync(d->count, 0, sizeof(int32_t) * ncells, s);
-    if (e != cudaSuccess) return e;
-    k_dem_cell_count<<<nb, 128, 0, s>>>(n, d->dd, x, r, d->cell_of, d->slot, d->count,
-                                        d->flags);
-    const int ntiles = (int)((ncells + kScanTile - 1) / kScanTile);
-    k_dem_scan_tiles<<<ntiles, 256, 0, s>>>((int)ncells, d->count, d->tsum);
-    k_dem_scan_sums<<<1, 256, 0, s>>>(ntiles, d->tsum);
-    k_dem_scan_final<<<ntiles, 256, 0, s>>>((int)ncells, d->count, d->tsum, d->start);
-    k_dem_cell_scatter<<<nb, 128, 0, s>>>(n, d->dd, x, w, r, d->cell_of, d->slot, d->start,
-                                          d->perm, d->xs, d->wf);
+  const unsigned nb = (unsigned)((n + 127) / 128), nbf = (unsigned)((n + kDemPer - 1) / kDemPer);
+  const int rows = std::max(1, kRangeTile / d->dd.nc[0]);
+  const int tile = rows * d->dd.nc[0];
+  const unsigned ntiles = (unsigned)((ncells + tile - 1) / tile);
+  const bool mixed = d->prm.precision == 1;
+  DemCells cs{};
+  cs.xs = d->xs;
+  cs.perm = d->perm;
+  cs.cell = d->pcell;
+  cs.xl = d->body;
+  cs.vh = d->body + d->cap_n;
+  cs.vl = d->body + 2 * d->cap_n;
+  cs.wf = d->body + 3 * d->cap_n;
+  cs.xr = reinterpret_cast<double2*>(d->body);
+  cs.vw = reinterpret_cast<double2*>(d->body + 2 * d->cap_n);
+  int32_t* total = d->count;
+  int32_t* cells[2] = {d->count + 1, d->count + 1 + ncells};
+  int set = 0;
+  // forces at the current positions and the integration that follows; the
+  // cells of the positions are in cells[set]
+  auto forces = [&](double hdt, int close, int open) -> cudaError_t {
+    k_dem_ranges<<<ntiles, 256, 0, s>>>((int)ncells, tile, cells[set], cells[1 - set], total,
+                                        d->start);
+    const DemTurn turn{dt, close, open};
     const int o = d->cur, nw = 1 - d->cur;
-    if (d->prm.precision == 1)  // FP32 tangential history in the same buffers
-      k_dem_forces<float><<<nb, 128, 0, s>>>(
-          n, d->dd, hdt, x, v, w, r, f_ext, d->start, d->perm, d->xs, d->wf, d->hj[o],
-          reinterpret_cast<const float*>(d->ht[o]), d->hj[nw],
-          reinterpret_cast<float*>(d->ht[nw]), d->wh, d->acc, d->alpha, d->flags);
-    else
-      k_dem_forces<double><<<nb, 128, 0, s>>>(n, d->dd, hdt, x, v, w, r, f_ext, d->start,
-                                              d->perm, d->xs, d->wf, d->hj[o], d->ht[o],
-                                              d->hj[nw], d->ht[nw], d->wh, d->acc, d->alpha,
-                                              d->flags);
-    count_launches(6);
+    if (mixed) {  // FP32 tangential history in the same buffers
+      k_dem_cell_scatter<float><<<nb, 128, 0, s>>>(n, d->dd, x, v, w, r, d->cell_of, d->slot,
+                                                   d->start, cs, total);
+      const DemHist<float> h{d->hj[o], reinterpret_cast<const float*>(d->ht[o]), d->hj[nw],
+                             reinterpret_cast<float*>(d->ht[nw]),
+                             reinterpret_cast<float*>(d->wh), d->wmask};
+      float* sums = reinterpret_cast<float*>(d->sums);
+      k_dem_forces<float><<<nbf, kDemBlock, 0, s>>>(n, d->dd, in_float(d->pp), in_float(d->pw),
+                                                    (float)hdt, d->start, cells[set], cs, h,
+                                                    sums, d->flags);
+      k_dem_advance<float><<<nb, 128, 0, s>>>(n, d->dd, turn, sums, d->inv, x, v, w, f_ext,
+                                              d->cell_of, d->slot, cells[1 - set], d->acc,
+                                              d->alpha);
+    } else {
+      k_dem_cell_scatter<double><<<nb, 128, 0, s>>>(n, d->dd, x, v, w, r, d->cell_of, d->slot,
+                                                    d->start, cs, total);
+      const DemHist<double> h{d->hj[o], d->ht[o], d->hj[nw], d->ht[nw], d->wh, d->wmask};
+      k_dem_forces<double><<<nbf, kDemBlock, 0, s>>>(n, d->dd, d->pp, d->pw, hdt, d->start,
+                                                     cells[set], cs, h, d->sums, d->flags);
+      k_dem_advance<double><<<nb, 128, 0, s>>>(n, d->dd, turn, d->sums, d->inv, x, v, w, f_ext,
+                                               d->cell_of, d->slot, cells[1 - set], d->acc,
+                                               d->alpha);
+    }
+    count_launches(4);
     d->cur = nw;
+    set = 1 - set;
     return cudaGetLastError();
   };
-  if (!d->have_acc) {
-    DCK(forces(0.0), "dem forces");
-    d->have_acc = 1;
-  }
-  k_dem_kick_drift<<<nb3, 256, 0, s>>>(n, dt, x, v, w, d->acc, d->alpha);
+  DCK(cudaMemsetAsync(d->count, 0, sizeof(int32_t) * (ncells + 1), s), "dem cells");
+  k_dem_begin<<<nb, 128, 0, s>>>(n, d->dd, dt, d->have_acc, x, v, w, r, d->acc, d->alpha,
+                                 d->cell_of, d->slot, cells[0], d->inv, d->flags);
   count_launches(1);
-  DCK(cudaGetLastError(), "dem drift");
-  for (int it = 0; it < nsub; ++it) {
-    DCK(forces(dt), "dem forces");
-    if (it + 1 < nsub)
-      k_dem_kick_kick_drift<<<nb3, 256, 0, s>>>(n, dt, x, v, w, d->acc, d->alpha);
-    else
-      k_dem_kick<<<nb3, 256, 0, s>>>(n, dt, v, w, d->acc, d->alpha);
-    count_launches(1);
-    DCK(cudaGetLastError(), "dem kick");
-  }
+  DCK(cudaGetLastError(), "dem begin");
+  if (!d->have_acc) DCK(forces(0.0, 0, 1), "dem forces");
+  d->have_acc = 0;  // until the last sub-step has stored them
+  for (int it = 0; it < nsub; ++it)
+    DCK(forces(dt, 1, it + 1 < nsub ? 1 : 0), "dem forces");
+  d->have_acc = 1;
   return CFDEM_OK;
 }
 
