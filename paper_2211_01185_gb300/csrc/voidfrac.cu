@@ -503,7 +503,12 @@ k_qcm(MeshDev m, QcmParams P, BinDev b, const int32_t* __restrict__ bin_start,
 // lanes take every fourth candidate) and adds the lens volume to a
 // Neumaier-compensated sum in registers.  No hit queue and no scan: the
 // instructions per candidate are a distance, a compare and, for the lanes
-// that hit, the lens volume.  Sums run over the candidates in a fixed order
+// that hit, the lens volume.  Q3's batches of 64 come from eight places of
+// the reach: 16 % of its pairs overlap, and lists of 64 mixed candidates are
+// even enough for the warp to run about twice the hits of a mean lane, where
+// testing and evaluating candidate by candidate ran every one (1,000,000
+// spheres, 24 x 24 x 96 Q3: 765 -> 712 us, the same bits).  Sums run over the
+// candidates in a fixed order
 // (the Q1 groups combined by a fixed shuffle tree), so results are
 // reproducible.
 
@@ -511,12 +516,16 @@ template <int K>
 struct QcmPtsSmem {
   static constexpr int Q = (K + 1) * (K + 1) * (K + 1);
   float4 qrel[Q];                  // Gauss point minus element centre
-  float4 cand[kQcmWarps][64];      // culled candidates: position - centre, R + r
-  float4 cons[kQcmWarps][64];      // (R + r)^2, (R - r)^2, full-overlap volume, weight
-  int32_t slot[kQcmWarps][64];     // their sorted slots
-  // per lane, the candidates (of the 32 being tested) that overlap its Gauss
-  // point, in candidate order: [warp][hit][lane] (Q <= 32 only)
-  uint8_t hits[kQcmWarps][Q > 32 ? 1 : 32][32];
+  // candidates tested at a time (Q3: lists long enough to even out over the
+  // lanes) and room for them plus the 31 kept before and the next 32
+  static constexpr int B = Q > 32 ? 64 : 32;
+  static constexpr int CAP = B + 32;
+  float4 cand[kQcmWarps][CAP];     // culled candidates: position - centre, R + r
+  float4 cons[kQcmWarps][CAP];     // (R + r)^2, (R - r)^2, full-overlap volume, weight
+  int32_t slot[kQcmWarps][CAP];    // their sorted slots
+  // per lane and point, the candidates (of the B being tested) that overlap
+  // its Gauss point, in candidate order: [warp][point][hit][lane]
+  uint8_t hits[kQcmWarps][Q > 32 ? 2 : 1][B][32];
 };
 
 template <int K>
@@ -530,6 +539,7 @@ k_qcm_pts(MeshDev m, QcmParams P, BinDev b, const int32_t* __restrict__ bin_star
   constexpr int Q = NQ * NQ * NQ;
   constexpr int G = Q <= 8 ? 4 : 1;     // candidate groups of lanes (Q1)
   constexpr int PPL = Q > 32 ? 2 : 1;   // Gauss points per lane (Q3)
+  constexpr int B = QcmPtsSmem<K>::B;   // candidates tested at a time
   __shared__ QcmPtsSmem<K> sm;
   const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
@@ -603,7 +613,7 @@ k_qcm_pts(MeshDev m, QcmParams P, BinDev b, const int32_t* __restrict__ bin_star
   int my_s0 = 0, my_excl = 0;
   bool more = true;
   for (;;) {
-    while (more && nb < 32) {
+    while (more && nb < B) {
       if (base >= total) {
         rb += 32;
         if (rb >= nrows) {
@@ -630,7 +640,11 @@ k_qcm_pts(MeshDev m, QcmParams P, BinDev b, const int32_t* __restrict__ bin_star
         base = 0;
         continue;
       }
-      const int kk = base + lane;
+      // Q3: runs of four candidates from eight places all over the reach, so
+      // that the hits of a batch spread over the points (32 neighbours hit
+      // some points all and others not at all); otherwise consecutive ones
+      const int kk = PPL > 1 ? (base >> 3) + (lane & 3) + (lane >> 2) * (((total + 31) >> 5) << 2)
+                             : base + lane;
       int lo = 0, hi = 31;
 #pragma unroll
       for (int stp = 0; stp < 5; ++stp) {
@@ -669,13 +683,12 @@ k_qcm_pts(MeshDev m, QcmParams P, BinDev b, const int32_t* __restrict__ bin_star
     }
     if (nb == 0) break;
     __syncwarp();
-    const int cn = nb < 32 ? nb : 32;
-    // Q <= 32 (one point per lane, a few hits per point): each lane first
-    // lists the candidates that overlap its point, then evaluates the lens
-    // volumes of its own list in candidate order (the order of its sum) --
-    // the warp runs as many lens rounds as its busiest lane has hits instead
-    // of one for every candidate any lane hits.  Q3 (two points per lane,
-    // most lanes hit most candidates): test and evaluate in one pass.
+    const int cn = nb < B ? nb : B;
+    // each lane first lists the candidates that overlap its point (Q3: each
+    // of its two points), then evaluates the lens volumes of its own list in
+    // candidate order (the order of its sum): the warp runs as many lens
+    // rounds as its longest list has hits, instead of one for every
+    // candidate that any lane hits
     auto lens = [&](int p, int j, float d2, const float4& A, const float4& B) {
       float v;
       if (d2 <= B.y) {
@@ -692,45 +705,40 @@ k_qcm_pts(MeshDev m, QcmParams P, BinDev b, const int32_t* __restrict__ bin_star
         if (want_ids) ids[p] += perm[sm.slot[wp][j]];
       }
     };
-    if constexpr (PPL == 1) {
-      int nh = 0;
-      for (int j = grp; j < cn; j += G) {
-        const float4 A = sm.cand[wp][j];
-        const float rr2 = sm.cons[wp][j].x;
-        const float dx = A.x - qx[0], dy = A.y - qy[0], dz = A.z - qz[0];
-        const float d2 = dx * dx + dy * dy + dz * dz;
-        if (qok[0] && d2 < rr2) sm.hits[wp][nh++][lane] = (uint8_t)j;
-      }
-      const int mh = (int)__reduce_max_sync(FULL, (unsigned)nh);
-      for (int h = 0; h < mh; ++h) {
-        if (h < nh) {
-          const int j = sm.hits[wp][h][lane];
-          const float4 A = sm.cand[wp][j];
-          const float4 B = sm.cons[wp][j];
-          const float dx = A.x - qx[0], dy = A.y - qy[0], dz = A.z - qz[0];
-          lens(0, j, dx * dx + dy * dy + dz * dz, A, B);
-        }
-      }
-    } else {
-      for (int j = grp; j < cn; j += G) {
-        const float4 A = sm.cand[wp][j];
-        const float4 B = sm.cons[wp][j];
+    int nh[PPL];
 #pragma unroll
-        for (int p = 0; p < PPL; ++p) {
+    for (int p = 0; p < PPL; ++p) nh[p] = 0;
+    for (int j = grp; j < cn; j += G) {
+      const float4 A = sm.cand[wp][j];
+      const float rr2 = sm.cons[wp][j].x;
+#pragma unroll
+      for (int p = 0; p < PPL; ++p) {
+        const float dx = A.x - qx[p], dy = A.y - qy[p], dz = A.z - qz[p];
+        const float d2 = dx * dx + dy * dy + dz * dz;
+        if (qok[p] && d2 < rr2) sm.hits[wp][p][nh[p]++][lane] = (uint8_t)j;
+      }
+    }
+#pragma unroll
+    for (int p = 0; p < PPL; ++p) {
+      const int mh = (int)__reduce_max_sync(FULL, (unsigned)nh[p]);
+      for (int h = 0; h < mh; ++h) {
+        if (h < nh[p]) {
+          const int j = sm.hits[wp][p][h][lane];
+          const float4 A = sm.cand[wp][j];
+          const float4 C = sm.cons[wp][j];
           const float dx = A.x - qx[p], dy = A.y - qy[p], dz = A.z - qz[p];
-          const float d2 = dx * dx + dy * dy + dz * dz;
-          if (qok[p] && d2 < B.x) lens(p, j, d2, A, B);
+          lens(p, j, dx * dx + dy * dy + dz * dz, A, C);
         }
       }
     }
-    // keep the candidates past the 32 tested at the front
+    // keep the candidates past those tested at the front
     const int rest = nb - cn;
     float4 ta = make_float4(0.f, 0.f, 0.f, 0.f), tb = ta;
     int ts = 0;
     if (lane < rest) {
-      ta = sm.cand[wp][32 + lane];
-      tb = sm.cons[wp][32 + lane];
-      ts = sm.slot[wp][32 + lane];
+      ta = sm.cand[wp][B + lane];
+      tb = sm.cons[wp][B + lane];
+      ts = sm.slot[wp][B + lane];
     }
     __syncwarp();
     if (lane < rest) {
