@@ -211,7 +211,11 @@ cfdem_status cfdem_apply(cfdem_t ctx, const double *x_dev, double *y_dev);
  * inside FP64 iterative refinement.  Preconditioner: Jacobi or fast
  * diagonalisation (cg_precond).  eps_q_dev: NULL = the context's last void
  * fraction.  eps_nodal_dev[n_nodes]: start vector on entry, solution on exit.
- * The iteration count and relative residual go to cfdem_get_stats.
+ * The iteration count and relative residual go to cfdem_get_stats.  From the
+ * second solve of a configuration on the CG loop runs as a CUDA graph of the
+ * context's own (stage timers off, fast-diagonalisation preconditioner), so
+ * the call returns without waiting for convergence; a solve that stopped
+ * above cg_rtol is reported by the next cfdem_synchronize either way.
  * While the context's stream is being captured into a CUDA graph the CG
  * loop becomes a conditional (while) node of that graph that iterates on the
  * device until convergence or cg_maxit; the statistics of a replay are read

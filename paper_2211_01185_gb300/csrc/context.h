@@ -76,6 +76,14 @@ struct cfdem_ctx {
   // call
   bool stats_pending = false;
   cudaStream_t loop_stream = nullptr;  // capture stream of device-driven CG loops
+  // the CG loop of eager solves as a graph (see solve()): captured on
+  // cap_stream at the second solve of a configuration (gen, tile shape)
+  cudaStream_t cap_stream = nullptr;
+  cudaGraphExec_t loop_exec = nullptr;
+  unsigned loop_gen = 0;
+  int loop_shape = -1;
+  int loop_solves = 0;       // eager solves of this configuration so far
+  bool loop_failed = false;  // the capture failed: this configuration stays eager
   unsigned gen = 0;                    // bumped by every change of mesh, parameters or timing
   Timer timer;
   long long launches_at_reset = 0;

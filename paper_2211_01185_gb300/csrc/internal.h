@@ -2,6 +2,7 @@
 // coupling library.  Nothing here is part of the public C ABI (cfdem.h).
 #pragma once
 
+#include <cstddef>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -88,7 +89,18 @@ struct CgScalars {
   int loops;       // bodies of a device-driven CG loop run so far
   float alpha_hi, alpha_lo;  // double-float split of alpha (mixed solve)
   int xnz;          // 1 if the start vector has a nonzero entry (else A x0 = 0 is skipped)
+  double* x;        // iterate of the FP64 solve, where its loop is not given it (a graph)
+  // kept over the resets between solves (kCgReset): 1 once a solve whose
+  // statistics the host had not read yet stopped above its tolerance
+  int failed;
 };
+constexpr size_t kCgReset = offsetof(CgScalars, failed);
+
+// The parts of a solve.  All queues it whole.  Start, Loop and Finish are the
+// same launches split so that Loop, which touches the solver's own vectors
+// only, can be kept as a CUDA graph: Start takes b and the start vector,
+// Finish writes the solution.
+enum SolvePart { kSolveAll, kSolveStart, kSolveLoop, kSolveFinish };
 
 // Optional per-stage CUDA-event timers of a context (off by default).  A
 // stage is a group of launches on the context's stream; begin/end record an
@@ -277,7 +289,10 @@ struct CgWork {
   // non-null while the solve is being captured into a CUDA graph: the stream
   // on which the body of the device-driven CG loop is captured
   cudaStream_t loop;
+  SolvePart part;     // what run_cg64 / run_cg_mixed queue (kSolveAll = 0)
 };
+// folds the last solve's outcome into CgScalars::failed
+cudaError_t launch_cg_keep(CgScalars* sc, cudaStream_t s);
 // true when s is a stream under active capture
 bool stream_capturing(cudaStream_t s);
 int cg_blocks(const MeshDev& m);

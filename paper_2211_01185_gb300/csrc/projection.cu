@@ -738,9 +738,10 @@ k_cg_update_fdm(int64_t n, TX_* __restrict__ xv, T* __restrict__ r, const T* __r
   __shared__ double red[32];
   T alpha = (T)sc->alpha;
   T rr = 0;
+  TX_* const xs = xv ? xv : reinterpret_cast<TX_*>(sc->x);
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
-    xv[i] += (TX_)(alpha * p[i]);
+    xs[i] += (TX_)(alpha * p[i]);
     T ri = r[i] - alpha * Ap[i];
     r[i] = ri;
     if (rf) rf[i] = (float)ri;
@@ -807,7 +808,7 @@ template <typename T, typename TB>
 __global__ void __launch_bounds__(256)
 k_cg_start_fdm(int64_t n, const TB* __restrict__ b, const T* __restrict__ Ax,
                T* __restrict__ r, float* __restrict__ rf, double* partials, CgScalars* sc,
-               double rtol, int use_flag) {
+               double rtol, int use_flag, void* x) {
   __shared__ double red[32];
   T rr = 0, bb = 0;
   // with use_flag, A x was skipped for a zero start vector (sc->xnz == 0)
@@ -833,6 +834,7 @@ k_cg_start_fdm(int64_t n, const TB* __restrict__ b, const T* __restrict__ Ax,
     sc->it = 0;
     sc->done = out[0] <= sc->tol2 ? 1 : 0;
     sc->beta = 0.0;
+    sc->x = static_cast<double*>(x);
   }
 }
 
@@ -1203,7 +1205,7 @@ __global__ void k_loop_cond(cudaGraphConditionalHandle h, CgScalars* sc, int max
   cudaGraphSetConditional(h, (!v->done && n < max_bodies) ? 1u : 0u);
 }
 
-// bodies allowed for maxit iterations: two queued ahead, two per body
+// bodies allowed for maxit iterations: at least two queued ahead, two per body
 static int loop_max_bodies(int maxit) { return maxit / 2 + 2; }
 
 static cudaError_t loop_open(cudaStream_t s, cudaStream_t ls, cudaGraphConditionalHandle* h,
@@ -1246,6 +1248,16 @@ static cudaError_t loop_close(cudaStream_t ls, cudaGraphConditionalHandle h, CgS
   cudaGraph_t body = nullptr;
   cudaError_t e = cudaStreamEndCapture(ls, &body);
   return body_status != cudaSuccess ? body_status : e;
+}
+
+__global__ void k_cg_keep(CgScalars* sc) {
+  if (!(sc->rr <= sc->tol2)) sc->failed = 1;
+}
+
+cudaError_t launch_cg_keep(CgScalars* sc, cudaStream_t s) {
+  k_cg_keep<<<1, 1, 0, s>>>(sc);
+  count_launches(1);
+  return cudaGetLastError();
 }
 
 bool stream_capturing(cudaStream_t s) {
@@ -1335,27 +1347,32 @@ static cudaError_t cg_solve_fdm(const MeshDev& m, const T* bands, const double* 
                                 T* r, T* z, T* zn, T* p0, T* p1, T* Ap, float* rf, float* zf,
                                 FdmPlan* fdm, double* partials, CgScalars* sc,
                                 cudaStream_t s, int* iters, double* relres, Timer* tm,
-                                bool x_is_zero, cudaStream_t ls) {
+                                bool x_is_zero, cudaStream_t ls, SolvePart part = kSolveAll) {
+  if (part == kSolveFinish) return cudaSuccess;  // the loop has updated x in place
   cudaError_t e;
   int64_t n = m.n_nodes;
   int vb = vec_blocks(n);
   const int op_stage = sizeof(T) == 8 ? kStageOp64 : kStageOp32;
   const bool conv = sizeof(T) == 8;  // FP32 copies needed for the preconditioner
   float* rin = conv ? rf : reinterpret_cast<float*>(r);
-  if (x_is_zero) {
-    if ((e = cudaMemsetAsync(Ap, 0, sizeof(T) * n, s)) != cudaSuccess) return e;
-  } else {
-    // the operator is skipped on the device when x0 has no nonzero entry
-    k_flag_nonzero<TX_><<<vb, 256, 0, s>>>(n, x, &sc->xnz);
+  if (part != kSolveLoop) {
+    if (x_is_zero) {
+      if ((e = cudaMemsetAsync(Ap, 0, sizeof(T) * n, s)) != cudaSuccess) return e;
+    } else {
+      // the operator is skipped on the device when x0 has no nonzero entry
+      k_flag_nonzero<TX_><<<vb, 256, 0, s>>>(n, x, &sc->xnz);
+      count_launches(1);
+      if (tm) tm->begin(op_stage, s);
+      if ((e = apply_t<T>(m, bands, coef, x_as_T, Ap, s, &sc->xnz)) != cudaSuccess) return e;
+      if (tm) tm->end(op_stage, s);
+    }
+    k_cg_start_fdm<T, TB><<<vb, 256, 0, s>>>(n, b, Ap, r, conv ? rf : nullptr, partials, sc, rtol,
+                                            x_is_zero ? 0 : 1, x);
     count_launches(1);
-    if (tm) tm->begin(op_stage, s);
-    if ((e = apply_t<T>(m, bands, coef, x_as_T, Ap, s, &sc->xnz)) != cudaSuccess) return e;
-    if (tm) tm->end(op_stage, s);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  k_cg_start_fdm<T, TB><<<vb, 256, 0, s>>>(n, b, Ap, r, conv ? rf : nullptr, partials, sc, rtol,
-                                          x_is_zero ? 0 : 1);
-  count_launches(1);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if (part == kSolveStart) return cudaSuccess;
+  if (part == kSolveLoop) x = nullptr;  // the pointer that the start left in the scalars
   // z = P^-1 r
   float* zout = conv ? zf : reinterpret_cast<float*>(z);
   if ((e = fdm_apply(fdm, rin, zout, nullptr, s)) != cudaSuccess) return e;
@@ -1391,8 +1408,10 @@ static cudaError_t cg_solve_fdm(const MeshDev& m, const T* bands, const double* 
     return cudaSuccess;
   };
   if (ls) {  // device-driven loop inside a stream capture
-    if ((e = iter(1, s)) != cudaSuccess) return e;
-    if ((e = iter(0, s)) != cudaSuccess) return e;
+    // as many iterations ahead of the node as the solve usually takes (three
+    // to 1e-13): the body's two would be one too many
+    for (int it = 0; it < (sizeof(T) == 8 ? 3 : 2); ++it)
+      if ((e = iter(it == 0, s)) != cudaSuccess) return e;
     cudaGraphConditionalHandle h;
     if ((e = loop_open(s, ls, &h, sc, maxit)) != cudaSuccess) return e;
     e = iter(0, ls);
@@ -1472,12 +1491,20 @@ static cudaError_t cg_solve_df(const MeshDev& m, const df64* bands, const double
   const dim3 g = apply_grid_s<S>(m);
   const size_t sm = apply_smem<K, S, df64>();
   Timer* tm = w.timer;
-  if ((e = cudaMemsetAsync(w.sc, 0, sizeof(CgScalars), s)) != cudaSuccess) return e;
-  k_split_df<<<vb, 256, 0, s>>>(n, b, x, w.x_df, w.r_df, w.r32, w.partials, w.sc);
-  k_residual_df<K, S><<<g, kApplyThreads, sm, s>>>(m, bands, cf, w.x_df, b, w.r_df, w.r32,
-                                                w.partials, w.sc, rtol);
-  count_launches(2);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if (w.part == kSolveFinish) {
+    k_join_df<<<vb, 256, 0, s>>>(n, w.x_df, x);
+    count_launches(1);
+    return cudaGetLastError();
+  }
+  if (w.part != kSolveLoop) {
+    if ((e = cudaMemsetAsync(w.sc, 0, kCgReset, s)) != cudaSuccess) return e;
+    k_split_df<<<vb, 256, 0, s>>>(n, b, x, w.x_df, w.r_df, w.r32, w.partials, w.sc);
+    k_residual_df<K, S><<<g, kApplyThreads, sm, s>>>(m, bands, cf, w.x_df, b, w.r_df, w.r32,
+                                                     w.partials, w.sc, rtol);
+    count_launches(2);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  if (w.part == kSolveStart) return cudaSuccess;
   float* zc = w.z32;
   float* zo = w.zn32;
   df64* pc = w.p0_df;
@@ -1525,12 +1552,12 @@ static cudaError_t cg_solve_df(const MeshDev& m, const df64* bands, const double
     e = iter(0, w.loop);
     if (e == cudaSuccess) e = iter(0, w.loop);
     if ((e = loop_close(w.loop, h, w.sc, maxit, e)) != cudaSuccess) return e;
-    k_join_df<<<vb, 256, 0, s>>>(n, w.x_df, x);
-    count_launches(1);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     *iters = -1;
     *relres = -1.0;
-    return cudaSuccess;
+    if (w.part == kSolveLoop) return cudaSuccess;
+    k_join_df<<<vb, 256, 0, s>>>(n, w.x_df, x);
+    count_launches(1);
+    return cudaGetLastError();
   }
   CgScalars hs;
   if ((e = cudaMemcpyAsync(&hs, w.sc, sizeof(CgScalars), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
@@ -1563,12 +1590,13 @@ cudaError_t run_cg64(const MeshDev& m, const double* bands, const double* coef,
                      const double* b, double* x, double rtol, int maxit, CgWork& w,
                      cudaStream_t s, int* iters_host, double* relres_host, int* converged) {
   cudaError_t e;
-  if ((e = cudaMemsetAsync(w.sc, 0, sizeof(CgScalars), s)) != cudaSuccess) return e;
+  if (w.part == kSolveAll || w.part == kSolveStart)
+    if ((e = cudaMemsetAsync(w.sc, 0, kCgReset, s)) != cudaSuccess) return e;
   if (w.fdm) {
     e = cg_solve_fdm<double, double, double>(m, bands, coef, b, x, x, rtol, maxit, w.r, w.z,
                                              w.zn, w.p0, w.p1, w.Ap, w.r32, w.z32, w.fdm,
                                              w.partials, w.sc, s, iters_host, relres_host,
-                                             w.timer, false, w.loop);
+                                             w.timer, false, w.loop, w.part);
     if (e != cudaSuccess) return e;
     *converged = *relres_host <= rtol;
     return cudaSuccess;
@@ -1620,7 +1648,7 @@ cudaError_t run_cg_mixed(const MeshDev& m, const double* bands64, const float* b
     if (w.timer) w.timer->begin(kStageOp64, s);
     if ((e = apply_t<double>(m, bands64, coef, x, w.Ap, s)) != cudaSuccess) return e;
     if (w.timer) w.timer->end(kStageOp64, s);
-    if ((e = cudaMemsetAsync(w.sc, 0, sizeof(CgScalars), s)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(w.sc, 0, kCgReset, s)) != cudaSuccess) return e;
     k_residual<double><<<vb, 256, 0, s>>>(n, b, w.Ap, w.r, w.partials, w.sc);
     count_launches(1);
     if ((e = cudaMemcpyAsync(&hs, w.sc, sizeof(CgScalars), cudaMemcpyDeviceToHost, s)) !=
@@ -1635,7 +1663,7 @@ cudaError_t run_cg_mixed(const MeshDev& m, const double* bands64, const float* b
     double scale = rn > 0 ? 1.0 / rn : 1.0;
     k_to_f32<<<vb, 256, 0, s>>>(n, w.r, scale, w.rin32, w.d32);
     count_launches(1);
-    if ((e = cudaMemsetAsync(w.sc, 0, sizeof(CgScalars), s)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(w.sc, 0, kCgReset, s)) != cudaSuccess) return e;
     int it = 0;
     double rr = 0;
     if (w.fdm)
