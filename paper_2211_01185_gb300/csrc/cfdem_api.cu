@@ -271,6 +271,8 @@ void build_tables(int k, int kp, Tables* t) {
   for (int q = 0; q < nq; ++q) lagr(k, t->z, t->lw, t->g[q], l[q], dl[q]);
   for (int a = 0; a <= k; ++a)
     for (int q = 0; q < nq; ++q) {
+      t->Bl[q][a] = l[q][a];
+      t->Blf[q][a] = (float)l[q][a];
       t->Bw[a][q] = l[q][a] * t->w[q];
       t->Bwf[a][q] = (float)t->Bw[a][q];
     }
@@ -1123,6 +1125,25 @@ cfdem_status cfdem_project(cfdem_t c, const double* eps_q, double* eps_nodal) {
 
 }  // extern "C"
 
+namespace {
+// mixed path with many particles per node (large elements, dense beds):
+// split the nodal velocity and void fraction into double-float pairs once
+// per node instead of once per particle that reads them (the same split,
+// so the same bits); the buffer is allocated outside a stream capture
+cfdem_status split_nodal(cfdem_t c, int64_t n, const double* u_nodal, const double* eps_nodal,
+                         ForceParams* fp) {
+  const MeshDev& m = c->mesh;
+  const int64_t nq = (int64_t)(m.k + 1) * (m.k + 1) * (m.k + 1);
+  if (c->prm.precision != 1 || n * nq < 8 * m.n_nodes) return CFDEM_OK;
+  if (!c->nodal_df && !stream_capturing(c->stream))
+    CK(grow(&c->nodal_df, 2 * (size_t)m.n_nodes), "forces");
+  if (!c->nodal_df) return CFDEM_OK;
+  CK(launch_split_nodal(m.n_nodes, u_nodal, eps_nodal, c->nodal_df, c->stream), "forces");
+  fp->nodal_df = c->nodal_df;
+  return CFDEM_OK;
+}
+}  // namespace
+
 cfdem_status forces_with_event(cfdem_t c, int64_t n, const double* x, const double* r,
                                const double* u_p, const double* u_nodal, const double* p_nodal,
                                const double* eps_nodal, double* f, double* f_drag,
@@ -1143,19 +1164,8 @@ cfdem_status forces_with_event(cfdem_t c, int64_t n, const double* x, const doub
     CK(cudaMemsetAsync(c->src_max, 0, 3 * sizeof(unsigned long long), c->stream), "forces");
   c->timer.begin(kStageForces, c->stream);
   ForceParams fp = force_params(c);
-  // mixed path with many particles per node (large elements, dense beds):
-  // split the nodal velocity and void fraction into double-float pairs once
-  // per node instead of once per particle that reads them (the same split,
-  // so the same bits); the buffer is allocated outside a stream capture
-  const int64_t nq = (int64_t)(m.k + 1) * (m.k + 1) * (m.k + 1);
-  if (c->prm.precision == 1 && n * nq >= 8 * m.n_nodes) {
-    if (!c->nodal_df && !stream_capturing(c->stream))
-      CK(grow(&c->nodal_df, 2 * (size_t)m.n_nodes), "forces");
-    if (c->nodal_df) {
-      CK(launch_split_nodal(m.n_nodes, u_nodal, eps_nodal, c->nodal_df, c->stream), "forces");
-      fp.nodal_df = c->nodal_df;
-    }
-  }
+  s = split_nodal(c, n, u_nodal, eps_nodal, &fp);
+  if (s != CFDEM_OK) return s;
   CK(launch_forces(m, c->tab, c->prm.precision, fp, n, x, r, u_p, u_nodal, p_nodal, eps_nodal,
                    f, f_drag, ps, c->st, c->stream),
      "forces");
@@ -1248,7 +1258,10 @@ cfdem_status cfdem_adjoint(cfdem_t c, int64_t n, const double* x, const double* 
   else
     CK(cudaMemsetAsync(c->adj_geps, 0, sizeof(double) * m.n_nodes, c->stream), "adjoint");
   if (dJ_du) CK(cudaMemsetAsync(dJ_du, 0, sizeof(double) * 3 * m.n_nodes, c->stream), "adjoint");
-  CK(launch_adj_forces(m, c->tab, c->prm.precision, force_params(c), n, x, r, u_p, u_nodal,
+  ForceParams fp = force_params(c);
+  s = split_nodal(c, n, u_nodal, eps_nodal, &fp);
+  if (s != CFDEM_OK) return s;
+  CK(launch_adj_forces(m, c->tab, c->prm.precision, fp, n, x, r, u_p, u_nodal,
                        p_nodal, eps_nodal, g_f, g_fdrag, dJ_dx, dJ_du, c->adj_geps, c->st,
                        c->stream),
      "adjoint forces");
@@ -1257,7 +1270,7 @@ cfdem_status cfdem_adjoint(cfdem_t c, int64_t n, const double* x, const double* 
     CK(cudaMemsetAsync(c->adj_lam, 0, sizeof(double) * m.n_nodes, c->stream), "adjoint");
     s = solve(c, c->adj_geps, c->adj_lam, "adjoint solve");
     if (s != CFDEM_OK) return s;
-    CK(launch_adj_qcm(m, c->tab, c->prm.precision, force_params(c), c->R, c->adj_lam, c->adj_gq,
+    CK(launch_adj_qcm(m, c->tab, c->prm.precision, fp, c->R, c->adj_lam, c->adj_gq,
                       n, x, r, dJ_dx, c->stream),
        "adjoint void fraction");
   }

@@ -211,5 +211,39 @@ struct Closure<float> {
   static __device__ __forceinline__ float tiny() { return 1e-37f; }
 };
 
+// element index and local coordinate (as double-float) along axis a on the
+// mixed path: t = (x - x0) / h from the double-float split of x (~2^-46
+// |x| / h); where t lies within 1e-5 of an element face (or outside the
+// mesh) the FP64 rule of elem_axis_fast decides, so the element is the one
+// the definition gives
+__device__ __forceinline__ int elem_axis_mixed(double x, const MeshDev& m, const ForceParams& fp,
+                                               int a, df64* xi) {
+  if (fp.loc32) {
+    const int i = cell_df(x, fp.x0_hi[a], fp.x0_lo[a], fp.inv_h_hi[a], fp.inv_h_lo[a],
+                          fp.nem1f[a], xi);
+    if (i >= 0) return i;
+  }
+  double xd;
+  const int i = elem_axis_slow(x, m.x0[a], m.h[a], fp.inv_h[a], m.ne[a], &xd);
+  *xi = df_from_double_int(xd);
+  return i;
+}
+
+// Lagrange basis of degree D at t in double-float (nodes and barycentric
+// weights split on the host)
+template <int D>
+__device__ __forceinline__ void lagrange_df(const Tables& tb, df64 t, df64* l) {
+  df64 d[D + 1];
+#pragma unroll
+  for (int a = 0; a <= D; ++a) d[a] = t - df64(tb.zf[a], tb.z_lo[a]);
+#pragma unroll
+  for (int a = 0; a <= D; ++a) {
+    df64 v(tb.lwf[a], tb.lw_lo[a]);
+#pragma unroll
+    for (int b = 0; b <= D; ++b)
+      if (b != a) v = v * d[b];
+    l[a] = v;
+  }
+}
 
 }  // namespace cfdem

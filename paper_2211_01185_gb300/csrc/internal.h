@@ -45,6 +45,8 @@ struct Tables {
   double Bw[4][4];          // Bw[a][q] = l_a(g_q) w_q  (k basis, Gauss weight folded in)
   double Mh[4][4];          // reference mass     int_0^1 l_a l_b
   double Kh[4][4];          // reference stiffness int_0^1 l_a' l_b'
+  double Bl[4][4];          // Bl[q][a] = l_a(g_q)
+  float Blf[4][4];
   float zf[4], zpf[4];      // FP32 copies of z, zp, lw, lwp (mixed path)
   float lwf[4], lwpf[4];
   float z_lo[4], lw_lo[4];  // z - zf and lw - lwf: z and lw as double-float

@@ -301,41 +301,6 @@ __device__ __forceinline__ float f32_of(double v) {
 // rounding of itself, not of a or b
 __device__ __forceinline__ float df_diff(df64 a, df64 b) { return (a.hi - b.hi) + (a.lo - b.lo); }
 
-// element index and local coordinate (as double-float) along axis a on the
-// mixed path: t = (x - x0) / h from the double-float split of x (~2^-46
-// |x| / h); where t lies within 1e-5 of an element face (or outside the
-// mesh) the FP64 rule of elem_axis_fast decides, so the element is the one
-// the definition gives
-__device__ __forceinline__ int elem_axis_mixed(double x, const MeshDev& m, const ForceParams& fp,
-                                               int a, df64* xi) {
-  if (fp.loc32) {
-    const int i = cell_df(x, fp.x0_hi[a], fp.x0_lo[a], fp.inv_h_hi[a], fp.inv_h_lo[a],
-                          fp.nem1f[a], xi);
-    if (i >= 0) return i;
-  }
-  double xd;
-  const int i = elem_axis_slow(x, m.x0[a], m.h[a], fp.inv_h[a], m.ne[a], &xd);
-  *xi = df_from_double_int(xd);
-  return i;
-}
-
-// Lagrange basis of degree D at t in double-float (nodes and barycentric
-// weights split on the host)
-template <int D>
-__device__ __forceinline__ void lagrange_df(const Tables& tb, df64 t, df64* l) {
-  df64 d[D + 1];
-#pragma unroll
-  for (int a = 0; a <= D; ++a) d[a] = t - df64(tb.zf[a], tb.z_lo[a]);
-#pragma unroll
-  for (int a = 0; a <= D; ++a) {
-    df64 v(tb.lwf[a], tb.lw_lo[a]);
-#pragma unroll
-    for (int b = 0; b <= D; ++b)
-      if (b != a) v = v * d[b];
-    l[a] = v;
-  }
-}
-
 // FP64 value written from a T
 template <typename T>
 __device__ __forceinline__ double out_double(T v);
@@ -370,19 +335,30 @@ __device__ __forceinline__ void shear_force(const Tables& tb, const ForceParams&
   const T ih2 = MIX ? (T)fp.inv_h32[2] : (T)fp.inv_h[2];
   const T sxx = ih0 * ih0, syy = ih1 * ih1, szz = ih2 * ih2;
   const T sxy = ih0 * ih1, sxz = ih0 * ih2, syz = ih1 * ih2;
+  const double u00 = __ldg(u_nodal + 3 * base), u01 = __ldg(u_nodal + 3 * base + 1),
+               u02 = __ldg(u_nodal + 3 * base + 2);
+  const df64 r0 = df_from_double_int(u00), r1 = df_from_double_int(u01),
+             r2 = df_from_double_int(u02);
+  // the six second derivatives of the three components, sum factorised: the x
+  // sums of a row with l, l', l'', then the y and z sums of the combinations
+  // in use (936 multiply-adds for Q3 instead of 64 nodes x 30)
   T H[3][6];  // per component: xx, yy, zz, xy, xz, yz
 #pragma unroll
   for (int c = 0; c < 3; ++c)
 #pragma unroll
     for (int q = 0; q < 6; ++q) H[c][q] = (T)0;
-  const double u00 = __ldg(u_nodal + 3 * base), u01 = __ldg(u_nodal + 3 * base + 1),
-               u02 = __ldg(u_nodal + 3 * base + 2);
-  const df64 r0 = df_from_double_int(u00), r1 = df_from_double_int(u01),
-             r2 = df_from_double_int(u02);
 #pragma unroll
-  for (int c = 0; c <= K; ++c)
+  for (int c = 0; c <= K; ++c) {
+    T Y[3][6];  // xx, yy, ll, xy, x, y sums of the layer
 #pragma unroll
-    for (int b = 0; b <= K; ++b)
+    for (int d = 0; d < 3; ++d)
+#pragma unroll
+      for (int q = 0; q < 6; ++q) Y[d][q] = (T)0;
+#pragma unroll
+    for (int b = 0; b <= K; ++b) {
+      T X[3][3];  // sums with l, l', l'' along x
+#pragma unroll
+      for (int d = 0; d < 3; ++d) X[d][0] = X[d][1] = X[d][2] = (T)0;
 #pragma unroll
       for (int a = 0; a <= K; ++a) {
         const int64_t nd = base + a + nx * b + nxy * c;
@@ -396,14 +372,42 @@ __device__ __forceinline__ void shear_force(const Tables& tb, const ForceParams&
           du[1] = (T)(__ldg(u_nodal + 3 * nd + 1) - u01);
           du[2] = (T)(__ldg(u_nodal + 3 * nd + 2) - u02);
         }
-        const T w[6] = {d2[0][a] * l[1][b] * l[2][c] * sxx, l[0][a] * d2[1][b] * l[2][c] * syy,
-                        l[0][a] * l[1][b] * d2[2][c] * szz, d1[0][a] * d1[1][b] * l[2][c] * sxy,
-                        d1[0][a] * l[1][b] * d1[2][c] * sxz, l[0][a] * d1[1][b] * d1[2][c] * syz};
 #pragma unroll
-        for (int cc = 0; cc < 3; ++cc)
-#pragma unroll
-          for (int q = 0; q < 6; ++q) H[cc][q] += w[q] * du[cc];
+        for (int d = 0; d < 3; ++d) {
+          X[d][0] += l[0][a] * du[d];
+          X[d][1] += d1[0][a] * du[d];
+          X[d][2] += d2[0][a] * du[d];
+        }
       }
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        Y[d][0] += l[1][b] * X[d][2];
+        Y[d][1] += d2[1][b] * X[d][0];
+        Y[d][2] += l[1][b] * X[d][0];
+        Y[d][3] += d1[1][b] * X[d][1];
+        Y[d][4] += l[1][b] * X[d][1];
+        Y[d][5] += d1[1][b] * X[d][0];
+      }
+    }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      H[d][0] += l[2][c] * Y[d][0];
+      H[d][1] += l[2][c] * Y[d][1];
+      H[d][2] += d2[2][c] * Y[d][2];
+      H[d][3] += l[2][c] * Y[d][3];
+      H[d][4] += d1[2][c] * Y[d][4];
+      H[d][5] += d1[2][c] * Y[d][5];
+    }
+  }
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    H[d][0] *= sxx;
+    H[d][1] *= syy;
+    H[d][2] *= szz;
+    H[d][3] *= sxy;
+    H[d][4] *= sxz;
+    H[d][5] *= syz;
+  }
   const T mu = MIX ? (T)fp.mu32 : (T)fp.mu;
   const T mu3 = mu / (T)3;
   const T gd[3] = {H[0][0] + H[1][3] + H[2][4], H[0][3] + H[1][1] + H[2][5],
@@ -617,9 +621,9 @@ k_forces(MeshDev m, Tables tb, ForceParams fp, int64_t n, const double* __restri
     gp1 *= fp.inv_h32[1];
     gp2 *= fp.inv_h32[2];
   } else {
-    gp0 = gp0 / m.h[0];
-    gp1 = gp1 / m.h[1];
-    gp2 = gp2 / m.h[2];
+    gp0 *= fp.inv_h[0];
+    gp1 *= fp.inv_h[1];
+    gp2 *= fp.inv_h[2];
   }
 
   // closures
@@ -722,7 +726,9 @@ static void launch_forces_t(const MeshDev& m, const Tables& t, const ForceParams
                             const double* u_nodal, const double* p_nodal,
                             const double* eps_nodal, double* f, double* f_drag, PartSrc ps,
                             DevStatus* st, cudaStream_t s) {
-  int bs = 128;
+  // FP64: blocks of two warps, as the kernel is long and its time on the
+  // narrow pipe goes by the SM with the most warps
+  const int bs = std::is_same<T, float>::value ? 128 : 64;
   const unsigned nb = (unsigned)((n + bs - 1) / bs);
   // the pre-split nodal values (mixed path, no shear force) are a separate
   // instantiation, so that the per-particle splits keep their registers
@@ -941,110 +947,138 @@ cudaError_t launch_fluid_source(const MeshDev& m, const double* S_elem, double* 
 
 // Fluid source with the fluid-side drag (Sec. 2.3.2: the drag written with
 // the fluid velocity at the quadrature point and the cell-mean particle
-// velocity), one thread per element:
+// velocity):
 //   F_q = -beta_e (u_f(x_q) - u_p,avg) - S_e / V_e,  beta_e = B_e / V_e,
 // u_f at the Gauss points by sum-factorised interpolation of the nodal
 // velocity relative to u_p,avg (so that FP32 does not carry the mean),
 // S_e the model-B pressure (and shear) part.  F_e is the Gauss average.
+//
+// 3 (k + 1) threads per element, one per component and layer: a thread
+// contracts its layer of nodes along x and y in registers and leaves it in
+// shared memory, then does the z sums of one layer of Gauss points.  (One
+// thread per element left a Q3 mesh of 4,433 elements 35 blocks, each thread
+// a chain of 3,000 FP64 operations: 126 -> 30 us.)
+constexpr int kSemiThreads = 128;
+template <int K>
+constexpr int kSemiElems = kSemiThreads / (3 * (K + 1));  // per block
+
 template <int K, typename T>
-__global__ void __launch_bounds__(128)
-k_fluid_source_semi(MeshDev m, Tables tb, const double* __restrict__ S, SemiAcc acc,
-                    const double* __restrict__ u_nodal, double* __restrict__ F_e,
+__global__ void __launch_bounds__(kSemiThreads)
+k_fluid_source_semi(MeshDev m, Tables tb, double inv_ve, const double* __restrict__ S,
+                    SemiAcc acc, const double* __restrict__ u_nodal, double* __restrict__ F_e,
                     double* __restrict__ F_q) {
-  constexpr int NQ = K + 1, Q = NQ * NQ * NQ;
-  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (e >= m.E) return;
-  const double inv_ve = 1.0 / m.Ve;
-  const double cnt = acc.N[e];
-  const double beta = acc.B[e] * inv_ve;
-  double upa[3] = {0.0, 0.0, 0.0};
-  if (cnt > 0.0)
-    for (int d = 0; d < 3; ++d) upa[d] = acc.U[3 * e + d] / cnt;
-  const int e32 = (int)e, exy = m.ne[0] * m.ne[1];  // E < 2^31
-  const int ez = e32 / exy;
-  const int ey = (e32 - ez * exy) / m.ne[0];
-  const int ex = e32 - ez * exy - ey * m.ne[0];
-  const int64_t nx = m.nn[0], nxy = (int64_t)m.nn[0] * m.nn[1];
-  const int64_t base = (int64_t)ex * K + nx * ((int64_t)ey * K) + nxy * ((int64_t)ez * K);
+  constexpr int NQ = K + 1, Q = NQ * NQ * NQ, EB = kSemiElems<K>;
+  __shared__ T s_t[EB][3][NQ][NQ * NQ + 1];   // [c][qy][qx], one word of padding
+  __shared__ double s_mean[EB][3][NQ];
+  const int per = 3 * NQ;
+  const int le = threadIdx.x / per, rest = threadIdx.x - le * per;
+  const int d = rest / NQ, c = rest - d * NQ;
+  const int64_t e = blockIdx.x * (int64_t)EB + le;
+  const bool live = le < EB && e < m.E;
+  double beta = 0.0, upa = 0.0;
   T L[NQ][NQ];  // L[q][a] = l_a(g_q)
 #pragma unroll
-  for (int q = 0; q < NQ; ++q) {
-    T l[NQ];
-    lagrange<K, T>(tb.z, tb.lw, (T)tb.g[q], l, (T*)nullptr);
+  for (int q = 0; q < NQ; ++q)
 #pragma unroll
-    for (int a = 0; a < NQ; ++a) L[q][a] = l[a];
-  }
-  const T bt = (T)beta;
-  double mean[3] = {0.0, 0.0, 0.0};
-#pragma unroll 1
-  for (int d = 0; d < 3; ++d) {
-    T v[NQ][NQ][NQ];  // [c][b][a]: u_j - u_p,avg
+    for (int a = 0; a < NQ; ++a) {
+      if constexpr (std::is_same<T, float>::value) L[q][a] = tb.Blf[q][a];
+      else L[q][a] = tb.Bl[q][a];
+    }
+  if (live) {
+    const double cnt = acc.N[e];
+    beta = acc.B[e] * inv_ve;
+    if (cnt > 0.0) upa = acc.U[3 * e + d] / cnt;
+    const int e32 = (int)e, exy = m.ne[0] * m.ne[1];  // E < 2^31
+    const int ez = e32 / exy;
+    const int ey = (e32 - ez * exy) / m.ne[0];
+    const int ex = e32 - ez * exy - ey * m.ne[0];
+    const int64_t nx = m.nn[0], nxy = (int64_t)m.nn[0] * m.nn[1];
+    const int64_t base =
+        (int64_t)ex * K + nx * ((int64_t)ey * K) + nxy * ((int64_t)ez * K + c);
+    T t2[NQ][NQ];  // [qy][qx]
 #pragma unroll
-    for (int c = 0; c < NQ; ++c)
+    for (int qy = 0; qy < NQ; ++qy)
 #pragma unroll
-      for (int b = 0; b < NQ; ++b)
+      for (int qx = 0; qx < NQ; ++qx) t2[qy][qx] = (T)0;
 #pragma unroll
-        for (int a = 0; a < NQ; ++a)
-          v[c][b][a] = (T)(__ldg(u_nodal + 3 * (base + a + nx * b + nxy * c) + d) - upa[d]);
-    T t1[NQ][NQ][NQ];  // [c][b][qx]
+    for (int b = 0; b < NQ; ++b) {
+      T v[NQ], t1[NQ];  // u_j - u_p,avg along x, and its x sums
 #pragma unroll
-    for (int c = 0; c < NQ; ++c)
+      for (int a = 0; a < NQ; ++a) v[a] = (T)(__ldg(u_nodal + 3 * (base + a + nx * b) + d) - upa);
 #pragma unroll
-      for (int b = 0; b < NQ; ++b)
+      for (int qx = 0; qx < NQ; ++qx) {
+        t1[qx] = (T)0;
 #pragma unroll
-        for (int qx = 0; qx < NQ; ++qx) {
-          T s = 0;
-#pragma unroll
-          for (int a = 0; a < NQ; ++a) s += L[qx][a] * v[c][b][a];
-          t1[c][b][qx] = s;
-        }
-    T t2[NQ][NQ][NQ];  // [c][qy][qx]
-#pragma unroll
-    for (int c = 0; c < NQ; ++c)
+        for (int a = 0; a < NQ; ++a) t1[qx] += L[qx][a] * v[a];
+      }
 #pragma unroll
       for (int qy = 0; qy < NQ; ++qy)
 #pragma unroll
-        for (int qx = 0; qx < NQ; ++qx) {
-          T s = 0;
+        for (int qx = 0; qx < NQ; ++qx) t2[qy][qx] += L[qy][b] * t1[qx];
+    }
 #pragma unroll
-          for (int b = 0; b < NQ; ++b) s += L[qy][b] * t1[c][b][qx];
-          t2[c][qy][qx] = s;
-        }
+    for (int qy = 0; qy < NQ; ++qy)
+#pragma unroll
+      for (int qx = 0; qx < NQ; ++qx) s_t[le][d][c][qx + NQ * qy] = t2[qy][qx];
+  }
+  __syncthreads();
+  if (live) {
+    const int qz = c;
+    T Lz[NQ];
+#pragma unroll
+    for (int k = 0; k < NQ; ++k) {
+      Lz[k] = L[0][k];
+#pragma unroll
+      for (int q = 1; q < NQ; ++q)
+        if (qz == q) Lz[k] = L[q][k];
+    }
+    double wz = tb.w[0];
+#pragma unroll
+    for (int q = 1; q < NQ; ++q)
+      if (qz == q) wz = tb.w[q];
+    const T bt = (T)beta;
     const double sv = -S[3 * e + d] * inv_ve;
+    double mean = 0.0;
 #pragma unroll
-    for (int qz = 0; qz < NQ; ++qz)
+    for (int qy = 0; qy < NQ; ++qy) {
+      double row = 0.0;
 #pragma unroll
-      for (int qy = 0; qy < NQ; ++qy)
+      for (int qx = 0; qx < NQ; ++qx) {
+        T sum = 0;
 #pragma unroll
-        for (int qx = 0; qx < NQ; ++qx) {
-          T s = 0;
-#pragma unroll
-          for (int c = 0; c < NQ; ++c) s += L[qz][c] * t2[c][qy][qx];
-          const double F = (double)(-bt * s) + sv;
-          const int q = qx + NQ * (qy + NQ * qz);
-          if (F_q) F_q[(e * Q + q) * 3 + d] = F;
-          mean[d] += tb.w[qx] * tb.w[qy] * tb.w[qz] * F;
-        }
+        for (int k = 0; k < NQ; ++k) sum += Lz[k] * s_t[le][d][k][qx + NQ * qy];
+        const double F = (double)(-bt * sum) + sv;
+        if (F_q) F_q[(e * Q + qx + NQ * (qy + NQ * qz)) * 3 + d] = F;
+        row += tb.w[qx] * F;
+      }
+      mean += tb.w[qy] * row;
+    }
+    s_mean[le][d][qz] = wz * mean;
   }
-  if (F_e)
-    for (int d = 0; d < 3; ++d) F_e[3 * e + d] = mean[d];
+  __syncthreads();
+  if (live && c == 0 && F_e) {
+    double mean = 0.0;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) mean += s_mean[le][d][q];
+    F_e[3 * e + d] = mean;
+  }
 }
 
 cudaError_t launch_fluid_source_semi(const MeshDev& m, const Tables& t, int precision,
                                      const double* S_elem, SemiAcc acc, const double* u_nodal,
                                      double* F_elem, double* F_q, cudaStream_t s) {
   if (!F_elem && !F_q) return cudaSuccess;
-  const unsigned nb = (unsigned)((m.E + 127) / 128);
-#define CFDEM_SEMI(KK)                                                                      \
-  if (m.k == KK) {                                                                          \
-    if (precision == 0)                                                                     \
-      k_fluid_source_semi<KK, double><<<nb, 128, 0, s>>>(m, t, S_elem, acc, u_nodal, F_elem, \
-                                                         F_q);                              \
-    else                                                                                    \
-      k_fluid_source_semi<KK, float><<<nb, 128, 0, s>>>(m, t, S_elem, acc, u_nodal, F_elem,  \
-                                                        F_q);                               \
-    count_launches(1);                                                                      \
-    return cudaGetLastError();                                                              \
+#define CFDEM_SEMI(KK)                                                                       \
+  if (m.k == KK) {                                                                           \
+    const unsigned nb = (unsigned)((m.E + kSemiElems<KK> - 1) / kSemiElems<KK>);         \
+    if (precision == 0)                                                                      \
+      k_fluid_source_semi<KK, double><<<nb, kSemiThreads, 0, s>>>(m, t, 1.0 / m.Ve, S_elem, acc, \
+                                                                  u_nodal, F_elem, F_q);     \
+    else                                                                                     \
+      k_fluid_source_semi<KK, float><<<nb, kSemiThreads, 0, s>>>(m, t, 1.0 / m.Ve, S_elem, acc,  \
+                                                                 u_nodal, F_elem, F_q);      \
+    count_launches(1);                                                                       \
+    return cudaGetLastError();                                                               \
   }
   CFDEM_SEMI(1)
   CFDEM_SEMI(2)
