@@ -481,7 +481,10 @@ def run_bed(env, name, steps, warmup, alu, headline=False, e2e=True, cpu=True,
                            "kernel_launches_per_step": st.kernel_launches / ke,
                            "cg_iterations": st.cg_iterations}
         per[p]["autotune"] = {"bin_edge_m": list(st.bin_edge), "bins": list(st.nb),
-                              "tile_shape": ["16x8x8", "22x13x4", "25x15x4"][st.tile_shape],
+                              "tile_shape": {1: ["16x8x8", "22x13x4", "25x15x4"],
+                                             2: ["16x8x8", "22x14x4", "25x10x6"],
+                                             3: ["16x9x6", "19x15x6", "25x15x3"]}[
+                                                 w["k"]][st.tile_shape],
                               "tuned": {"bins": bool(st.tuned & 1), "tile": bool(st.tuned & 2)},
                               "tune_ms": st.tune_ms,
                               "fdm_tile": "%dx%d" % divmod(st.fdm_tile, 10)}

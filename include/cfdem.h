@@ -131,7 +131,8 @@ typedef struct {
     int32_t timer_overflow;       /* 1 if more than 1024 pairs per stage were asked */
     int64_t kernel_launches;      /* kernels launched by the library since set_timing */
     int32_t precond;              /* preconditioner in use: 0 Jacobi, 1 FDM */
-    int32_t tile_shape;           /* operator tile in use: 0 16x8x8, 1 22x13x4, 2 25x15x4 nodes */
+    int32_t tile_shape;           /* operator tile in use, nodes: 0 16x8x8 (Q3 16x9x6), 1 22x13x4
+                                     (Q2 22x14x4, Q3 19x15x6), 2 25x15x4 (Q2 25x10x6, Q3 25x15x3) */
     int32_t tuned;                /* bit 0: bins chosen by timing, bit 1: tile shape chosen by
                                      timing (autotune) */
     double tune_ms;               /* host time spent timing candidates in this context */

@@ -258,27 +258,64 @@ cudaError_t upload_bands(const MeshDev& m, const Tables& t, double /*L2*/, doubl
 
 // Node tiles of the operator: X x Y x Z owned nodes plus a halo of k.  The
 // shape is picked per mesh (pick_shape) to waste the fewest nodes on partial
-// tiles; e.g. 22 x 13 tiles cover a 65 x 65 node plane with 1.5 % waste
-// where 16 x 8 tiles waste 27 %.
+// tiles; e.g. 22 x 14 tiles cover a 65 x 65 node plane with 9 % waste
+// where 16 x 8 tiles waste 27 %.  Y and Z are multiples of k: the rows of the
+// bands then have the same zeros at the same place of every tile (see Taps).
 template <int X_, int Y_, int Z_>
 struct Shape {
   static constexpr int X = X_, Y = Y_, Z = Z_;
 };
-using Shape0 = Shape<16, 8, 8>;
-using Shape1 = Shape<22, 13, 4>;
-using Shape2 = Shape<25, 15, 4>;
+template <int K>
+struct Shapes;
+template <>
+struct Shapes<1> {
+  using A = Shape<16, 8, 8>;
+  using B = Shape<22, 13, 4>;
+  using C = Shape<25, 15, 4>;
+};
+template <>
+struct Shapes<2> {
+  using A = Shape<16, 8, 8>;
+  using B = Shape<22, 14, 4>;
+  using C = Shape<25, 10, 6>;
+};
+template <>
+struct Shapes<3> {
+  using A = Shape<16, 9, 6>;
+  using B = Shape<19, 15, 6>;
+  using C = Shape<25, 15, 3>;
+};
 constexpr int kShapes = 3;
 constexpr int kApplyThreads = 256;
+
+// The band row of node i couples it to the nodes of its element(s): 2k + 1
+// of them for an element corner (i mod k = 0), k + 1 inside an element, where
+// the other entries of the row are zero.  Taps of the row of residue r:
+// columns [lo(r), hi(r)) of the 2k + 1 -- 4 a row on average for Q2, 5 for Q3.
+template <int K>
+struct Taps {
+  static __host__ __device__ constexpr int lo(int r) { return r == 0 ? 0 : K - r; }
+  static __host__ __device__ constexpr int hi(int r) { return r == 0 ? 2 * K + 1 : 2 * K - r + 1; }
+};
 
 template <int K, class S>
 struct Tile {
   static constexpr int TX = S::X, TY = S::Y, TZ = S::Z;
+  static_assert(TY % K == 0 && TZ % K == 0, "tile rows keep their residue");
   static constexpr int H = K, W = 2 * K + 1;
-  static constexpr int XW = TX + 2 * H, YW = TY + 2 * H, ZW = TZ + 2 * H;
+  // The columns of a tile are kept sorted by their residue mod k (column c of
+  // the haloed row at (c mod k) PW + c / k), so that the x pass, which takes
+  // the residues one after the other, reads neighbouring words.
+  static constexpr int XH = TX + 2 * H;             // haloed columns
+  static constexpr int PW = (XH + K - 1) / K;       // columns per residue
+  static constexpr int TXC = (TX + K - 1) / K;      // owned columns per residue, at most
+  static constexpr int XW = K * PW, YW = TY + 2 * H, ZW = TZ + 2 * H;
+  static __host__ __device__ constexpr int col(int c) { return (c % K) * PW + c / K; }
+  static __host__ __device__ constexpr int own(int c) { return (c % K) * TXC + c / K; }
   static constexpr int NX = ZW * YW * XW;     // input with halo
   static constexpr int NT = TZ * YW * XW;     // after the z pass (each of t1, t2)
   static constexpr int NU = TZ * TY * XW;     // after the y pass (each of U, V)
-  static constexpr int NO = TZ * TY * TX;     // owned nodes (their input, for the epilogue)
+  static constexpr int NO = TZ * TY * K * TXC;  // owned nodes (their input, for the epilogue)
   // Two layouts: the z pass writes t1, t2 over the input (each thread
   // overwrites only the column it has read), with U, V apart; or t1, t2
   // apart and U, V over the input once the z pass is done.  The smaller one
@@ -291,24 +328,23 @@ struct Tile {
   static constexpr int SZ = T_IN_X ? SZ_TX : SZ_UX;
   // band coefficients of the tile's rows: z (M, K), y (three folded
   // combinations), x (M, K)
-  static constexpr int NBZ = 2 * TZ * W, NBY = 3 * TY * W, NBX = 2 * TX * W;
+  static constexpr int NBZ = 2 * TZ * W, NBY = 3 * TY * W, NBX = 2 * K * TXC * W;
   // with XE: the owned nodes' input kept for the epilogue
   static constexpr int nsm(bool xe) { return SZ + (xe ? NO : 0) + NBZ + NBY + NBX; }
   // y pass: one thread per (chunk of CY rows, z, x) column piece, the number
   // of chunks chosen for the fewest row outputs per thread over whole rounds
   // of the block's threads
   static constexpr int YCOLS = TZ * XW;
-  static constexpr int ycost(int nch) {
-    return ((YCOLS * nch + 255) / 256) * ((TY + nch - 1) / nch);
-  }
+  static constexpr int yrows(int nch) { return ((TY + nch - 1) / nch + K - 1) / K * K; }
+  static constexpr int ycost(int nch) { return ((YCOLS * nch + 255) / 256) * yrows(nch); }
   static constexpr int ypick() {
     int best = 1;
     for (int c = 2; c <= TY; ++c)
       if (ycost(c) < ycost(best)) best = c;
     return best;
   }
-  static constexpr int YNCH = ypick();
-  static constexpr int CY = (TY + YNCH - 1) / YNCH;
+  static constexpr int CY = yrows(ypick());            // a multiple of k
+  static constexpr int YNCH = (TY + CY - 1) / CY;
 };
 
 template <typename T>
@@ -322,7 +358,7 @@ struct Coefs {
 template <typename T>
 struct Acc {
   T v;
-  __device__ __forceinline__ void zero() { v = (T)0; }
+  __device__ __forceinline__ void first(T b, T x) { v = b * x; }
   __device__ __forceinline__ void add(T b, T x) { v += b * x; }
   __device__ __forceinline__ T get() const { return v; }
 };
@@ -333,7 +369,13 @@ struct Acc {
 // residuals accurate to ~1e-14 on the FP32 pipes, which on this part have 61
 // times the FP64 throughput.
 template <>
-struct Acc<df64> : DfDotAcc {};
+struct Acc<df64> : DfDotAcc {
+  // the first term needs no two-sum: 4 instructions instead of 12
+  __device__ __forceinline__ void first(df64 b, df64 x) {
+    s = b.hi * x.hi;
+    c = fmaf(b.lo, x.hi, fmaf(b.hi, x.lo, fmaf(b.hi, x.hi, -s)));
+  }
+};
 
 // --- load and epilogue policies of the tile operator -----------------------
 // Plain: x_eff = x[g]
@@ -434,6 +476,12 @@ struct EpiResidualDf {
 // with T1 = Mz x, T2 = Kz x.  The z pass runs one thread per haloed (x, y)
 // column over all TZ outputs, the y pass one thread per run of CY outputs
 // along y (inputs held in registers), the x pass one thread per owned node.
+// The passes leave out the zero entries of the band rows, a fifth (Q2) to
+// 29 % (Q3) of the multiply-adds: along z and y the residue of a row is known
+// when the code is compiled, along x the block takes the residues in turn;
+// and a double-float sum starts with a product instead of a two-sum with zero.
+// Double-float, warm: Q2 65 x 65 x 257 51 -> 46.5 us, Q3 73 x 73 x 289 115 ->
+// 104 us; FP64 Q2 119 -> 106 us.
 template <int K, class S, typename T, class Load, class Epi>
 __device__ __forceinline__ typename Epi::acc_t apply_tile(const MeshDev& m,
                                                           const T* __restrict__ bands,
@@ -442,7 +490,7 @@ __device__ __forceinline__ typename Epi::acc_t apply_tile(const MeshDev& m,
   using TL = Tile<K, S>;
   constexpr int TX = TL::TX, TY = TL::TY, TZ = TL::TZ;
   constexpr int H = TL::H, W = TL::W;
-  constexpr int XW = TL::XW, YW = TL::YW, ZW = TL::ZW;
+  constexpr int XW = TL::XW, YW = TL::YW, ZW = TL::ZW, TXC = TL::TXC;
   constexpr int PL = YW * XW;  // one z plane of the haloed input
   const int nx = m.nn[0], ny = m.nn[1], nz = m.nn[2];
   const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, z0 = blockIdx.z * TZ;
@@ -453,10 +501,10 @@ __device__ __forceinline__ typename Epi::acc_t apply_tile(const MeshDev& m,
   T* T2 = T1 + TL::NT;
   T* U = TL::T_IN_X ? sm + TL::RA : (TL::UV_IN_X ? X : T2 + TL::NT);  // [TZ][TY][XW]
   T* V = U + TL::NU;
-  T* XE = sm + TL::SZ;       // [TZ][TY][TX] input at the owned nodes (kXE)
+  T* XE = sm + TL::SZ;       // [TZ][TY][K TXC] input at the owned nodes (kXE)
   T* BZ = XE + (kXE ? TL::NO : 0);  // [TZ][W][2]   Mz, Kz of row z0 + o
   T* BY = BZ + TL::NBZ;      // [TY][W][3]   cM My + cKy Ky, cKz My, cKx My of row y0 + j
-  T* BX = BY + TL::NBY;      // [2][W][TX]   Mx, Kx of column x0 + i
+  T* BX = BY + TL::NBY;      // [2][W][K TXC]  Mx, Kx of column x0 + i, sorted by residue
   const T* bMx = bands;
   const T* bKx = bMx + (size_t)nx * W;
   const T* bMy = bKx + (size_t)nx * W;
@@ -495,8 +543,8 @@ __device__ __forceinline__ typename Epi::acc_t apply_tile(const MeshDev& m,
       a = bMx[(size_t)gx * W + w];
       b = bKx[(size_t)gx * W + w];
     }
-    BX[w * TX + i] = a;
-    BX[(W + w) * TX + i] = b;
+    BX[w * (K * TXC) + TL::own(i)] = a;
+    BX[(W + w) * (K * TXC) + TL::own(i)] = b;
   }
 
   // load with halo: each thread keeps one x column of the haloed tile (its
@@ -504,10 +552,10 @@ __device__ __forceinline__ typename Epi::acc_t apply_tile(const MeshDev& m,
   // owned nodes' input also to XE
   int nonzero = 0;
   {
-    constexpr int RT = kApplyThreads / XW;  // rows taken per pass
-    const int lx = (int)threadIdx.x % XW, tr = (int)threadIdx.x / XW;
+    constexpr int RT = kApplyThreads / TL::XH;  // rows taken per pass
+    const int lx = (int)threadIdx.x % TL::XH, tr = (int)threadIdx.x / TL::XH;
     if (tr < RT) {
-      const int gx = x0 + lx - H;
+      const int gx = x0 + lx - H, lxs = TL::col(lx);
       const bool xin = gx >= 0 && gx < nx, xown = lx >= H && lx < H + TX;
       for (int row = tr; row < ZW * YW; row += RT) {
         const int lz = row / YW, ly = row - lz * YW;
@@ -516,9 +564,9 @@ __device__ __forceinline__ typename Epi::acc_t apply_tile(const MeshDev& m,
         if (xin && gy >= 0 && gy < ny && gz >= 0 && gz < nz) {
           const bool own = xown && ly >= H && ly < H + TY && lz >= H && lz < H + TZ;
           v = ld(gx + (int64_t)nx * gy + sxy * gz, own);
-          if (kXE && own) XE[((lz - H) * TY + (ly - H)) * TX + (lx - H)] = v;
+          if (kXE && own) XE[((lz - H) * TY + (ly - H)) * (K * TXC) + TL::own(lx - H)] = v;
         }
-        X[row * XW + lx] = v;
+        X[row * XW + lxs] = v;
         nonzero |= (v != T(0));
       }
     }
@@ -542,12 +590,17 @@ __device__ __forceinline__ typename Epi::acc_t apply_tile(const MeshDev& m,
 #pragma unroll
     for (int o = 0; o < TZ; ++o) {
       Acc<T> a1, a2;
-      a1.zero();
-      a2.zero();
 #pragma unroll
       for (int w = 0; w < W; ++w) {
-        a1.add(BZ[2 * (o * W + w)], xv[o + w]);
-        a2.add(BZ[2 * (o * W + w) + 1], xv[o + w]);
+        if (w < Taps<K>::lo(o % K) || w >= Taps<K>::hi(o % K)) continue;
+        const T m1 = BZ[2 * (o * W + w)], k1 = BZ[2 * (o * W + w) + 1];
+        if (w == Taps<K>::lo(o % K)) {
+          a1.first(m1, xv[o + w]);
+          a2.first(k1, xv[o + w]);
+        } else {
+          a1.add(m1, xv[o + w]);
+          a2.add(k1, xv[o + w]);
+        }
       }
       T1[o * PL + c] = a1.get();
       T2[o * PL + c] = a2.get();
@@ -577,13 +630,17 @@ __device__ __forceinline__ typename Epi::acc_t apply_tile(const MeshDev& m,
       if (j < len) {
         const T* by = BY + (j0 + j) * (3 * W);
         Acc<T> au, av;
-        au.zero();
-        av.zero();
 #pragma unroll
         for (int w = 0; w < W; ++w) {
-          au.add(by[3 * w], t1[j + w]);
+          if (w < Taps<K>::lo(j % K) || w >= Taps<K>::hi(j % K)) continue;
+          if (w == Taps<K>::lo(j % K)) {
+            au.first(by[3 * w], t1[j + w]);
+            av.first(by[3 * w + 2], t1[j + w]);
+          } else {
+            au.add(by[3 * w], t1[j + w]);
+            av.add(by[3 * w + 2], t1[j + w]);
+          }
           au.add(by[3 * w + 1], t2[j + w]);
-          av.add(by[3 * w + 2], t1[j + w]);
         }
         du[j * XW] = au.get();
         dv[j * XW] = av.get();
@@ -592,32 +649,46 @@ __device__ __forceinline__ typename Epi::acc_t apply_tile(const MeshDev& m,
   }
   __syncthreads();
   // x pass + output (per-thread partial in the epilogue's type, one
-  // conversion per thread)
-  // (each thread keeps one x column of the owned nodes and walks the rows)
+  // conversion per thread): the owned columns of residue p in the tile, one
+  // after the other; their residue r on the axis (block-wide) gives the taps
   typename Epi::acc_t dot = 0;
-  {
-    constexpr int RT = kApplyThreads / TX;
-    const int lx = (int)threadIdx.x % TX, tr = (int)threadIdx.x / TX;
-    const int gx = x0 + lx;
-    if (tr < RT && gx < nx) {
-      for (int row = tr; row < TZ * TY; row += RT) {
-        const int lz = row / TY, ly = row - lz * TY;
-        const int gy = y0 + ly, gz = z0 + lz;
-        if (gy >= ny || gz >= nz) continue;
-        const T* u = U + row * XW + lx;
-        const T* v = V + row * XW + lx;
-        Acc<T> ax;
-        ax.zero();
+  auto xpass = [&](auto pc, auto rc) {
+    constexpr int P = decltype(pc)::value, R = decltype(rc)::value;
+    constexpr int NC = (TX - P + K - 1) / K;  // columns of the residue
+    for (int it = threadIdx.x; it < NC * TY * TZ; it += blockDim.x) {
+      const int row = it / NC, cx = it - row * NC;
+      const int lz = row / TY, ly = row - lz * TY;
+      const int gx = x0 + cx * K + P, gy = y0 + ly, gz = z0 + lz;
+      if (gx >= nx || gy >= ny || gz >= nz) continue;
+      const T* u = U + row * XW + cx;
+      const T* v = V + row * XW + cx;
+      const T* bx = BX + P * TXC + cx;
+      Acc<T> ax;
 #pragma unroll
-        for (int w = 0; w < W; ++w) {
-          ax.add(BX[w * TX + lx], u[w]);
-          ax.add(BX[(W + w) * TX + lx], v[w]);
-        }
-        dot += ep(gx + (int64_t)nx * gy + sxy * gz, ax.get(),
-                  kXE ? XE[row * TX + lx] : T(0));
+      for (int w = 0; w < W; ++w) {
+        if (w < Taps<K>::lo(R) || w >= Taps<K>::hi(R)) continue;
+        // haloed column cx K + P + w
+        const int at = ((P + w) % K) * TL::PW + (P + w) / K;
+        if (w == Taps<K>::lo(R))
+          ax.first(bx[w * (K * TXC)], u[at]);
+        else
+          ax.add(bx[w * (K * TXC)], u[at]);
+        ax.add(bx[(W + w) * (K * TXC)], v[at]);
       }
+      dot += ep(gx + (int64_t)nx * gy + sxy * gz, ax.get(),
+                kXE ? XE[row * (K * TXC) + P * TXC + cx] : T(0));
     }
-  }
+  };
+  auto residue = [&](auto pc) {
+    constexpr int P = decltype(pc)::value;
+    const int r = (x0 + P) % K;
+    if (r == 0) xpass(pc, std::integral_constant<int, 0>{});
+    if (K > 1 && r == 1) xpass(pc, std::integral_constant<int, 1 % K>{});
+    if (K > 2 && r == 2) xpass(pc, std::integral_constant<int, 2 % K>{});
+  };
+  residue(std::integral_constant<int, 0>{});
+  if constexpr (K > 1) residue(std::integral_constant<int, 1 % K>{});
+  if constexpr (K > 2) residue(std::integral_constant<int, 2 % K>{});
   return dot;
 }
 
@@ -1036,12 +1107,12 @@ static dim3 apply_grid_s(const MeshDev& m) {
               (m.nn[2] + S::Z - 1) / S::Z);
 }
 
-// call f(Shape) with the mesh's tile shape
-template <class F>
+// call f(Shape) with the mesh's tile shape of degree K
+template <int K, class F>
 static auto with_shape(const MeshDev& m, F&& f) {
-  if (m.shape == 1) return f(Shape1{});
-  if (m.shape == 2) return f(Shape2{});
-  return f(Shape0{});
+  if (m.shape == 1) return f(typename Shapes<K>::B{});
+  if (m.shape == 2) return f(typename Shapes<K>::C{});
+  return f(typename Shapes<K>::A{});
 }
 
 // call f(integral_constant<int, k>)
@@ -1063,12 +1134,23 @@ static double tile_cost(const MeshDev& m) {
   return per * g.x * g.y * g.z;
 }
 
+// shared memory of the three shapes' FP64 operator (the largest)
+template <int K>
+static void shapes_smem(size_t sm[kShapes]) {
+  using S = Shapes<K>;
+  sm[0] = apply_smem<K, typename S::A, double>();
+  sm[1] = apply_smem<K, typename S::B, double>();
+  sm[2] = apply_smem<K, typename S::C, double>();
+}
+
 int pick_shape(const MeshDev& m) {
   return with_k(m, [&](auto kc) {
     constexpr int K = decltype(kc)::value;
-    double c[kShapes] = {tile_cost<K, Shape0>(m), tile_cost<K, Shape1>(m), tile_cost<K, Shape2>(m)};
-    size_t sm[kShapes] = {apply_smem<K, Shape0, double>(), apply_smem<K, Shape1, double>(),
-                          apply_smem<K, Shape2, double>()};
+    using S = Shapes<K>;
+    double c[kShapes] = {tile_cost<K, typename S::A>(m), tile_cost<K, typename S::B>(m),
+                         tile_cost<K, typename S::C>(m)};
+    size_t sm[kShapes];
+    shapes_smem<K>(sm);
     int best = 0;
     for (int i = 1; i < kShapes; ++i)
       if (sm[i] <= 200 * 1024 && c[i] < 0.97 * c[best]) best = i;
@@ -1079,19 +1161,21 @@ int pick_shape(const MeshDev& m) {
 bool shape_fits(const MeshDev& m, int shape) {
   return with_k(m, [&](auto kc) {
     constexpr int K = decltype(kc)::value;
-    const size_t sm[kShapes] = {apply_smem<K, Shape0, double>(), apply_smem<K, Shape1, double>(),
-                                apply_smem<K, Shape2, double>()};
+    size_t sm[kShapes];
+    shapes_smem<K>(sm);
     return shape >= 0 && shape < kShapes && sm[shape] <= 200 * 1024;
   });
 }
 
 int cg_blocks(const MeshDev& m) {
-  int na = 0;
-  dim3 g0 = apply_grid_s<Shape0>(m), g1 = apply_grid_s<Shape1>(m), g2 = apply_grid_s<Shape2>(m);
-  na = (int)(g0.x * g0.y * g0.z);
-  na = na > (int)(g1.x * g1.y * g1.z) ? na : (int)(g1.x * g1.y * g1.z);
-  na = na > (int)(g2.x * g2.y * g2.z) ? na : (int)(g2.x * g2.y * g2.z);
-  return na > 1216 ? na : 1216;
+  return with_k(m, [&](auto kc) {
+    using S = Shapes<decltype(kc)::value>;
+    const dim3 g[kShapes] = {apply_grid_s<typename S::A>(m), apply_grid_s<typename S::B>(m),
+                             apply_grid_s<typename S::C>(m)};
+    int na = 1216;
+    for (const dim3& d : g) na = std::max(na, (int)(d.x * d.y * d.z));
+    return na;
+  });
 }
 
 template <typename T>
@@ -1124,7 +1208,7 @@ static cudaError_t apply_t(const MeshDev& m, const T* bands, const double* coef,
   Coefs<T> cf = make_coefs<T>(coef);
   return with_k(m, [&](auto kc) {
     constexpr int K = decltype(kc)::value;
-    return with_shape(m, [&](auto sh) {
+    return with_shape<K>(m, [&](auto sh) {
       using S = decltype(sh);
       cudaError_t e = set_smem<K, S, T>();
       if (e != cudaSuccess) return e;
@@ -1143,7 +1227,7 @@ static cudaError_t cg_apply_t(const MeshDev& m, const T* bands, const double* co
   Coefs<T> cf = make_coefs<T>(coef);
   return with_k(m, [&](auto kc) {
     constexpr int K = decltype(kc)::value;
-    return with_shape(m, [&](auto sh) {
+    return with_shape<K>(m, [&](auto sh) {
       using S = decltype(sh);
       cudaError_t e = set_smem<K, S, T>();
       if (e != cudaSuccess) return e;
@@ -1622,7 +1706,7 @@ cudaError_t run_cg_mixed(const MeshDev& m, const double* bands64, const float* b
     double rel = 0.0;
     e = with_k(m, [&](auto kc) {
       constexpr int K = decltype(kc)::value;
-      return with_shape(m, [&](auto sh) {
+      return with_shape<K>(m, [&](auto sh) {
         return cg_solve_df<K, decltype(sh)>(m, w.bands_df, coef, b, x, rtol, maxit, w, s, &it,
                                              &rel);
       });
