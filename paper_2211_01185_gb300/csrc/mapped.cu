@@ -19,23 +19,23 @@
 //
 // FP64 runs at 1/61 of the FP32 rate on this part, and most of those Newton
 // steps only show that a neighbour does not hold the point.  So a candidate
-// is first screened in FP32 on element-relative Bernstein control points
-// (screen_in).  The element lies in their convex hull, so a point beyond all
-// of them in the direction of a row of the centre's inverse Jacobian is
-// outside, whatever Newton's method would do there: one pass rejects 94 % of
-// the wrong candidates and the ones whose iteration would wander for 20 to 50
-// steps without a root (one lane of those held the kernel for 1.6 ms).  What is left
-// runs the same Newton iteration in FP32, which throws out the candidates
+// is first screened in FP32 on element-relative Bernstein control points.
+// The element lies in their convex hull, so a point beyond all of them in the
+// direction of a row of the centre's inverse Jacobian is outside, whatever
+// Newton's method would do there: three products with tabulated rows
+// (k_frames, screen_hull) reject 94 % of the wrong candidates, among them the
+// ones whose iteration would wander for 20 to 50 steps without a root (one
+// lane of those held the kernel for 1.6 ms).  What is left runs the same
+// Newton iteration in FP32 (screen_newton), which throws out the candidates
 // whose root lies outside by far more than FP32 and the last step can err,
 // hands the rest on with a start good to ~1e-6, and leaves the doubtful ones
 // (no quick convergence, iterates far out, a Jacobian that changes much) to
 // the FP64 iteration from the centre.  polish_in finishes an accepted start
-// with FP64 residuals and the FP32 inverse Jacobian: each step gains about
-// five digits, so two residuals (each a third of the operations of a Newton
-// step) reach the 1e-13.  120,000 points on a Q2 cylinder of 5,280 elements:
-// locate and interpolate a 3-vector 13.6 ms with plain FP64 Newton, 0.44 ms
-// now (what is left: scattered loads of the control points and nodes, and
-// about 300 FP64 operations a point).
+// with double-float residuals and the FP32 inverse Jacobian: each step gains
+// about five digits, so two residuals reach the 1e-13.  120,000 points on a
+// Q2 cylinder of 5,280 elements: locate and interpolate a 3-vector 13.6 ms
+// with plain FP64 Newton, 0.225 ms now
+// (locate 175 us: scattered loads of control points, 16 warps an SM).
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -53,8 +53,12 @@ struct cfdem_mapped {
   int32_t* conn = nullptr;   // [E][(k+1)^3]
   double* nodes = nullptr;   // [N][3]
   double* box = nullptr;     // [E][6] widened lo, hi
+  float4* box32 = nullptr;   // [E][2] the same rounded to FP32
   double* ref = nullptr;     // [E][4] centre of the nodes' box, 1 / its largest half edge
-  float* rel = nullptr;      // [E][(k+1)^3][3] Bernstein control points relative to ref
+  // [E][(k+1)^3] Bernstein control points relative to ref as double-float, high
+  // parts and low parts apart (one 128-bit load a point for the screen)
+  float4 *rel = nullptr, *rel_lo = nullptr;
+  float4* frame = nullptr;   // [E][5] centre Jacobian and hull bounds (k_frames)
   int32_t* cell_start = nullptr;
   int32_t* cell_elems = nullptr;
   double g0[3] = {0, 0, 0}, inv_cs[3] = {0, 0, 0};
@@ -63,6 +67,8 @@ struct cfdem_mapped {
 
 namespace {
 
+using cfdem::df64;
+using cfdem::DfDotAcc;
 using cfdem::Tables;
 
 struct MappedDev {
@@ -70,13 +76,25 @@ struct MappedDev {
   const int32_t* conn;
   const double* nodes;
   const double* box;
+  const float4* box32;
   const double* ref;
-  const float* rel;
+  const float4 *rel, *rel_lo, *frame;
   const int32_t* cell_start;
   const int32_t* cell_elems;
   double g0[3], inv_cs[3];
   int nc[3];
 };
+
+// the boxes rounded to FP32: rounding keeps the order, so a point within a
+// box lies, rounded, within the rounded box
+__global__ void k_round_boxes(int64_t E, const double* __restrict__ box,
+                              float4* __restrict__ box32) {
+  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (e >= E) return;
+  const double* b = box + 6 * e;
+  box32[2 * e] = make_float4((float)b[0], (float)b[1], (float)b[2], 0.0f);
+  box32[2 * e + 1] = make_float4((float)b[3], (float)b[4], (float)b[5], 0.0f);
+}
 
 // values at the GLL nodes -> Bernstein coefficients, per axis
 struct ToBernstein {
@@ -87,7 +105,7 @@ struct ToBernstein {
 template <int K>
 __global__ void k_control_points(int64_t E, ToBernstein tb, const int32_t* __restrict__ conn,
                                  const double* __restrict__ nodes, double* __restrict__ ref,
-                                 float* __restrict__ rel) {
+                                 float* __restrict__ rel, float* __restrict__ rel_lo) {
   constexpr int N = K + 1, NL = N * N * N;
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= 3 * E) return;
@@ -142,7 +160,9 @@ __global__ void k_control_points(int64_t E, ToBernstein tb, const int32_t* __res
     double w = 0.0;
 #pragma unroll
     for (int k = 0; k < N; ++k) w += tb.t[j / (N * N)][k] * u[k][j / N % N][j % N];
-    rel[(e * NL + j) * 3 + ax] = (float)w;
+    const float hi = (float)w;
+    rel[(e * NL + j) * 4 + ax] = hi;
+    rel_lo[(e * NL + j) * 4 + ax] = (float)(w - (double)hi);
   }
 }
 
@@ -174,30 +194,137 @@ __device__ __forceinline__ void bernstein(float t, float* l, float* dl) {
   }
 }
 
-enum Screen { kOutside, kStart, kUnsure };
-
-// The FP32 screen of candidate e at p (see the file comment).  kStart: xi is
-// a start near the cube and Ji the inverse Jacobian there (in the element's
-// scaled coordinates).  kOutside: the root lies outside the cube.  The error
-// of an iterate is taken as four times its quadratic estimate kappa big^2
-// (kappa from the last two steps, at least 1) and must leave a margin of
-// 1e-2, ten times what FP32 loses of xi in the flattest element let through.
+// What the screen needs of an element before it looks at its control points:
+// the inverse Jacobian at the centre (rows J_a), the range of J_a . X over the
+// control points -- the element lies in their convex hull, so a point whose
+// J_a . q lies outside that range is outside the element --, the centre's
+// image X_0 and the Jacobian's determinant.  The ranges are widened by what
+// FP32 loses in J_a . q for coordinates below ten and by the 1e-10 by which
+// xi may pass the cube.  frame[5]: (J_0, lo_0), (J_1, lo_1), (J_2, lo_2),
+// (hi, det), (X_0, 0); det = 0 marks an element too flat for FP32.
 template <int K>
-__device__ __forceinline__ Screen screen_in(const MappedDev& md, int64_t e, const double p[3],
-                                            float xi[3], float Ji[3][3]) {
-  constexpr int NQ = K + 1, NL = NQ * NQ * NQ;
-  const double* rf = md.ref + 4 * e;
-  const float* P = md.rel + e * (NL * 3);
-  const double inv = rf[3];
-  if (!(inv > 0.0)) return kUnsure;
-  float q[3];
+__global__ void k_frames(int64_t E, const double* __restrict__ ref,
+                         const float4* __restrict__ rel, float4* __restrict__ frame) {
+  constexpr int N = K + 1, NL = N * N * N;
+  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (e >= E) return;
+  const float4* P = rel + e * NL;
+  float b[N], db[N];
+  bernstein<K>(0.5f, b, db);
+  double X[3] = {0.0, 0.0, 0.0}, J[3][3] = {{0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}};
+  for (int j = 0; j < NL; ++j) {
+    const float4 B = P[j];
+    const double v[3] = {(double)B.x, (double)B.y, (double)B.z};
+    double w = 0.0, w0 = 0.0, w1 = 0.0, w2 = 0.0;
+#pragma unroll
+    for (int c = 0; c < N; ++c)
+#pragma unroll
+      for (int bb = 0; bb < N; ++bb)
+#pragma unroll
+        for (int a = 0; a < N; ++a)
+          if (j == a + N * (bb + N * c)) {
+            w = (double)b[a] * b[bb] * b[c];
+            w0 = (double)db[a] * b[bb] * b[c];
+            w1 = (double)b[a] * db[bb] * b[c];
+            w2 = (double)b[a] * b[bb] * db[c];
+          }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      X[i] += w * v[i];
+      J[i][0] += w0 * v[i];
+      J[i][1] += w1 * v[i];
+      J[i][2] += w2 * v[i];
+    }
+  }
+  double A[3][3], nrm = 1.0;  // adjugate
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    q[i] = (float)((p[i] - rf[i]) * inv);
-    xi[i] = 0.5f;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const int i1 = (j + 1) % 3, i2 = (j + 2) % 3, j1 = (i + 1) % 3, j2 = (i + 2) % 3;
+      A[i][j] = J[i1][j1] * J[i2][j2] - J[i1][j2] * J[i2][j1];
+    }
+    nrm *= sqrt(J[0][i] * J[0][i] + J[1][i] * J[1][i] + J[2][i] * J[2][i]);
   }
-  float prev = 0.0f, det0 = 0.0f;
-  for (int it = 0; it < 10; ++it) {
+  const double det = J[0][0] * A[0][0] + J[0][1] * A[1][0] + J[0][2] * A[2][0];
+  bool ok = ref[4 * e + 3] > 0.0 && fabs(det) >= 1e-3 * nrm && nrm > 1e-12;
+  float4 f[5];
+  float hi[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    float r[3];
+    float row = 0.0f;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      r[i] = ok ? (float)(A[a][i] / det) : 0.0f;
+      row += fabsf(r[i]);
+    }
+    ok = ok && row <= 500.0f;
+    double lo = 1e30, up = -1e30;
+    for (int j = 0; j < NL; ++j) {
+      const double t = (double)r[0] * P[j].x + (double)r[1] * P[j].y + (double)r[2] * P[j].z;
+      lo = fmin(lo, t);
+      up = fmax(up, t);
+    }
+    const float m = 1e-5f * row + 1e-4f;
+    f[a] = make_float4(r[0], r[1], r[2], (float)lo - m);
+    hi[a] = (float)up + m;
+  }
+  f[3] = make_float4(hi[0], hi[1], hi[2], ok ? (float)det : 0.0f);
+  f[4] = make_float4((float)X[0], (float)X[1], (float)X[2], 0.0f);
+  for (int q = 0; q < 5; ++q) frame[5 * e + q] = f[q];
+}
+
+enum Screen { kOutside, kStart, kUnsure };
+
+// The hull test of candidate e at p; kStart: not excluded, and xi is the
+// first Newton iterate from the centre, `step` its step and det0 the
+// centre's determinant.  kUnsure: no FP32 screen for this element.
+__device__ __forceinline__ Screen screen_hull(const MappedDev& md, int64_t e, const double p[3],
+                                              float q[3], float xi[3], float* step,
+                                              float* det0) {
+  const float4* f = md.frame + 5 * e;
+  const double* rf = md.ref + 4 * e;
+  const float4 h = __ldg(f + 3);
+  if (h.w == 0.0f) return kUnsure;
+  const double inv = rf[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) q[i] = (float)((p[i] - rf[i]) * inv);
+  const float4 X0 = __ldg(f + 4);
+  const float up[3] = {h.x, h.y, h.z};
+  const float d0[3] = {X0.x - q[0], X0.y - q[1], X0.z - q[2]};
+  float big = 0.0f;
+  bool out = false;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const float4 r = __ldg(f + a);
+    const float t = fmaf(r.z, q[2], fmaf(r.y, q[1], r.x * q[0]));
+    out = out || t < r.w || t > up[a];
+    const float d = fmaf(r.z, d0[2], fmaf(r.y, d0[1], r.x * d0[0]));
+    xi[a] = 0.5f - d;
+    big = fmaxf(big, fabsf(d));
+  }
+  *step = big;
+  *det0 = h.w;
+  return out ? kOutside : kStart;
+}
+
+// The FP32 Newton screen (see the file comment), from the hull test's first
+// iterate.  kStart: xi is a start near the cube and Ji the inverse Jacobian
+// there (in the element's scaled coordinates).  kOutside: the root lies
+// outside the cube.  The error of an iterate is taken as four times its
+// quadratic estimate kappa big^2 (kappa from the last two steps, at least 1)
+// and must leave a margin of 1e-2, ten times what FP32 loses of xi in the
+// flattest element let through.
+template <int K>
+__device__ __forceinline__ Screen screen_newton(const MappedDev& md, int64_t e, const float q[3],
+                                                float step, float det0, float xi[3],
+                                                float Ji[3][3]) {
+  constexpr int NQ = K + 1, NL = NQ * NQ * NQ;
+  const float4* P = md.rel + e * NL;
+  float prev = step;
+  if (!(prev <= 4.0f)) return kUnsure;
+  for (int it = 1; it < 10; ++it) {
     float l[3][NQ], dl[3][NQ];
 #pragma unroll
     for (int a = 0; a < 3; ++a) bernstein<K>(xi[a], l[a], dl[a]);
@@ -210,13 +337,15 @@ __device__ __forceinline__ Screen screen_in(const MappedDev& md, int64_t e, cons
       for (int b = 0; b < NQ; ++b) {
         float v[3] = {0.f, 0.f, 0.f}, v0[3] = {0.f, 0.f, 0.f};
 #pragma unroll
-        for (int a = 0; a < NQ; ++a)
+        for (int a = 0; a < NQ; ++a) {
+          const float4 B = __ldg(P + a + NQ * (b + NQ * c));
+          const float w[3] = {B.x, B.y, B.z};
 #pragma unroll
           for (int i = 0; i < 3; ++i) {
-            const float w = __ldg(P + (a + NQ * (b + NQ * c)) * 3 + i);
-            v[i] = fmaf(l[0][a], w, v[i]);
-            v0[i] = fmaf(dl[0][a], w, v0[i]);
+            v[i] = fmaf(l[0][a], w[i], v[i]);
+            v0[i] = fmaf(dl[0][a], w[i], v0[i]);
           }
+        }
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
           u[i] = fmaf(l[1][b], v[i], u[i]);
@@ -241,37 +370,7 @@ __device__ __forceinline__ Screen screen_in(const MappedDev& md, int64_t e, cons
         Ji[i][j] = J[i1][j1] * J[i2][j2] - J[i1][j2] * J[i2][j1];
       }
     const float det = J[0][0] * Ji[0][0] + J[0][1] * Ji[1][0] + J[0][2] * Ji[2][0];
-    if (it == 0) {
-      // a flat element: its FP32 Jacobian has too few digits
-      float nrm = 1.0f;
-#pragma unroll
-      for (int j = 0; j < 3; ++j)
-        nrm *= sqrtf(J[0][j] * J[0][j] + J[1][j] * J[1][j] + J[2][j] * J[2][j]);
-      if (!(fabsf(det) >= 1e-3f * nrm && nrm > 1e-12f)) return kUnsure;
-      det0 = det;
-      // the hull test along the rows of the adjugate (any direction is a
-      // valid one): the margin covers the rounding of the row's products with
-      // coordinates below ten, and the 1e-10 by which xi may pass the cube
-      float lo[3], hi[3];
-#pragma unroll
-      for (int j = 0; j < NL; ++j)
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-          float t = Ji[a][0] * (__ldg(P + 3 * j) - q[0]);
-          t = fmaf(Ji[a][1], __ldg(P + 3 * j + 1) - q[1], t);
-          t = fmaf(Ji[a][2], __ldg(P + 3 * j + 2) - q[2], t);
-          lo[a] = j == 0 ? t : fminf(lo[a], t);
-          hi[a] = j == 0 ? t : fmaxf(hi[a], t);
-        }
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        const float m = 1e-5f * (fabsf(Ji[a][0]) + fabsf(Ji[a][1]) + fabsf(Ji[a][2])) +
-                        1e-4f * fabsf(det);
-        if (lo[a] > m || hi[a] < -m) return kOutside;
-      }
-    } else if (!(det * det0 > 0.0f && fabsf(det) >= 0.05f * fabsf(det0))) {
-      return kUnsure;
-    }
+    if (!(det * det0 > 0.0f && fabsf(det) >= 0.05f * fabsf(det0))) return kUnsure;
     const float id = 1.0f / det;
     float big = 0.0f, out = 0.0f, row = 0.0f;
 #pragma unroll
@@ -289,22 +388,44 @@ __device__ __forceinline__ Screen screen_in(const MappedDev& md, int64_t e, cons
     }
     // far out, or a very flat element (FP32 leaves 2e-6 row of xi); also NaN
     if (!(out <= 2.5f && big <= 4.0f && row <= 500.0f)) return kUnsure;
-    if (it > 0) {
-      const float kappa = fmaxf(1.0f, big / fmaxf(prev * prev, 1e-12f));
-      const float err = 4.0f * kappa * big * big;
-      // kappa is only an estimate where the steps do shrink
-      if (big <= 0.25f * prev || big <= 1e-5f) {
-        if (out > 1e-2f + err) return kOutside;
-        // one more FP32 step costs a twentieth of the FP64 residual it saves
-        if (big <= (it < 5 ? 2e-5f : 2e-3f) && out <= 1.1e-2f + err) return kStart;
-      }
+    const float kappa = fmaxf(1.0f, big / fmaxf(prev * prev, 1e-12f));
+    const float err = 4.0f * kappa * big * big;
+    // kappa is only an estimate where the steps do shrink
+    if (big <= 0.25f * prev || big <= 1e-5f) {
+      if (out > 1e-2f + err) return kOutside;
+      // one more FP32 step costs a fraction of the residual it saves
+      if (big <= (it < 5 ? 2e-5f : 2e-3f) && out <= 1.1e-2f + err) return kStart;
     }
     prev = big;
   }
   return kUnsure;
 }
 
-// Finishes a start of the screen: X_e(xi) = p with FP64 residuals and the
+// Bernstein basis of degree K at t in double-float
+template <int K>
+__device__ __forceinline__ void bernstein_df(df64 t, df64* l) {
+  const df64 s = df64(1.0f) - t;
+  if (K == 1) {
+    l[0] = s;
+    l[1] = t;
+  } else if (K == 2) {
+    const df64 st = s * t;
+    l[0] = s * s;
+    l[1] = st + st;
+    l[2 % (K + 1)] = t * t;
+  } else {
+    const df64 ss = s * s, tt = t * t;
+    const df64 a = ss * t, b = s * tt;
+    l[0] = ss * s;
+    l[1] = a + a + a;
+    l[2 % (K + 1)] = b + b + b;
+    l[3 % (K + 1)] = tt * t;
+  }
+}
+
+// Finishes a start of the screen: X_e(xi) = p with residuals in double-float
+// (the element's control points relative to its centre carry 2^-48 of its
+// size, more than FP64 keeps of coordinates 32 element sizes away) and the
 // FP32 inverse Jacobian.  A linear iteration with ratio rho ~ 1e-5: done when
 // the step is at most 1e-13, or the step that would follow it (step * rho,
 // rho from the last two) at most 1e-15 -- the latter only where coordinates
@@ -313,55 +434,70 @@ __device__ __forceinline__ Screen screen_in(const MappedDev& md, int64_t e, cons
 // in the cube, 0 when xi lies outside it, -1 when the steps do not shrink
 // fast.
 template <int K>
-__device__ __forceinline__ int polish_in(const MappedDev& md, const Tables& tb, int64_t e,
-                                         const double p[3], const float start[3],
-                                         const float Ji[3][3], double xi_out[3]) {
+__device__ __forceinline__ int polish_in(const MappedDev& md, int64_t e, const double p[3],
+                                         const float start[3], const float Ji[3][3],
+                                         double xi_out[3]) {
   constexpr int NQ = K + 1, NL = NQ * NQ * NQ;
-  const int32_t* cn = md.conn + e * NL;
-  const double inv = md.ref[4 * e + 3];
-  double xi[3] = {(double)start[0], (double)start[1], (double)start[2]};
+  const float4* Ph = md.rel + e * NL;
+  const float4* Pl = md.rel_lo + e * NL;
+  const double* rf = md.ref + 4 * e;
+  const double inv = rf[3];
   const bool near = fmax(fmax(fabs(p[0]), fabs(p[1])), fabs(p[2])) * inv <= 256.0;
+  df64 xi[3], q[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    xi[i] = df64(start[i]);
+    q[i] = cfdem::df_from_double_int((p[i] - rf[i]) * inv);
+  }
   float prev = 1.0f;
   for (int it = 0; it < 8; ++it) {
-    double l[3][NQ];
+    df64 l[3][NQ];
 #pragma unroll
-    for (int a = 0; a < 3; ++a)
-      cfdem::lagrange<K, double>(tb.z, tb.lw, xi[a], l[a], (double*)nullptr);
-    double X[3] = {0.0, 0.0, 0.0};
+    for (int a = 0; a < 3; ++a) bernstein_df<K>(xi[a], l[a]);
+    DfDotAcc X[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) X[i].zero();
 #pragma unroll
     for (int c = 0; c < NQ; ++c) {
-      double u[3] = {0.0, 0.0, 0.0};
+      DfDotAcc u[3];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) u[i].zero();
 #pragma unroll
       for (int b = 0; b < NQ; ++b) {
-        double v[3] = {0.0, 0.0, 0.0};
+        DfDotAcc v[3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) v[i].zero();
 #pragma unroll
         for (int a = 0; a < NQ; ++a) {
-          const double* P = md.nodes + 3 * (int64_t)__ldg(cn + a + NQ * (b + NQ * c));
-#pragma unroll
-          for (int i = 0; i < 3; ++i) v[i] = fma(l[0][a], __ldg(P + i), v[i]);
+          const float4 H = __ldg(Ph + a + NQ * (b + NQ * c)), L = __ldg(Pl + a + NQ * (b + NQ * c));
+          v[0].add(l[0][a], df64(H.x, L.x));
+          v[1].add(l[0][a], df64(H.y, L.y));
+          v[2].add(l[0][a], df64(H.z, L.z));
         }
 #pragma unroll
-        for (int i = 0; i < 3; ++i) u[i] = fma(l[1][b], v[i], u[i]);
+        for (int i = 0; i < 3; ++i) u[i].add(l[1][b], v[i].get());
       }
 #pragma unroll
-      for (int i = 0; i < 3; ++i) X[i] = fma(l[2][c], u[i], X[i]);
+      for (int i = 0; i < 3; ++i) X[i].add(l[2][c], u[i].get());
     }
     float r[3], big = 0.0f;
 #pragma unroll
-    for (int i = 0; i < 3; ++i) r[i] = (float)((X[i] - p[i]) * inv);
+    for (int i = 0; i < 3; ++i) r[i] = (X[i].get() - q[i]).hi;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       const float d = Ji[a][0] * r[0] + Ji[a][1] * r[1] + Ji[a][2] * r[2];
-      xi[a] -= (double)d;
+      xi[a] = xi[a] - df64(d);
       big = fmaxf(big, fabsf(d));
     }
     if (!(big <= 0.1f * prev || big <= 1e-13f)) return -1;  // also NaN
     if (big <= 1e-13f || (near && it > 0 && big * (big / prev) <= 1e-15f)) {
 #pragma unroll
-      for (int a = 0; a < 3; ++a)
-        if (!(xi[a] >= -1e-10 && xi[a] <= 1.0 + 1e-10)) return 0;
+      for (int a = 0; a < 3; ++a) {
+        xi_out[a] = (double)xi[a].hi + (double)xi[a].lo;
+        if (!(xi_out[a] >= -1e-10 && xi_out[a] <= 1.0 + 1e-10)) return 0;
+      }
 #pragma unroll
-      for (int a = 0; a < 3; ++a) xi_out[a] = fmin(fmax(xi[a], 0.0), 1.0);
+      for (int a = 0; a < 3; ++a) xi_out[a] = fmin(fmax(xi_out[a], 0.0), 1.0);
       return 1;
     }
     prev = big;
@@ -453,47 +589,85 @@ __device__ __noinline__ bool newton_in(const MappedDev& md, const Tables& tb, in
   return false;
 }
 
+// small blocks, and registers for 16 warps an SM: the kernel waits on its
+// scattered loads
+constexpr int kLocateBlock = 64;
+
 template <int K>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(kLocateBlock, K == 3 ? 6 : 8)
 k_locate_mapped(MappedDev md, Tables tb, int64_t n, const double* __restrict__ x,
                 int32_t* __restrict__ elem, double* __restrict__ xi) {
+  constexpr unsigned FULL = 0xffffffffu;
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const double p[3] = {x[3 * i], x[3 * i + 1], x[3 * i + 2]};
+  const bool live = i < n;  // every thread stays for the warp's votes
+  double p[3] = {0.0, 0.0, 0.0};
+  if (live) {
+    p[0] = x[3 * i];
+    p[1] = x[3 * i + 1];
+    p[2] = x[3 * i + 2];
+  }
+  const float pf[3] = {(float)p[0], (float)p[1], (float)p[2]};
   int32_t found = -1;
   double xo[3] = {0.0, 0.0, 0.0};
   int ci[3];
-  bool in_grid = true;
+  bool in_grid = live;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     const double t = (p[a] - md.g0[a]) * md.inv_cs[a];
     in_grid = in_grid && t >= 0.0 && t <= (double)md.nc[a];  // false for NaN
     ci[a] = in_grid ? min((int)t, md.nc[a] - 1) : 0;
   }
+  int32_t s = 0, end = 0;
   if (in_grid) {
     const int64_t cell = ci[0] + (int64_t)md.nc[0] * (ci[1] + (int64_t)md.nc[1] * ci[2]);
-    int32_t s = md.cell_start[cell];
-    const int32_t end = md.cell_start[cell + 1];
-    // the screens of a warp run together, then its FP64 finishes
-    while (found < 0) {
-      Screen sc = kOutside;
-      int32_t e = -1;
-      float start[3], Ji[3][3];
-      for (; s < end && sc == kOutside; ++s) {
-        e = md.cell_elems[s];
-        const double* bx = md.box + 6 * (int64_t)e;
-        if (!(p[0] >= bx[0] && p[0] <= bx[3] && p[1] >= bx[1] && p[1] <= bx[4] &&
-              p[2] >= bx[2] && p[2] <= bx[5]))
-          continue;
-        sc = screen_in<K>(md, e, p, start, Ji);
-      }
-      if (sc == kOutside) break;
-      int in = -1;
-      if (sc == kStart) in = polish_in<K>(md, tb, e, p, start, Ji, xo);
-      if (in < 0) in = newton_in<K>(md, tb, e, p, xo) ? 1 : 0;
-      if (in) found = e;
-    }
+    s = md.cell_start[cell];
+    end = md.cell_start[cell + 1];
   }
+  // the next element of the cell whose widened box holds the point (-1: none
+  // left); the FP32 test on the rounded box lets every one of them through
+  auto next = [&]() -> int32_t {
+    while (s < end) {
+      const int32_t e = md.cell_elems[s++];
+      const float4 lo = __ldg(md.box32 + 2 * (int64_t)e), hi = __ldg(md.box32 + 2 * (int64_t)e + 1);
+      if (!(pf[0] >= lo.x && pf[0] <= hi.x && pf[1] >= lo.y && pf[1] <= hi.y && pf[2] >= lo.z &&
+            pf[2] <= hi.z))
+        continue;
+      const double* bx = md.box + 6 * (int64_t)e;
+      if (p[0] >= bx[0] && p[0] <= bx[3] && p[1] >= bx[1] && p[1] <= bx[4] && p[2] >= bx[2] &&
+          p[2] <= bx[5])
+        return e;
+    }
+    return -1;
+  };
+  // The lanes' phases run together: each finds its next candidate that the
+  // hull test does not exclude, then those take their Newton screens, then
+  // the accepted ones are finished (with the phases in one loop 5 of 32 lanes
+  // were at work)
+  bool done = !in_grid;
+  while (__any_sync(FULL, !done)) {
+    Screen sc = kOutside;
+    int32_t e = -1;
+    float q[3], start[3], Ji[3][3], step = 0.0f, det0 = 0.0f;
+    if (!done)
+      while ((e = next()) >= 0 &&
+             (sc = screen_hull(md, e, p, q, start, &step, &det0)) == kOutside) {
+      }
+    __syncwarp();
+    done = done || e < 0;
+    if (!done && sc == kStart) sc = screen_newton<K>(md, e, q, step, det0, start, Ji);
+    __syncwarp();
+    if (!done && sc != kOutside) {
+      int in = -1;
+      if (sc == kStart) in = polish_in<K>(md, e, p, start, Ji, xo);
+      if (in < 0) in = newton_in<K>(md, tb, e, p, xo) ? 1 : 0;
+      if (in) {
+        found = e;
+        done = true;
+      }
+    }
+    __syncwarp();
+  }
+  if (!live) return;
   elem[i] = found;
   if (xi) {
     xi[3 * i] = found >= 0 ? xo[0] : 0.0;
@@ -588,8 +762,11 @@ MappedDev dev_view(const cfdem_mapped* m) {
   d.conn = m->conn;
   d.nodes = m->nodes;
   d.box = m->box;
+  d.box32 = m->box32;
   d.ref = m->ref;
   d.rel = m->rel;
+  d.rel_lo = m->rel_lo;
+  d.frame = m->frame;
   d.cell_start = m->cell_start;
   d.cell_elems = m->cell_elems;
   for (int a = 0; a < 3; ++a) {
@@ -613,7 +790,8 @@ struct Guard {
 };
 
 void release(cfdem_mapped* m) {
-  void* ps[] = {m->conn, m->nodes, m->box, m->ref, m->rel, m->cell_start, m->cell_elems};
+  void* ps[] = {m->conn, m->nodes, m->box, m->box32, m->ref, m->rel, m->rel_lo, m->frame, m->cell_start,
+                m->cell_elems};
   for (void* p : ps)
     if (p) cudaFree(p);
   delete m;
@@ -734,20 +912,29 @@ extern "C" cfdem_status cfdem_mapped_create(cfdem_mapped_t* out, int device, int
         release(m);
         return CFDEM_ENOMEM;
       }
-      if (cudaMalloc((void**)&m->ref, sizeof(double) * 4 * n_elem) != cudaSuccess ||
-          cudaMalloc((void**)&m->rel, sizeof(float) * 3 * n_elem * nl) != cudaSuccess) {
+      if (cudaMalloc((void**)&m->box32, sizeof(float4) * 2 * n_elem) != cudaSuccess ||
+          cudaMalloc((void**)&m->ref, sizeof(double) * 4 * n_elem) != cudaSuccess ||
+          cudaMalloc((void**)&m->rel, sizeof(float4) * n_elem * nl) != cudaSuccess ||
+          cudaMalloc((void**)&m->rel_lo, sizeof(float4) * n_elem * nl) != cudaSuccess ||
+          cudaMalloc((void**)&m->frame, sizeof(float4) * 5 * n_elem) != cudaSuccess) {
         release(m);
         return CFDEM_ENOMEM;
       }
       const unsigned eb = (unsigned)((3 * n_elem + 127) / 128);
       const ToBernstein tb = to_bernstein(degree, m->tab.z);
+      float *hi = reinterpret_cast<float*>(m->rel), *lo = reinterpret_cast<float*>(m->rel_lo);
       if (degree == 1)
-        k_control_points<1><<<eb, 128>>>(n_elem, tb, m->conn, m->nodes, m->ref, m->rel);
+        k_control_points<1><<<eb, 128>>>(n_elem, tb, m->conn, m->nodes, m->ref, hi, lo);
       if (degree == 2)
-        k_control_points<2><<<eb, 128>>>(n_elem, tb, m->conn, m->nodes, m->ref, m->rel);
+        k_control_points<2><<<eb, 128>>>(n_elem, tb, m->conn, m->nodes, m->ref, hi, lo);
       if (degree == 3)
-        k_control_points<3><<<eb, 128>>>(n_elem, tb, m->conn, m->nodes, m->ref, m->rel);
-      cfdem::count_launches(1);
+        k_control_points<3><<<eb, 128>>>(n_elem, tb, m->conn, m->nodes, m->ref, hi, lo);
+      const unsigned nb = (unsigned)((n_elem + 127) / 128);
+      k_round_boxes<<<nb, 128>>>(n_elem, m->box, m->box32);
+      if (degree == 1) k_frames<1><<<nb, 128>>>(n_elem, m->ref, m->rel, m->frame);
+      if (degree == 2) k_frames<2><<<nb, 128>>>(n_elem, m->ref, m->rel, m->frame);
+      if (degree == 3) k_frames<3><<<nb, 128>>>(n_elem, m->ref, m->rel, m->frame);
+      cfdem::count_launches(3);
       // locate may run on any stream, also one that does not wait for this one
       if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(0) != cudaSuccess) {
         release(m);
@@ -773,11 +960,11 @@ extern "C" cfdem_status cfdem_mapped_locate(cfdem_mapped_t m, int64_t n, const d
   if (n == 0) return CFDEM_OK;
   Guard g(m->device);
   const MappedDev d = dev_view(m);
-  const unsigned nb = (unsigned)((n + 127) / 128);
+  const unsigned nb = (unsigned)((n + kLocateBlock - 1) / kLocateBlock);
   cudaStream_t s = (cudaStream_t)stream;
-  if (m->k == 1) k_locate_mapped<1><<<nb, 128, 0, s>>>(d, m->tab, n, x, elem, xi);
-  if (m->k == 2) k_locate_mapped<2><<<nb, 128, 0, s>>>(d, m->tab, n, x, elem, xi);
-  if (m->k == 3) k_locate_mapped<3><<<nb, 128, 0, s>>>(d, m->tab, n, x, elem, xi);
+  if (m->k == 1) k_locate_mapped<1><<<nb, kLocateBlock, 0, s>>>(d, m->tab, n, x, elem, xi);
+  if (m->k == 2) k_locate_mapped<2><<<nb, kLocateBlock, 0, s>>>(d, m->tab, n, x, elem, xi);
+  if (m->k == 3) k_locate_mapped<3><<<nb, kLocateBlock, 0, s>>>(d, m->tab, n, x, elem, xi);
   cfdem::count_launches(1);
   return cudaGetLastError() == cudaSuccess ? CFDEM_OK : CFDEM_ECUDA;
 }
