@@ -408,9 +408,9 @@ cfdem_status ensure_particles(cfdem_t c, int64_t n) {
 
 void free_mesh_arena(cfdem_t c) {
   void* ps[] = {c->eps64, c->eps32, c->b, c->S, c->vol, c->cg.r, c->cg.z, c->cg.p0,
-                c->cg.p1, c->cg.Ap, c->cg.dinv, c->cg.xcor, c->cg.r32, c->cg.z32,
+                c->cg.p1, c->cg.Ap, c->cg.dinv, c->cg.r32, c->cg.z32,
                 c->cg.q0, c->cg.q1, c->cg.Aq, c->cg.dinv32, c->cg.d32, c->cg.partials,
-                c->cg.sc, c->cg.zn, c->cg.zn32, c->cg.rin32, c->cg.x_df, c->cg.r_df,
+                c->cg.sc, c->cg.zn32, c->cg.rin32, c->cg.x_df, c->cg.r_df,
                 c->cg.Ap_df, c->cg.p0_df, c->cg.p1_df, c->adj_geps,
                 c->adj_lam, c->adj_gq, c->rhs_local, c->semi, c->tune_x, c->src_acc,
                 c->src_max, c->nodal_df};
@@ -464,7 +464,6 @@ cfdem_status alloc_mesh_arena(cfdem_t c) {
   CK(grow(&w.Aq, nn), "cg");
   CK(grow(&w.dinv32, nn), "cg");
   CK(grow(&w.d32, nn), "cg");
-  CK(grow(&w.zn, nn), "cg");
   CK(grow(&w.zn32, nn), "cg");
   CK(grow(&w.rin32, nn), "cg");
   {

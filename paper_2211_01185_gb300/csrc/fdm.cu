@@ -478,6 +478,7 @@ __global__ void k_fdm_slab(SlabArgs sa, const float* __restrict__ in, int in_str
   if (done && *(volatile const int*)done) return;
   __shared__ double red[32];
   float rz = 0.f;
+  double rz64 = 0.0, rzo64 = 0.0;
   extern __shared__ __align__(16) float fsm[];
   const int nx = sa.nx, ny = sa.ny, nz = sa.nz;
   const SlabAxis ax = slab_axis(nx), ay = slab_axis(ny);
@@ -561,18 +562,35 @@ __global__ void k_fdm_slab(SlabArgs sa, const float* __restrict__ in, int in_str
       __syncthreads();
     }
     float* dst = out + (int64_t)z * out_stride;
-    const float* rr = dot.r ? dot.r + (int64_t)z * nx * ny : nullptr;
+    const int64_t plane = (int64_t)z * nx * ny;
+    const float* rr = INV && dot.r ? dot.r + plane : nullptr;
+    const double* r64 = INV && dot.r64 ? dot.r64 + plane : nullptr;
+    const float* zo = INV && dot.z_old ? dot.z_old + plane : nullptr;
     for (int y = wid; y < ny; y += nw) {
       const float* row = X + slot_of(ay, y) * lx;
       for (int x = lane; x < nx; x += 32) {
         const float v = row[slot_of(ax, x)];
         dst[y * nx + x] = v;
         if (rr) rz = fmaf(rr[y * nx + x], v, rz);
+        if (r64) {
+          const double rd = r64[y * nx + x];
+          rz64 = fma(rd, double_from_float_int(v), rz64);
+          if (zo) rzo64 = fma(rd, double_from_float_int(zo[y * nx + x]), rzo64);
+        }
       }
     }
     __syncthreads();
   }
-  if (dot.r) {
+  if (INV && dot.r64) {
+    double vals[2] = {block_sum(rz64, red), 0.0};
+    if (!dot.first) vals[1] = block_sum(rzo64, red);
+    double o[2];
+    if (last_block_reduce(dot.partials, 2, vals, &dot.sc->ticket, o, red) && threadIdx.x == 0) {
+      if (!dot.first) dot.sc->beta = (o[0] - o[1]) / dot.sc->rz;
+      dot.sc->rz = o[0];
+    }
+  }
+  if (INV && dot.r) {
     const double sblk = block_sum(rz, red);
     double vals[1] = {sblk};
     double o[1];

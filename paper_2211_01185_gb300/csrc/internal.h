@@ -255,9 +255,13 @@ cudaError_t fdm_create(const MeshDev& m, const Tables& t, const double coef[4], 
                        const char** why);
 // r . z of the CG formed by the FDM's last pass (slab form only): r the
 // residual the FDM was applied to (FP32), the block sums go to partials,
-// rz and (unless first) the Fletcher-Reeves beta to sc.
+// rz and (unless first) the Fletcher-Reeves beta to sc.  With r64 (the FP64
+// residual) instead of r the sums are FP64 and, unless first, r . z_old is
+// formed too, for the Polak-Ribiere beta.
 struct FdmDot {
   const float* r = nullptr;
+  const double* r64 = nullptr;
+  const float* z_old = nullptr;
   double* partials = nullptr;
   CgScalars* sc = nullptr;
   int first = 0;
@@ -273,7 +277,7 @@ int fdm_tile(const FdmPlan* p);
 
 struct CgWork {
   // FP64 vectors
-  double *r, *z, *p0, *p1, *Ap, *dinv, *xcor, *zn;
+  double *r, *z, *p0, *p1, *Ap, *dinv;
   // FP32 vectors (mixed inner solve, FDM conversions)
   float *r32, *z32, *q0, *q1, *Aq, *dinv32, *d32, *zn32, *rin32;
   FdmPlan* fdm;       // fast-diagonalisation preconditioner, or null (Jacobi)

@@ -399,17 +399,30 @@ struct LoadDir {
     return v;
   }
 };
-// the same for FP32 directions promoted to df64
-struct LoadDirF32 {
+// CG direction of the FP64 solve from the FP32 preconditioned residual
+struct LoadDir64 {
   const float* z;
-  const float* p_old;
-  float* p_new;
-  float beta;
+  const double* p_old;
+  double* p_new;
+  double beta;
   bool first;
-  __device__ __forceinline__ df64 operator()(int64_t g, bool own) const {
-    float v = first ? z[g] : fmaf(beta, p_old[g], z[g]);
+  __device__ __forceinline__ double operator()(int64_t g, bool own) const {
+    const double zv = double_from_float_int(z[g]);
+    const double v = first ? zv : fma(beta, p_old[g], zv);
     if (own) p_new[g] = v;
-    return df64(v);
+    return v;
+  }
+};
+// the same formed and applied in double-float, the direction kept in FP64
+struct LoadDirSplit {
+  const float* z;
+  const double* p_old;
+  double* p_new;
+  df64 beta;
+  __device__ __forceinline__ df64 operator()(int64_t g, bool own) const {
+    const df64 v = df64(z[g]) + beta * df_from_double_int(p_old[g]);
+    if (own) p_new[g] = double_from_df_int(v);
+    return v;
   }
 };
 // CG direction in double-float from the FP32 preconditioned residual:
@@ -447,6 +460,17 @@ struct EpiStoreDf {
   __device__ __forceinline__ float operator()(int64_t g, df64 acc, df64) const {
     y[g] = acc;
     return __ldcg(reinterpret_cast<const float*>(p + g)) * acc.hi;
+  }
+};
+// df64 image of an FP64 direction, stored in FP64; the dot product in df64
+struct EpiStoreSplit {
+  using acc_t = df64;
+  static constexpr bool kXE = false;
+  double* y;
+  const double* p;  // the direction, written by this block's load phase
+  __device__ __forceinline__ df64 operator()(int64_t g, df64 acc, df64) const {
+    y[g] = double_from_df_int(acc);
+    return df_from_double_int(__ldcg(p + g)) * acc;
   }
 };
 // residual r = b - A x in df64; r32 = high part (input of the FP32
@@ -728,6 +752,60 @@ k_cg_apply(MeshDev m, const T* __restrict__ bands, Coefs<T> cf, const T* __restr
   }
 }
 
+// The FP64 solve with the FDM takes its operator in FP64 while the residual
+// is not small against b, and in double-float from then on: with |r| <= 1e-4
+// |b| the direction is of that size too, and the 2^-47 of the double-float
+// image are 1e-18 of b -- a hundredth of an FP64 rounding of what the first
+// directions added, so the solution keeps its FP64 accuracy, at less than half
+// the time (Q2 65 x 65 x 257: 106 -> 60 us).  Both kernels are
+// queued and one of them returns at once.
+__device__ __forceinline__ bool small_residual(const CgScalars* sc) {
+  const volatile CgScalars* v = sc;
+  return v->rr <= 1e-8 * v->bb;
+}
+
+// p = z + beta p_old ; Ap = A p ; alpha = rz / (p . Ap)
+template <int K, class S>
+__global__ void __launch_bounds__(kApplyThreads)
+k_cg_apply64(MeshDev m, const double* __restrict__ bands, Coefs<double> cf,
+             const float* __restrict__ z, const double* __restrict__ p_old,
+             double* __restrict__ p_new, double* __restrict__ Ap, double* partials, CgScalars* sc,
+             int first) {
+  if (((volatile CgScalars*)sc)->done || (!first && small_residual(sc))) return;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ double red[32];
+  LoadDir64 ld{z, p_old, p_new, first ? 0.0 : sc->beta, first != 0};
+  EpiStore<double> ep{Ap};
+  const double d =
+      apply_tile<K, S, double>(m, bands, cf, ld, ep, reinterpret_cast<double*>(smraw));
+  double vals[1] = {block_sum(d, red)};
+  double out[1];
+  if (last_block_reduce(partials, 1, vals, &sc->ticket, out, red) && threadIdx.x == 0) {
+    sc->pAp = out[0];
+    sc->alpha = sc->rz / out[0];
+  }
+}
+
+template <int K, class S>
+__global__ void __launch_bounds__(kApplyThreads)
+k_cg_apply64_split(MeshDev m, const df64* __restrict__ bands, Coefs<df64> cf,
+                   const float* __restrict__ z, const double* __restrict__ p_old,
+                   double* __restrict__ p_new, double* __restrict__ Ap, double* partials,
+                   CgScalars* sc) {
+  if (((volatile CgScalars*)sc)->done || !small_residual(sc)) return;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ double red[32];
+  LoadDirSplit ld{z, p_old, p_new, df_from_double(sc->beta)};
+  EpiStoreSplit ep{Ap, p_new};
+  const df64 d = apply_tile<K, S, df64>(m, bands, cf, ld, ep, reinterpret_cast<df64*>(smraw));
+  double vals[1] = {block_sum(double_from_df_int(d), red)};
+  double out[1];
+  if (last_block_reduce(partials, 1, vals, &sc->ticket, out, red) && threadIdx.x == 0) {
+    sc->pAp = out[0];
+    sc->alpha = sc->rz / out[0];
+  }
+}
+
 // CG step 2: x += alpha p ; r -= alpha Ap ; z = D^-1 r ; beta ; convergence
 template <typename T, typename TX_>
 __global__ void __launch_bounds__(256)
@@ -797,29 +875,27 @@ k_cg_start(int64_t n, const TB* __restrict__ b, const T* __restrict__ Ax, T* __r
   }
 }
 
-// --- preconditioned by the fast diagonalisation (FDM) ---------------------
-// update without preconditioning: x += alpha p ; r -= alpha Ap ; rf = (float) r
-// for the FDM ; r . r and the convergence flag
-template <typename T, typename TX_>
+// --- preconditioned by the fast diagonalisation (FDM), FP64 ---------------
+// x += alpha p ; r -= alpha Ap ; rf = (float) r for the FDM ; r . r and the
+// convergence flag (x: the iterate the start left in the scalars)
 __global__ void __launch_bounds__(256)
-k_cg_update_fdm(int64_t n, TX_* __restrict__ xv, T* __restrict__ r, const T* __restrict__ p,
-                const T* __restrict__ Ap, float* __restrict__ rf, double* partials,
-                CgScalars* sc, int maxit) {
+k_cg_update64(int64_t n, double* __restrict__ r, const double* __restrict__ p,
+              const double* __restrict__ Ap, float* __restrict__ rf, double* partials,
+              CgScalars* sc, int maxit) {
   if (((volatile CgScalars*)sc)->done) return;
-  __shared__ double red[32];
-  T alpha = (T)sc->alpha;
-  T rr = 0;
-  TX_* const xs = xv ? xv : reinterpret_cast<TX_*>(sc->x);
+  __shared__ double red[256];
+  const double alpha = sc->alpha;
+  double* __restrict__ x = sc->x;
+  double rr = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
-    xs[i] += (TX_)(alpha * p[i]);
-    T ri = r[i] - alpha * Ap[i];
+    x[i] = fma(alpha, p[i], x[i]);
+    const double ri = fma(-alpha, Ap[i], r[i]);
     r[i] = ri;
-    if (rf) rf[i] = (float)ri;
-    rr += ri * ri;
+    rf[i] = (float)ri;  // residuals soon leave the range of the integer split
+    rr = fma(ri, ri, rr);
   }
-  double s = block_sum(rr, red);
-  double vals[1] = {s};
+  double vals[1] = {block_sum256(rr, red)};
   double out[1];
   if (last_block_reduce(partials, 1, vals, &sc->ticket, out, red) && threadIdx.x == 0) {
     sc->rr = out[0];
@@ -828,37 +904,52 @@ k_cg_update_fdm(int64_t n, TX_* __restrict__ xv, T* __restrict__ r, const T* __r
   }
 }
 
-// after z_new = P^-1 r: z_new (from the FP32 FDM output zf) ; rz_new = r . z_new ;
-// Polak-Ribiere beta = (rz_new - r . z_old) / rz_old (robust to the rounding
-// of the FP32 preconditioner) ; first: plain rz.  With fletcher_reeves the
-// plain beta = rz_new / rz_old is used: when the dots are formed from FP32
-// products, r . z_old (zero in exact arithmetic, large terms) carries an
-// error of order 1e-7 |r||z_old|, which is comparable to rz_new itself once
-// the residual has dropped by 1e-6 and would spoil the Polak-Ribiere beta
-template <typename T>
+// r . z, r . z_old and beta of the FP64 solve where the FDM has not formed
+// them (its dense form)
 __global__ void __launch_bounds__(256)
-k_cg_dot_fdm(int64_t n, const T* __restrict__ r, const float* __restrict__ zf,
-             const T* __restrict__ z_old, T* __restrict__ z_new, double* partials,
-             CgScalars* sc, int first, int ignore_done, int fletcher_reeves = 0) {
+k_cg_dot64(int64_t n, const double* __restrict__ r, const float* __restrict__ z,
+           const float* __restrict__ z_old, double* partials, CgScalars* sc, int first,
+           int ignore_done) {
   if (!ignore_done && ((volatile CgScalars*)sc)->done) return;
-  __shared__ double red[32];
-  // per-thread sums in T (a few terms each), one conversion per thread: FP64
-  // arithmetic per element would run on the slow FP64 pipe
-  T rz = 0, rzo = 0;
+  __shared__ double red[256];
+  double rz = 0.0, rzo = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
-    T zi = zf ? (T)zf[i] : z_new[i];
-    if (zf) z_new[i] = zi;
-    T ri = r[i];
-    rz += ri * zi;
-    if (!first && !fletcher_reeves) rzo += ri * z_old[i];
+    const double ri = r[i];
+    rz = fma(ri, double_from_float_int(z[i]), rz);
+    if (!first) rzo = fma(ri, double_from_float_int(z_old[i]), rzo);
   }
-  double s1 = block_sum(rz, red);
-  double s2 = block_sum(rzo, red);
-  double vals[2] = {s1, s2};
+  double vals[2] = {block_sum256(rz, red), block_sum256(rzo, red)};
   double out[2];
   if (last_block_reduce(partials, 2, vals, &sc->ticket, out, red) && threadIdx.x == 0) {
     if (!first) sc->beta = (out[0] - out[1]) / sc->rz;
+    sc->rz = out[0];
+  }
+}
+
+// after z = P^-1 r of the mixed solve, where the FDM has not formed the dot
+// product (its dense form): r . z and the Fletcher-Reeves beta = rz_new /
+// rz_old (first: plain rz).  The FP64 solve uses the Polak-Ribiere beta
+// (rz_new - r . z_old) / rz_old, robust to the rounding of the FP32
+// preconditioner; with the dots formed from FP32 products, r . z_old (zero in
+// exact arithmetic, large terms) carries an error of order 1e-7 |r||z_old|,
+// which is comparable to rz_new itself once the residual has dropped by 1e-6
+// and would spoil it
+__global__ void __launch_bounds__(256)
+k_cg_dot32(int64_t n, const float* __restrict__ r, const float* __restrict__ z, double* partials,
+           CgScalars* sc, int first, int ignore_done) {
+  if (!ignore_done && ((volatile CgScalars*)sc)->done) return;
+  __shared__ double red[32];
+  // per-thread sums in FP32 (a few terms each), one conversion per thread:
+  // FP64 arithmetic per element would run on the slow FP64 pipe
+  float rz = 0.f;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x)
+    rz = fmaf(r[i], z[i], rz);
+  double vals[1] = {block_sum(rz, red)};
+  double out[1];
+  if (last_block_reduce(partials, 1, vals, &sc->ticket, out, red) && threadIdx.x == 0) {
+    if (!first) sc->beta = out[0] / sc->rz;
     sc->rz = out[0];
   }
 }
@@ -874,28 +965,30 @@ k_flag_nonzero(int64_t n, const T* __restrict__ x, int* flag) {
   if (__syncthreads_or(nz) && threadIdx.x == 0) atomicOr(flag, 1);
 }
 
-// start: r = b - Ax ; rf = (float) r ; rr, bb, tolerance
-template <typename T, typename TB>
+// start: r = b - Ax (r = b for a zero start vector, sc->xnz == 0, whose A x
+// was skipped) ; rf = (float) r ; rr, bb, tolerance ; the iterate's address
 __global__ void __launch_bounds__(256)
-k_cg_start_fdm(int64_t n, const TB* __restrict__ b, const T* __restrict__ Ax,
-               T* __restrict__ r, float* __restrict__ rf, double* partials, CgScalars* sc,
-               double rtol, int use_flag, void* x) {
-  __shared__ double red[32];
-  T rr = 0, bb = 0;
-  // with use_flag, A x was skipped for a zero start vector (sc->xnz == 0)
-  const bool ax = !use_flag || ((volatile CgScalars*)sc)->xnz;
+k_cg_start64(int64_t n, const double* __restrict__ b, const double* __restrict__ Ax,
+             double* __restrict__ r, float* __restrict__ rf, double* partials, CgScalars* sc,
+             double rtol, double* x) {
+  __shared__ double red[256];
+  double rr = 0.0, bb = 0.0;
+  const bool ax = ((volatile CgScalars*)sc)->xnz;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
-    T bi = (T)b[i];
-    T ri = ax ? bi - Ax[i] : bi;
+    const double bi = b[i];
+    double ri = bi;
+    if (ax) {
+      ri = bi - Ax[i];
+      rr = fma(ri, ri, rr);
+    }
     r[i] = ri;
-    if (rf) rf[i] = (float)ri;
-    rr += ri * ri;
-    bb += bi * bi;
+    const df64 q = df_from_double_int(ri);
+    rf[i] = q.hi + q.lo;
+    bb = fma(bi, bi, bb);
   }
-  double s1 = block_sum(rr, red);
-  double s2 = block_sum(bb, red);
-  double vals[2] = {s1, s2};
+  const double s2 = block_sum256(bb, red);
+  double vals[2] = {ax ? block_sum256(rr, red) : s2, s2};
   double out[2];
   if (last_block_reduce(partials, 2, vals, &sc->ticket, out, red) && threadIdx.x == 0) {
     sc->rr = out[0];
@@ -905,7 +998,7 @@ k_cg_start_fdm(int64_t n, const TB* __restrict__ b, const T* __restrict__ Ax,
     sc->it = 0;
     sc->done = out[0] <= sc->tol2 ? 1 : 0;
     sc->beta = 0.0;
-    sc->x = static_cast<double*>(x);
+    sc->x = x;
   }
 }
 
@@ -1423,115 +1516,6 @@ static cudaError_t cg_solve(const MeshDev& m, const T* bands, const double* coef
   return cudaSuccess;
 }
 
-// PCG with the FDM preconditioner.  T = vector precision; the preconditioner
-// always runs in FP32 (rf: FP32 copy of r when T = double, else r itself).
-template <typename T, typename TX_, typename TB>
-static cudaError_t cg_solve_fdm(const MeshDev& m, const T* bands, const double* coef,
-                                const TB* b, TX_* x, const T* x_as_T, double rtol, int maxit,
-                                T* r, T* z, T* zn, T* p0, T* p1, T* Ap, float* rf, float* zf,
-                                FdmPlan* fdm, double* partials, CgScalars* sc,
-                                cudaStream_t s, int* iters, double* relres, Timer* tm,
-                                bool x_is_zero, cudaStream_t ls, SolvePart part = kSolveAll) {
-  if (part == kSolveFinish) return cudaSuccess;  // the loop has updated x in place
-  cudaError_t e;
-  int64_t n = m.n_nodes;
-  int vb = vec_blocks(n);
-  const int op_stage = sizeof(T) == 8 ? kStageOp64 : kStageOp32;
-  const bool conv = sizeof(T) == 8;  // FP32 copies needed for the preconditioner
-  float* rin = conv ? rf : reinterpret_cast<float*>(r);
-  if (part != kSolveLoop) {
-    if (x_is_zero) {
-      if ((e = cudaMemsetAsync(Ap, 0, sizeof(T) * n, s)) != cudaSuccess) return e;
-    } else {
-      // the operator is skipped on the device when x0 has no nonzero entry
-      k_flag_nonzero<TX_><<<vb, 256, 0, s>>>(n, x, &sc->xnz);
-      count_launches(1);
-      if (tm) tm->begin(op_stage, s);
-      if ((e = apply_t<T>(m, bands, coef, x_as_T, Ap, s, &sc->xnz)) != cudaSuccess) return e;
-      if (tm) tm->end(op_stage, s);
-    }
-    k_cg_start_fdm<T, TB><<<vb, 256, 0, s>>>(n, b, Ap, r, conv ? rf : nullptr, partials, sc, rtol,
-                                            x_is_zero ? 0 : 1, x);
-    count_launches(1);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
-  if (part == kSolveStart) return cudaSuccess;
-  if (part == kSolveLoop) x = nullptr;  // the pointer that the start left in the scalars
-  // z = P^-1 r
-  float* zout = conv ? zf : reinterpret_cast<float*>(z);
-  if ((e = fdm_apply(fdm, rin, zout, nullptr, s)) != cudaSuccess) return e;
-  k_cg_dot_fdm<T><<<vb, 256, 0, s>>>(n, r, conv ? zf : nullptr, z, z, partials, sc, 1, 1);
-  count_launches(1);
-  T* pc = p0;
-  T* pn = p1;
-  T* zc = z;   // current preconditioned residual
-  T* zo = zn;  // spare buffer
-  auto iter = [&](int first, cudaStream_t st) -> cudaError_t {
-    cudaError_t ee;
-    if (tm) tm->begin(op_stage, st);
-    if ((ee = cg_apply_t<T>(m, bands, coef, zc, pc, pn, Ap, partials, sc, first, st)) !=
-        cudaSuccess)
-      return ee;
-    if (tm) tm->end(op_stage, st);
-    k_cg_update_fdm<T, TX_><<<vb, 256, 0, st>>>(n, x, r, pn, Ap, conv ? rf : nullptr, partials,
-                                                sc, maxit);
-    count_launches(1);
-    if ((ee = cudaGetLastError()) != cudaSuccess) return ee;
-    // z_new = P^-1 r, beta (skipped on the device once converged)
-    float* zo_f = conv ? zf : reinterpret_cast<float*>(zo);
-    if ((ee = fdm_apply(fdm, rin, zo_f, &sc->done, st)) != cudaSuccess) return ee;
-    k_cg_dot_fdm<T><<<vb, 256, 0, st>>>(n, r, conv ? zf : nullptr, zc, zo, partials, sc, 0, 0);
-    count_launches(1);
-    if ((ee = cudaGetLastError()) != cudaSuccess) return ee;
-    T* t = zc;
-    zc = zo;
-    zo = t;
-    t = pc;
-    pc = pn;
-    pn = t;
-    return cudaSuccess;
-  };
-  if (ls) {  // device-driven loop inside a stream capture
-    // as many iterations ahead of the node as the solve usually takes (three
-    // to 1e-13): the body's two would be one too many
-    for (int it = 0; it < (sizeof(T) == 8 ? 3 : 2); ++it)
-      if ((e = iter(it == 0, s)) != cudaSuccess) return e;
-    cudaGraphConditionalHandle h;
-    if ((e = loop_open(s, ls, &h, sc, maxit)) != cudaSuccess) return e;
-    e = iter(0, ls);
-    if (e == cudaSuccess) e = iter(0, ls);
-    if ((e = loop_close(ls, h, sc, maxit, e)) != cudaSuccess) return e;
-    *iters = -1;
-    *relres = -1.0;
-    return cudaSuccess;
-  }
-  CgScalars hs;
-  if ((e = cudaMemcpyAsync(&hs, sc, sizeof(CgScalars), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
-    return e;
-  if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
-  // iterations are queued in chunks: every kernel of an iteration (operator,
-  // update, FDM transforms and solves, dot) returns at once on the device flag
-  // `done`, so only one host round trip per chunk is needed; with the FDM
-  // (an inverse up to rounding) the FP64 solve converges in about three
-  // iterations, so chunks of three leave few launches that return at once
-  const int chunk = sizeof(T) == 8 ? 3 : 2;
-  int launched = 0;
-  while (!hs.done && launched < maxit) {
-    int todo = maxit - launched < chunk ? maxit - launched : chunk;
-    for (int c = 0; c < todo; ++c)
-      if ((e = iter(launched + c == 0, s)) != cudaSuccess) return e;
-    launched += todo;
-    if ((e = cudaMemcpyAsync(&hs, sc, sizeof(CgScalars), cudaMemcpyDeviceToHost, s)) !=
-        cudaSuccess)
-      return e;
-    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
-  }
-  *iters = hs.it;
-  double bb = hs.bb > 0 ? hs.bb : 1.0;
-  *relres = std::sqrt(hs.rr / bb);
-  return cudaSuccess;
-}
-
 template <int K, class S>
 static cudaError_t set_smem_df() {
   static bool done = false;
@@ -1556,6 +1540,132 @@ static Coefs<df64> split_coefs(const double* c) {
   cf.cKy = sp(c[2]);
   cf.cKz = sp(c[3]);
   return cf;
+}
+
+template <int K, class S>
+static cudaError_t set_smem64() {
+  static bool done = false;
+  if (done) return cudaSuccess;
+  cudaError_t e =
+      cudaFuncSetAttribute(k_cg_apply64<K, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)apply_smem<K, S, double>());
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_cg_apply64_split<K, S>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)apply_smem<K, S, df64>());
+  if (e == cudaSuccess) done = true;
+  return e;
+}
+
+// FP64 solve: PCG with the FDM preconditioner, which runs in FP32 (rf: FP32
+// copy of r, z kept in FP32).
+template <int K, class S>
+static cudaError_t cg_solve64(const MeshDev& m, const double* bands, const double* coef,
+                              const double* b, double* x, double rtol, int maxit, CgWork& w,
+                              cudaStream_t s, int* iters, double* relres) {
+  if (w.part == kSolveFinish) return cudaSuccess;  // the loop has updated x in place
+  cudaError_t e;
+  const int64_t n = m.n_nodes;
+  const int vb = vec_blocks(n);
+  Timer* tm = w.timer;
+  CgScalars* sc = w.sc;
+  if ((e = set_smem64<K, S>()) != cudaSuccess) return e;
+  if (w.part != kSolveLoop) {
+    if ((e = cudaMemsetAsync(sc, 0, kCgReset, s)) != cudaSuccess) return e;
+    // the operator is skipped on the device when x0 has no nonzero entry
+    k_flag_nonzero<double><<<vb, 256, 0, s>>>(n, x, &sc->xnz);
+    count_launches(1);
+    if (tm) tm->begin(kStageOp64, s);
+    if ((e = apply_t<double>(m, bands, coef, x, w.Ap, s, &sc->xnz)) != cudaSuccess) return e;
+    if (tm) tm->end(kStageOp64, s);
+    k_cg_start64<<<vb, 256, 0, s>>>(n, b, w.Ap, w.r, w.r32, w.partials, sc, rtol, x);
+    count_launches(1);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  if (w.part == kSolveStart) return cudaSuccess;
+  const dim3 g = apply_grid_s<S>(m);
+  const Coefs<double> cf = make_coefs<double>(coef);
+  const Coefs<df64> cfd = split_coefs(coef);
+  float* zc = w.z32;   // current preconditioned residual
+  float* zo = w.zn32;  // spare buffer
+  double* pc = w.p0;
+  double* pn = w.p1;
+  // z = P^-1 r with r . z, r . z_old and beta (the FDM's last pass forms them
+  // where it can)
+  auto precondition = [&](float* z, const float* z_old, const int* done,
+                          cudaStream_t st) -> cudaError_t {
+    FdmDot dot;
+    dot.r64 = w.r;
+    dot.z_old = z_old;
+    dot.partials = w.partials;
+    dot.sc = sc;
+    dot.first = z_old == nullptr;
+    bool fused = false;
+    cudaError_t ee = fdm_apply(w.fdm, w.r32, z, done, st, &dot, &fused);
+    if (ee != cudaSuccess || fused) return ee;
+    k_cg_dot64<<<vb, 256, 0, st>>>(n, w.r, z, z_old, w.partials, sc, dot.first,
+                                   done ? 0 : 1);
+    count_launches(1);
+    return cudaGetLastError();
+  };
+  if ((e = precondition(zc, nullptr, nullptr, s)) != cudaSuccess) return e;
+  auto iter = [&](int first, cudaStream_t st) -> cudaError_t {
+    if (tm) tm->begin(kStageOp64, st);
+    k_cg_apply64<K, S><<<g, kApplyThreads, apply_smem<K, S, double>(), st>>>(
+        m, bands, cf, zc, pc, pn, w.Ap, w.partials, sc, first);
+    if (!first)
+      k_cg_apply64_split<K, S><<<g, kApplyThreads, apply_smem<K, S, df64>(), st>>>(
+          m, w.bands_df, cfd, zc, pc, pn, w.Ap, w.partials, sc);
+    if (tm) tm->end(kStageOp64, st);
+    k_cg_update64<<<vb, 256, 0, st>>>(n, w.r, pn, w.Ap, w.r32, w.partials, sc, maxit);
+    count_launches(first ? 2 : 3);
+    cudaError_t ee = cudaGetLastError();
+    if (ee != cudaSuccess) return ee;
+    // skipped on the device once converged
+    if ((ee = precondition(zo, zc, &sc->done, st)) != cudaSuccess) return ee;
+    std::swap(zc, zo);
+    std::swap(pc, pn);
+    return cudaSuccess;
+  };
+  if (w.loop) {  // device-driven loop inside a stream capture
+    // as many iterations ahead of the node as the solve usually takes (three
+    // to 1e-13): the body's two would be one too many
+    for (int it = 0; it < 3; ++it)
+      if ((e = iter(it == 0, s)) != cudaSuccess) return e;
+    cudaGraphConditionalHandle h;
+    if ((e = loop_open(s, w.loop, &h, sc, maxit)) != cudaSuccess) return e;
+    e = iter(0, w.loop);
+    if (e == cudaSuccess) e = iter(0, w.loop);
+    if ((e = loop_close(w.loop, h, sc, maxit, e)) != cudaSuccess) return e;
+    *iters = -1;
+    *relres = -1.0;
+    return cudaSuccess;
+  }
+  CgScalars hs;
+  if ((e = cudaMemcpyAsync(&hs, sc, sizeof(CgScalars), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
+    return e;
+  if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
+  // iterations are queued in chunks: every kernel of an iteration (operator,
+  // update, FDM transforms and solves) returns at once on the device flag
+  // `done`, so only one host round trip per chunk is needed; with the FDM
+  // (an inverse up to rounding) the solve converges in about three
+  // iterations, so chunks of three leave few launches that return at once
+  const int chunk = 3;
+  int launched = 0;
+  while (!hs.done && launched < maxit) {
+    int todo = maxit - launched < chunk ? maxit - launched : chunk;
+    for (int c = 0; c < todo; ++c)
+      if ((e = iter(launched + c == 0, s)) != cudaSuccess) return e;
+    launched += todo;
+    if ((e = cudaMemcpyAsync(&hs, sc, sizeof(CgScalars), cudaMemcpyDeviceToHost, s)) !=
+        cudaSuccess)
+      return e;
+    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
+  }
+  *iters = hs.it;
+  double bb = hs.bb > 0 ? hs.bb : 1.0;
+  *relres = std::sqrt(hs.rr / bb);
+  return cudaSuccess;
 }
 
 // Mixed solve: conjugate gradients whose iterate, residual and operator are
@@ -1594,11 +1704,15 @@ static cudaError_t cg_solve_df(const MeshDev& m, const df64* bands, const double
   df64* pc = w.p0_df;
   df64* pn = w.p1_df;
   // z = P^-1 r and r . z (the FDM's last pass forms the dot product where it can)
-  const FdmDot dot0{w.r32, w.partials, w.sc, 1};
+  FdmDot dot0;
+  dot0.r = w.r32;
+  dot0.partials = w.partials;
+  dot0.sc = w.sc;
+  dot0.first = 1;
   bool fused = false;
   if ((e = fdm_apply(w.fdm, w.r32, zc, nullptr, s, &dot0, &fused)) != cudaSuccess) return e;
   if (!fused) {
-    k_cg_dot_fdm<float><<<vb, 256, 0, s>>>(n, w.r32, nullptr, zc, zc, w.partials, w.sc, 1, 1);
+    k_cg_dot32<<<vb, 256, 0, s>>>(n, w.r32, zc, w.partials, w.sc, 1, 1);
     count_launches(1);
   }
   auto iter = [&](int first, cudaStream_t st) -> cudaError_t {
@@ -1611,12 +1725,12 @@ static cudaError_t cg_solve_df(const MeshDev& m, const df64* bands, const double
                                       maxit);
     count_launches(2);
     if ((ee = cudaGetLastError()) != cudaSuccess) return ee;
-    const FdmDot dot{w.r32, w.partials, w.sc, 0};
+    FdmDot dot = dot0;
+    dot.first = 0;
     bool fz = false;
     if ((ee = fdm_apply(w.fdm, w.r32, zo, &w.sc->done, st, &dot, &fz)) != cudaSuccess) return ee;
-    if (!fz) {  // Fletcher-Reeves beta (see k_cg_dot_fdm)
-      k_cg_dot_fdm<float><<<vb, 256, 0, st>>>(n, w.r32, nullptr, zc, zo, w.partials, w.sc, 0, 0,
-                                             1);
+    if (!fz) {
+      k_cg_dot32<<<vb, 256, 0, st>>>(n, w.r32, zo, w.partials, w.sc, 0, 0);
       count_launches(1);
     }
     if ((ee = cudaGetLastError()) != cudaSuccess) return ee;
@@ -1674,17 +1788,19 @@ cudaError_t run_cg64(const MeshDev& m, const double* bands, const double* coef,
                      const double* b, double* x, double rtol, int maxit, CgWork& w,
                      cudaStream_t s, int* iters_host, double* relres_host, int* converged) {
   cudaError_t e;
-  if (w.part == kSolveAll || w.part == kSolveStart)
-    if ((e = cudaMemsetAsync(w.sc, 0, kCgReset, s)) != cudaSuccess) return e;
   if (w.fdm) {
-    e = cg_solve_fdm<double, double, double>(m, bands, coef, b, x, x, rtol, maxit, w.r, w.z,
-                                             w.zn, w.p0, w.p1, w.Ap, w.r32, w.z32, w.fdm,
-                                             w.partials, w.sc, s, iters_host, relres_host,
-                                             w.timer, false, w.loop, w.part);
+    e = with_k(m, [&](auto kc) {
+      constexpr int K = decltype(kc)::value;
+      return with_shape<K>(m, [&](auto sh) {
+        return cg_solve64<K, decltype(sh)>(m, bands, coef, b, x, rtol, maxit, w, s, iters_host,
+                                           relres_host);
+      });
+    });
     if (e != cudaSuccess) return e;
     *converged = *relres_host <= rtol;
     return cudaSuccess;
   }
+  if ((e = cudaMemsetAsync(w.sc, 0, kCgReset, s)) != cudaSuccess) return e;
   if ((e = make_dinv<double>(m, bands, coef, w.dinv, s)) != cudaSuccess) return e;
   e = cg_solve<double, double, double>(m, bands, coef, b, x, x, rtol, maxit, w.r, w.z, w.p0,
                                        w.p1, w.Ap, w.dinv, w.partials, w.sc, s, iters_host,
@@ -1701,7 +1817,7 @@ cudaError_t run_cg_mixed(const MeshDev& m, const double* bands64, const float* b
   cudaError_t e;
   int64_t n = m.n_nodes;
   int vb = vec_blocks(n);
-  if (w.fdm && w.bands_df) {
+  if (w.fdm) {
     int it = 0;
     double rel = 0.0;
     e = with_k(m, [&](auto kc) {
@@ -1721,7 +1837,7 @@ cudaError_t run_cg_mixed(const MeshDev& m, const double* bands64, const float* b
   // the refinement loop below decides on the host: it cannot run inside a
   // stream capture (the graph form of the mixed solve needs the FDM path)
   if (w.loop) return cudaErrorNotSupported;
-  if (!w.fdm && (e = make_dinv<float>(m, bands64, coef, w.dinv32, s)) != cudaSuccess) return e;
+  if ((e = make_dinv<float>(m, bands64, coef, w.dinv32, s)) != cudaSuccess) return e;
   int total_it = 0, outer = 0;
   double relres = 1.0;
   const int max_outer = 8;
@@ -1750,16 +1866,9 @@ cudaError_t run_cg_mixed(const MeshDev& m, const double* bands64, const float* b
     if ((e = cudaMemsetAsync(w.sc, 0, kCgReset, s)) != cudaSuccess) return e;
     int it = 0;
     double rr = 0;
-    if (w.fdm)
-      e = cg_solve_fdm<float, float, float>(m, bands32, coef, w.rin32, w.d32, w.d32, inner_rtol,
-                                            maxit - total_it, w.r32, w.z32, w.zn32, w.q0, w.q1,
-                                            w.Aq, nullptr, nullptr, w.fdm, w.partials, w.sc, s,
-                                            &it, &rr, w.timer, true, nullptr);
-    else
-      e = cg_solve<float, float, float>(m, bands32, coef, w.rin32, w.d32, w.d32, inner_rtol,
-                                        maxit - total_it, w.r32, w.z32, w.q0, w.q1, w.Aq,
-                                        w.dinv32, w.partials, w.sc, s, &it, &rr, w.timer,
-                                        nullptr);
+    e = cg_solve<float, float, float>(m, bands32, coef, w.rin32, w.d32, w.d32, inner_rtol,
+                                      maxit - total_it, w.r32, w.z32, w.q0, w.q1, w.Aq,
+                                      w.dinv32, w.partials, w.sc, s, &it, &rr, w.timer, nullptr);
     if (e != cudaSuccess) return e;
     total_it += it;
     k_add_scaled<<<vb, 256, 0, s>>>(n, x, w.d32, rn);
