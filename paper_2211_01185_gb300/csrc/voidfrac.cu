@@ -13,12 +13,11 @@
 // walks the rows of bins that can hold a neighbour of the element, culls the
 // particles against the box of the element's Gauss points, and stages the
 // survivors in shared memory.  FP64 path (k_qcm): it then tests
-// (quadrature point, candidate) pairs with one candidate per lane, appends
-// the hits to a per-warp queue and evaluates the double-float lens volumes
-// only on full warps of hits; a segmented warp scan adds up each point's
-// share and the last lane of a segment updates that point's sum in shared
-// memory, so every sum is accumulated in a fixed order.  Mixed path
-// (k_qcm_pts): one Gauss point per lane (see there).
+// (quadrature point, candidate) pairs with one candidate per lane, queues the
+// hits point by point, evaluates their double-float lens volumes one per
+// lane, and a few lanes per point add up its stretch of them, so every sum is
+// accumulated in a fixed order.  Mixed path (k_qcm_pts): one Gauss point per
+// lane (see there).
 //
 // Neighbour predicate.  The FP64 path must reproduce the FP64 definition
 // exactly (bit-exact neighbour sets).  It first evaluates the distance in
@@ -27,6 +26,7 @@
 // (delta is chosen on the host above a proven bound on the FP32 error), and
 // only pairs inside the band are re-tested in FP64 with the exact
 // left-to-right expression.  The mixed path decides every pair in FP32.
+#include <cmath>
 #include <cstdint>
 
 #include "internal.h"
@@ -37,12 +37,43 @@ namespace cfdem {
 
 constexpr int kQcmWarps = 4;      // warps (elements) per block
 
+// n / d for 0 <= n < 2^31 by one wide multiplication (Granlund and Montgomery
+// 1994): an integer division converts both ways on the narrow FP64 pipe
+struct FastDiv {
+  unsigned mul;
+  int shift;
+  void set(int d) {
+    int l = 0;
+    while ((1ll << l) < d) ++l;
+    shift = 31 + l;
+    mul = (unsigned)((1ull << shift) / (unsigned)d + 1);
+  }
+  __device__ __forceinline__ int div(int n) const {
+    return (int)(((unsigned long long)(unsigned)n * mul) >> shift);
+  }
+};
+
+// row r of a block of rows nrx wide -> (r % nrx, r / nrx); inv ~ 1 / nrx.  In
+// FP32: r / nrx differs from the next integer by at least 1 / (2 nrx) once
+// 1/2 is added to r, above the error of the product for r < 2^20
+__device__ __forceinline__ void row_split(int r, int nrx, float inv, int* x, int* z) {
+  if (r < (1 << 20)) {
+    const float f = __int_as_float(0x4B000000 + r) - 8388608.0f;
+    floor_small((f + 0.5f) * inv, z);
+  } else {
+    *z = r / nrx;
+  }
+  *x = r - *z * nrx;
+}
+
 struct QcmParams {
   double R;            // averaging radius
   float R32;
   float inv_vr32;      // 1 / (4/3 pi R^3)
-  double inv_vr;
+  double inv_vr12;     // (pi / 12) / V_R = 1 / (16 R^3)
   float delta;         // relative band of the FP32 predicate
+  float delta_df;      // and of the double-float one (FP64 path)
+  FastDiv by_exy, by_ex;  // e / (ne_x ne_y), its remainder / ne_x
   float hx, hy, hz;    // element size (FP32)
   float hx_hi, hx_lo, hy_hi, hy_lo, hz_hi, hz_lo;  // float-float element size
   float inv_be[3];     // 1 / bin edge
@@ -91,27 +122,39 @@ __device__ __forceinline__ void neumaier(float& s, float& c, float v) {
   s = t;
 }
 
+// FP64 kernel: a group of up to 32 candidates against the element's Gauss
+// points, kPts points a pass, the hits of a pass stored q by q
+template <int K>
+struct QcmGeom {
+  static constexpr int NQ = K + 1;
+  static constexpr int kWarps = K == 3 ? 2 : 4;          // warps (elements) per block
+  static constexpr int kMinBlocks = K == 3 ? 9 : 6;      // resident blocks per SM
+  static constexpr int kLayers = K == 1 ? 2 : 1;         // layers of Gauss points per pass
+  static constexpr int kPts = kLayers * NQ * NQ;         // 8, 9, 16
+  static constexpr int kPasses = NQ / kLayers;           // 1, 3, 4
+  static constexpr int kLanes = 32 / kPts;               // lanes that sum one point's hits
+};
+
 template <int K>
 struct QcmSmem {
-  static constexpr int Q = (K + 1) * (K + 1) * (K + 1);
-  float4 qrel[Q];                          // Gauss point minus element centre
-  float4 buf[kQcmWarps][64];               // culled candidates not yet tested
-  int32_t bslot[kQcmWarps][64];            // their sorted slots
-  int32_t gslot[kQcmWarps][32];            // the group under test (one per lane)
-  // hits (lane of the group << 6) | q, q-sorted: room for the hits of one
-  // layer of Gauss points ((K+1)^2 points x 32 lanes) on top of < 32 pending
-  static constexpr int QCAP = 32 * (K + 1) * (K + 1) + 32;
-  int32_t queue[kQcmWarps][QCAP];
-  df64 accdf[kQcmWarps][Q];                // double-float sums
-  int32_t cnt[kQcmWarps][Q];
-  long long ids[kQcmWarps][Q];
-  double xq[kQcmWarps][Q][3];              // FP64 Gauss points
-  P4 g64[kQcmWarps][32];                   // FP64 positions of the group
-  // the group's positions relative to the mesh origin and radii as
-  // double-float (hi and lo parts), and the Gauss points of the element per
-  // axis (x0-relative, hi and lo)
-  float4 ghi[kQcmWarps][32], glo[kQcmWarps][32];
-  float xqf[kQcmWarps][3][4][2];
+  using G = QcmGeom<K>;
+  float4 buf[G::kWarps][64];               // culled candidates not yet tested
+  int32_t bslot[G::kWarps][64];            // their sorted slots
+  // of the group under test: (x - x_q)^2 per axis and 1D Gauss point, the sum
+  // and the squared difference of the radii, the smaller sphere's volume, all
+  // double-float
+  float2 sq[G::kWarps][3 * G::NQ][32];
+  float4 rad[G::kWarps][32];
+  float2 full[G::kWarps][32];
+  // hits of a pass, (candidate << 6) | point, and their lens volumes
+  uint16_t queue[G::kWarps][32 * G::kPts];
+  float2 vol[G::kWarps][32 * G::kPts];
+  int32_t off[G::kWarps][G::kPts + 1];     // first hit of each point of the pass
+  float2 acc[G::kWarps][G::kPasses][32];   // double-float sums, one per (point, lane)
+  double R, x0[3], h[3], g[4];             // radius, mesh origin, element size, 1D points
+  int32_t el[G::kWarps][3];                // the element
+  float xqf[G::kWarps][3][4][2];           // its Gauss points relative to x0 (hi and lo)
+  float gz[4];                             // 1D Gauss points in z minus the element centre
 };
 
 // lens volume of the FP64 path in double-float arithmetic (relative error
@@ -132,88 +175,121 @@ __device__ __forceinline__ df64 lens_df(df64 R, df64 r, df64 D, df64 c43, df64 c
   return c12 * sdist * sdist * num * df_recip(d);
 }
 
+__device__ __forceinline__ df64 df_sq(df64 a) {
+  const float p = a.hi * a.hi;
+  const float e = fmaf(a.hi, a.hi, -p);
+  return df_renorm(p, fmaf(a.hi + a.hi, a.lo, e));
+}
+// (s, e) += v, e the sum of the rounding errors and low parts
+__device__ __forceinline__ void df_gather(float& s, float& e, float v) {
+  const float t = s + v, bb = t - s;
+  e += (s - (t - bb)) + (v - bb);
+  s = t;
+}
+
+// lens volume of one hit in units of pi / 12 (the full smaller sphere is 16
+// min(R, r)^3 of them): D the squared distance, rad the pair's (R + r) and
+// (R - r)^2, full the smaller sphere's volume.  One reciprocal square root
+// gives both d and, after a Newton step in FP32 and one in double-float, 1/d.
+__device__ __forceinline__ df64 lens_hit(df64 D, float4 rad, float2 full) {
+  if (df_le(D, df64(rad.z, rad.w))) return df64(full.x, full.y);
+  const float y = rsqrtf(D.hi);
+  const float x0 = D.hi * y;
+  const float sq = x0 * x0;
+  const float r0 = (D.hi - sq) + (D.lo - fmaf(x0, x0, -sq));  // D - x0^2
+  const df64 d = df_renorm(x0, r0 * (0.5f * y));
+  const df64 S(rad.x, rad.y);
+  const df64 sd = S - d;
+  // D + 2 d S - 3 (R - r)^2, the three high parts and all errors apart
+  const df64 dS = d * S;
+  const float p3 = 3.0f * rad.z;
+  float hi = D.hi, lo = D.lo + 2.0f * dS.lo;
+  lo -= fmaf(3.0f, rad.w, fmaf(3.0f, rad.z, -p3));
+  df_gather(hi, lo, 2.0f * dS.hi);
+  df_gather(hi, lo, -p3);
+  const df64 num = df_renorm(hi, lo);
+  const float y1 = fmaf(y, fmaf(-d.hi, y, 1.0f), y);
+  const float pe = d.hi * y1;
+  const float re = (1.0f - pe) - fmaf(d.lo, y1, fmaf(d.hi, y1, -pe));
+  return df_sq(sd) * (num * df_renorm(y1, y1 * re));
+}
+
 struct QcmWarp {
   int warp, lane;
   unsigned lt_mask;
-  double R;
   float R32, band;
   float R_hi, R_lo;
-  df64 c43, c12;
-  bool want_counts, want_ids;
   const float2* cw;  // per sorted particle scale of its lens volumes, or null
 };
 
-// Evaluate the first cnt queued hits (q-sorted) and add each quadrature
-// point's share with one segmented warp scan; the last lane of a segment
-// updates that point's sum, so every sum is accumulated in a fixed order.
+// Neighbour test of a pair inside the FP32 band: by the tabulated
+// double-float squares when those decide it (delta_df, from the host, is
+// above their error and the definition's own rounding), else by the FP64
+// definition.  Real calls: inlined, the compiler predicates the FP64
+// instructions into every test and they issue on the narrow pipe even when
+// not taken (three times the kernel's time); and the FP64 Gauss points are
+// formed only here, since at 16 cycles of an SM per FP64 instruction those
+// of every element took a quarter of the kernel.
 template <int K>
-__device__ __forceinline__ void qcm_flush(QcmSmem<K>& sm, const QcmWarp& w, int base, int cnt,
-                                          const int32_t* __restrict__ perm) {
-  const unsigned FULL = 0xffffffffu;
-  const int lane = w.lane, wp = w.warp;
-  int q = -1 - lane;  // distinct sentinels for idle lanes
-  df64 vdf(0.f, 0.f);
-  long long id = 0;
-  int one = 0;
-  if (lane < cnt) {
-    int pk = sm.queue[wp][base + lane];
-    q = pk & 63;
-    int j = pk >> 6;
-    one = 1;
-    constexpr int NQ = K + 1;
-    const int qx = q % NQ, qy = (q / NQ) % NQ, qz = q / (NQ * NQ);
-    float4 H = sm.ghi[wp][j], L = sm.glo[wp][j];
-    df64 dx = df64(H.x, L.x) - df64(sm.xqf[wp][0][qx][0], sm.xqf[wp][0][qx][1]);
-    df64 dy = df64(H.y, L.y) - df64(sm.xqf[wp][1][qy][0], sm.xqf[wp][1][qy][1]);
-    df64 dz = df64(H.z, L.z) - df64(sm.xqf[wp][2][qz][0], sm.xqf[wp][2][qz][1]);
-    df64 D = dx * dx + dy * dy + dz * dz;
-    vdf = lens_df(df64(w.R_hi, w.R_lo), df64(H.w, L.w), D, w.c43, w.c12);
-    if (w.cw) {  // volume-conserving QCM: the particle's lens volumes scaled by c
-      const float2 c = __ldg(w.cw + sm.gslot[wp][j]);
-      vdf = vdf * df64(c.x, c.y);
-    }
-    if (w.want_ids) id = perm[sm.gslot[wp][j]];
-  }
-  if (w.want_counts) {
+__device__ __noinline__ bool in_reach64(const QcmSmem<K>& sm, int wp, const double* xs64, int slot,
+                                        int q) {
+  const P4 pj = reinterpret_cast<const P4*>(xs64)[slot];
+  const double xp[3] = {pj.x, pj.y, pj.z};
+  double d[3];
 #pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      int qu = __shfl_up_sync(FULL, q, off);
-      int nu = __shfl_up_sync(FULL, one, off);
-      df64 vu(__shfl_up_sync(FULL, vdf.hi, off), __shfl_up_sync(FULL, vdf.lo, off));
-      long long iu = w.want_ids ? __shfl_up_sync(FULL, id, off) : 0;
-      if (lane >= off && qu == q) {
-        one += nu;
-        vdf = vdf + vu;
-        id += iu;
-      }
-    }
-  } else {
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      int qu = __shfl_up_sync(FULL, q, off);
-      df64 vu(__shfl_up_sync(FULL, vdf.hi, off), __shfl_up_sync(FULL, vdf.lo, off));
-      if (lane >= off && qu == q) vdf = vdf + vu;
-    }
+  for (int ax = 0; ax < 3; ++ax) {
+    // the Gauss point's coordinate, rounded exactly as the definition
+    const double g = sm.g[(q >> (2 * ax)) & 3];
+    const double xq = __dadd_rn(
+        sm.x0[ax], __dmul_rn(sm.h[ax], __dadd_rn((double)sm.el[wp][ax], g)));
+    d[ax] = __dsub_rn(xp[ax], xq);
   }
-  int qn = __shfl_down_sync(FULL, q, 1);
-  bool last = lane < cnt && (lane == cnt - 1 || qn != q);
-  if (last) {
-    sm.accdf[wp][q] += vdf;
-    if (w.want_counts) {
-      sm.cnt[wp][q] += one;
-      sm.ids[wp][q] += id;
-    }
-  }
-  __syncwarp();
+  const double d2 = __dadd_rn(__dadd_rn(__dmul_rn(d[0], d[0]), __dmul_rn(d[1], d[1])),
+                              __dmul_rn(d[2], d[2]));
+  const double c = __dadd_rn(sm.R, pj.w);
+  return d2 < __dmul_rn(c, c);
+}
+template <int K>
+__device__ __forceinline__ df64 pair_d2(const QcmSmem<K>& sm, int wp, int j, int q) {
+  const float2 X = sm.sq[wp][q & 3][j], Y = sm.sq[wp][K + 1 + ((q >> 2) & 3)][j],
+               Z = sm.sq[wp][2 * (K + 1) + ((q >> 4) & 3)][j];
+  float hi = X.x, lo = X.y + (Y.y + Z.y);
+  df_gather(hi, lo, Y.x);
+  df_gather(hi, lo, Z.x);
+  return df_renorm(hi, lo);
+}
+template <int K>
+__device__ __noinline__ bool in_band(const QcmSmem<K>& sm, int wp, int j, float delta,
+                                     const double* xs64, int slot, int q) {
+  const float4 rad = sm.rad[wp][j];
+  const df64 c2 = df_sq(df64(rad.x, rad.y));
+  const float t = (pair_d2<K>(sm, wp, j, q) - c2).hi;
+  if (fabsf(t) > delta * c2.hi) return t < 0.f;
+  return in_reach64<K>(sm, wp, xs64, slot, q);
 }
 
-// test the cnt (<= 32) buffered candidates against every quadrature point
+// Test the cnt (<= 32) buffered candidates against every Gauss point, one
+// candidate per lane, and add up the hits' lens volumes.  A pass over kPts
+// points queues its hits point by point, evaluates them one per lane, and
+// then kLanes lanes per point add up its stretch of the volumes, each its
+// own share in a fixed order.  Bound by FP32 and integer issue (75 % of the
+// slots, the FP64 pipe 5 %): a hit costs about 130 instructions for its
+// volume -- what depends on the candidate alone, or on one axis, is tabulated
+// once per group -- and 30 for its sum.  100,000 spheres, Q2 32x32x128: 354 us
+// with everything formed per hit and a segmented warp scan of double-floats
+// per 32 hits, 300 us with the tables and the lane sums, 242 us with the FP64
+// and conversion instructions out of the per-element code; Q3 (23,000
+// spheres) 97 -> 64 us, Q1 (9,000) 17 -> 11 us.
 template <int K>
 __device__ __forceinline__ void qcm_group(QcmSmem<K>& sm, const QcmWarp& w,
                                           const QcmParams& P, int cnt,
                                           const double* __restrict__ xs64,
                                           const float* __restrict__ xs32,
-                                          const int32_t* __restrict__ perm) {
+                                          const int32_t* __restrict__ perm,
+                                          int32_t* __restrict__ nb_count,
+                                          int64_t* __restrict__ nb_idsum) {
+  using G = QcmGeom<K>;
+  constexpr int NQ = G::NQ;
   const unsigned FULL = 0xffffffffu;
   const int lane = w.lane, wp = w.warp;
   const bool valid = lane < cnt;
@@ -222,11 +298,22 @@ __device__ __forceinline__ void qcm_group(QcmSmem<K>& sm, const QcmWarp& w,
   if (valid) {
     my = sm.buf[wp][lane];
     myslot = sm.bslot[wp][lane];
-    sm.gslot[wp][lane] = myslot;
-    sm.g64[wp][lane] = reinterpret_cast<const P4*>(xs64)[myslot];
     const float4* ff = reinterpret_cast<const float4*>(xs32) + 2 * (int64_t)myslot;
-    sm.ghi[wp][lane] = ff[0];
-    sm.glo[wp][lane] = ff[1];
+    const float4 H = ff[0], L = ff[1];
+    const df64 pos[3] = {df64(H.x, L.x), df64(H.y, L.y), df64(H.z, L.z)};
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax)
+#pragma unroll
+      for (int a = 0; a < NQ; ++a) {
+        const df64 t = df_sq(pos[ax] - df64(sm.xqf[wp][ax][a][0], sm.xqf[wp][ax][a][1]));
+        sm.sq[wp][ax * NQ + a][lane] = make_float2(t.hi, t.lo);
+      }
+    const df64 R(w.R_hi, w.R_lo), r(H.w, L.w);
+    const df64 S = R + r, dm2 = df_sq(R - r);
+    const df64 mn = df_le(R, r) ? R : r;
+    const df64 V = df_sq(mn) * mn;
+    sm.rad[wp][lane] = make_float4(S.hi, S.lo, dm2.hi, dm2.lo);
+    sm.full[wp][lane] = make_float2(16.0f * V.hi, 16.0f * V.lo);
   }
   __syncwarp();
   const float c = w.R32 + my.w;
@@ -234,75 +321,85 @@ __device__ __forceinline__ void qcm_group(QcmSmem<K>& sm, const QcmWarp& w,
   const float c2_in = c2 / w.band, c2_out = c2 * w.band;
   // squared distance to Gauss point (a, b, c) = sx[a] + (sy[b] + sz[c]):
   // per-axis squares once per candidate, two additions per point
-  float sx[K + 1], sy[K + 1];
+  float sx[NQ], sy[NQ];
 #pragma unroll
-  for (int a = 0; a <= K; ++a) {
+  for (int a = 0; a < NQ; ++a) {
     float dx = my.x - P.g1[0][a];
     float dy = my.y - P.g1[1][a];
     sx[a] = dx * dx;
     sy[a] = dy * dy;
   }
-  int qn = 0;
-  // layers cz = 0..K of Gauss points, then one more pass that only drains
-  for (int cz = 0; cz <= K + 1; ++cz) {
-    if (cz <= K) {
-      // the z offset of Gauss layer cz, from shared memory (a runtime index into
-      // the kernel parameters would move them to local memory)
-      float dz = my.z - sm.qrel[cz * (K + 1) * (K + 1)].z;
+#pragma unroll 1
+  for (int ps = 0; ps < G::kPasses; ++ps) {
+    int qn = 0;
+#pragma unroll
+    for (int l = 0; l < G::kLayers; ++l) {
+      const int cz = ps * G::kLayers + l;
+      // the layer's z offset, from shared memory (a runtime index into the
+      // kernel parameters would move them to local memory)
+      float dz = my.z - sm.gz[cz];
       float sz = dz * dz;
 #pragma unroll
-      for (int b = 0; b <= K; ++b) {
+      for (int b = 0; b < NQ; ++b) {
         float syz = sy[b] + sz;
 #pragma unroll
-        for (int a = 0; a <= K; ++a) {
-          const int q = a + (K + 1) * (b + (K + 1) * cz);
+        for (int a = 0; a < NQ; ++a) {
           float d2 = sx[a] + syz;
           bool hit = valid && d2 < c2_in;
           if (valid && d2 >= c2_in && d2 <= c2_out) {  // inside the band: exact FP64 predicate
-            P4 pj = sm.g64[wp][lane];
-            double ddx = __dsub_rn(pj.x, sm.xq[wp][q][0]);
-            double ddy = __dsub_rn(pj.y, sm.xq[wp][q][1]);
-            double ddz = __dsub_rn(pj.z, sm.xq[wp][q][2]);
-            double dd2 = __dadd_rn(__dadd_rn(__dmul_rn(ddx, ddx), __dmul_rn(ddy, ddy)),
-                                   __dmul_rn(ddz, ddz));
-            double cc = __dadd_rn(w.R, pj.w);
-            hit = dd2 < __dmul_rn(cc, cc);
+            hit = in_band<K>(sm, wp, lane, P.delta_df, xs64, myslot, a | (b << 2) | (cz << 4));
           }
           unsigned mask = __ballot_sync(FULL, hit);
-          if (hit) sm.queue[wp][qn + __popc(mask & w.lt_mask)] = (lane << 6) | q;
+          if (hit)
+            sm.queue[wp][qn + __popc(mask & w.lt_mask)] =
+                (uint16_t)((lane << 6) | (cz << 4) | (b << 2) | a);
+          if (lane == 0) sm.off[wp][a + NQ * (b + NQ * l)] = qn;
           qn += __popc(mask);
         }
       }
     }
-    // evaluate the full batches of 32 hits queued so far (after the last
-    // layer: all of them) -- the only call of the flush -- and keep the rest
-    // at the front of the queue
-    const bool last = cz == K + 1;
-    if (qn >= 32 || (last && qn > 0)) {
-      __syncwarp();
-      int base = 0;
-      while (qn - base >= 32 || (last && qn > base)) {
-        const int c = qn - base < 32 ? qn - base : 32;
-        qcm_flush<K>(sm, w, base, c, perm);
-        base += c;
+    if (lane == 0) sm.off[wp][G::kPts] = qn;
+    __syncwarp();
+    for (int i = lane; i < qn; i += 32) {
+      const int pk = sm.queue[wp][i], j = pk >> 6;
+      df64 v = lens_hit(pair_d2<K>(sm, wp, j, pk & 63), sm.rad[wp][j], sm.full[wp][j]);
+      if (w.cw) {  // volume-conserving QCM: the particle's lens volumes scaled by c
+        const float2 cj = __ldg(w.cw + sm.bslot[wp][j]);
+        v = v * df64(cj.x, cj.y);
       }
-      int rest = qn - base;
-      int tmp = lane < rest ? sm.queue[wp][base + lane] : 0;
-      __syncwarp();
-      if (lane < rest) sm.queue[wp][lane] = tmp;
-      qn = rest;
+      sm.vol[wp][i] = make_float2(v.hi, v.lo);
     }
+    __syncwarp();
+    if (lane < G::kPts * G::kLanes) {
+      const int q = lane / G::kLanes;
+      const int i0 = sm.off[wp][q] + lane % G::kLanes, i1 = sm.off[wp][q + 1];
+      float s = 0.f, e = 0.f;
+      for (int i = i0; i < i1; i += G::kLanes) {
+        const float2 v = sm.vol[wp][i];
+        e += v.y;
+        df_gather(s, e, v.x);
+      }
+      const float2 o = sm.acc[wp][ps][lane];
+      const df64 t = df64(o.x, o.y) + df_renorm(s, e);
+      sm.acc[wp][ps][lane] = make_float2(t.hi, t.lo);
+      if (nb_count && lane % G::kLanes == 0)
+        nb_count[ps * G::kPts + q] += i1 - i0;
+      if (nb_idsum && lane % G::kLanes == 0)
+        for (int i = i0; i < i1; ++i)
+          nb_idsum[ps * G::kPts + q] += perm[sm.bslot[wp][sm.queue[wp][i] >> 6]];
+    }
+    __syncwarp();
   }
-  __syncwarp();
 }
 
 template <int K>
-__global__ void __launch_bounds__(kQcmWarps * 32, 6)
+__global__ void __launch_bounds__(QcmGeom<K>::kWarps * 32, QcmGeom<K>::kMinBlocks)
 k_qcm(MeshDev m, QcmParams P, BinDev b, const int32_t* __restrict__ bin_start,
       const int32_t* __restrict__ perm, const double* __restrict__ xs64,
       const float* __restrict__ xs32, const DevStatus* __restrict__ st,
       double* __restrict__ eps64, int32_t* __restrict__ nb_count,
       int64_t* __restrict__ nb_idsum) {
+  using G = QcmGeom<K>;
   constexpr int NQ = K + 1;
   constexpr int Q = NQ * NQ * NQ;
   __shared__ QcmSmem<K> sm;
@@ -311,79 +408,87 @@ k_qcm(MeshDev m, QcmParams P, BinDev b, const int32_t* __restrict__ bin_start,
   w.warp = threadIdx.x >> 5;
   w.lane = threadIdx.x & 31;
   w.lt_mask = (1u << w.lane) - 1u;
-  w.R = P.R;
   w.R32 = P.R32;
   w.band = 1.0f + P.delta;
   w.R_hi = P.R_hi;
   w.R_lo = P.R_lo;
-  w.c43 = df64(P.c43_hi, P.c43_lo);
-  w.c12 = df64(P.c12_hi, P.c12_lo);
-  w.want_ids = nb_idsum != nullptr;
-  w.want_counts = nb_count != nullptr || nb_idsum != nullptr;
   w.cw = P.cw;
   const int lane = w.lane, wp = w.warp;
-  for (int t = threadIdx.x; t < Q; t += blockDim.x)
-    sm.qrel[t] = make_float4(P.qrel[t][0], P.qrel[t][1], P.qrel[t][2], 0.f);
+  if (threadIdx.x == 0) {
+    sm.R = P.R;
+#pragma unroll
+    for (int a = 0; a < NQ; ++a) {
+      sm.gz[a] = P.g1[2][a];
+      sm.g[a] = P.g[a];
+    }
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) {
+      sm.x0[ax] = m.x0[ax];
+      sm.h[ax] = m.h[ax];
+    }
+  }
   __syncthreads();
-  const int64_t e = blockIdx.x * (int64_t)kQcmWarps + wp;
+  const int64_t e = blockIdx.x * (int64_t)G::kWarps + wp;
   if (e >= m.E) return;  // whole warp leaves together
   // element indices by 32-bit division (E < 2^31; a 64-bit division costs
   // several times as many instructions)
   const int e32 = (int)e, exy = m.ne[0] * m.ne[1];
-  const int ez = e32 / exy;
+  const int ez = P.by_exy.div(e32);
   const int rxy = e32 - ez * exy;
-  const int ey = rxy / m.ne[0];
+  const int ey = P.by_ex.div(rxy);
   const int ex = rxy - ey * m.ne[0];
 
+  const int64_t o = e * Q;
+  if (nb_count) nb_count += o;
+  if (nb_idsum) nb_idsum += o;
   for (int q = lane; q < Q; q += 32) {
-    sm.cnt[wp][q] = 0;
-    sm.ids[wp][q] = 0;
-    sm.accdf[wp][q] = df64(0.f, 0.f);
-    int qx = q % NQ, qy = (q / NQ) % NQ, qz = q / (NQ * NQ);
-    // FP64 Gauss point coordinates, rounded exactly as the definition
-    sm.xq[wp][q][0] = __dadd_rn(m.x0[0], __dmul_rn(m.h[0], __dadd_rn((double)ex, P.g[qx])));
-    sm.xq[wp][q][1] = __dadd_rn(m.x0[1], __dmul_rn(m.h[1], __dadd_rn((double)ey, P.g[qy])));
-    sm.xq[wp][q][2] = __dadd_rn(m.x0[2], __dmul_rn(m.h[2], __dadd_rn((double)ez, P.g[qz])));
+    if (nb_count) nb_count[q] = 0;
+    if (nb_idsum) nb_idsum[q] = 0;
   }
-  if (lane == 0) {
+#pragma unroll
+  for (int ps = 0; ps < G::kPasses; ++ps) sm.acc[wp][ps][lane] = make_float2(0.f, 0.f);
+  // small integers made floats by the 2^23 trick, here and below: conversion
+  // instructions issue on the narrow FP64 pipe
+  const float fex = __int_as_float(0x4B000000 + ex) - 8388608.0f;
+  const float fey = __int_as_float(0x4B000000 + ey) - 8388608.0f;
+  const float fez = __int_as_float(0x4B000000 + ez) - 8388608.0f;
+  if (lane < 3 * NQ) {
     // Gauss points relative to the origin as double-float, h (e + g), per axis
-    const int eax[3] = {ex, ey, ez};
-    const float hh[3] = {P.hx_hi, P.hy_hi, P.hz_hi}, hl[3] = {P.hx_lo, P.hy_lo, P.hz_lo};
-#pragma unroll
-    for (int ax = 0; ax < 3; ++ax)
-#pragma unroll
-      for (int a = 0; a <= K; ++a) {
-        df64 t = df64((float)eax[ax]) + df64(P.g_hi[a], P.g_lo[a]);
-        df64 G = df64(hh[ax], hl[ax]) * t;
-        sm.xqf[wp][ax][a][0] = G.hi;
-        sm.xqf[wp][ax][a][1] = G.lo;
-      }
+    const int ax = lane / NQ, a = lane % NQ;
+    const df64 t = df64(ax == 0 ? fex : ax == 1 ? fey : fez, 0.f) + df64(P.g_hi[a], P.g_lo[a]);
+    const df64 hd = ax == 0   ? df64(P.hx_hi, P.hx_lo)
+                    : ax == 1 ? df64(P.hy_hi, P.hy_lo)
+                              : df64(P.hz_hi, P.hz_lo);
+    const df64 xg = hd * t;
+    sm.xqf[wp][ax][a][0] = xg.hi;
+    sm.xqf[wp][ax][a][1] = xg.lo;
+    if (a == 0) sm.el[wp][ax] = ax == 0 ? ex : ax == 1 ? ey : ez;
   }
   // element centre relative to the mesh origin, float-float
   float chx, clx, chy, cly, chz, clz;
-  chx = ff_two_prod_sum((float)ex + 0.5f, P.hx_hi, P.hx_lo, &clx);
-  chy = ff_two_prod_sum((float)ey + 0.5f, P.hy_hi, P.hy_lo, &cly);
-  chz = ff_two_prod_sum((float)ez + 0.5f, P.hz_hi, P.hz_lo, &clz);
+  chx = ff_two_prod_sum(fex + 0.5f, P.hx_hi, P.hx_lo, &clx);
+  chy = ff_two_prod_sum(fey + 0.5f, P.hy_hi, P.hy_lo, &cly);
+  chz = ff_two_prod_sum(fez + 0.5f, P.hz_hi, P.hz_lo, &clz);
   // half extents of the box spanned by the element's Gauss points (every
   // neighbour of a Gauss point lies within R + r of it)
   const float hhx = P.gbox[0], hhy = P.gbox[1], hhz = P.gbox[2];
-  const double rmax = __longlong_as_double((long long)st->rmax_bits);
-  const float cut = (float)(P.R + rmax) * (1.0f + 1e-5f);
-  // bin range per axis (conservative)
+  const df64 rmx = df_from_double_int(__longlong_as_double((long long)st->rmax_bits));
+  const float cut = (P.R32 + rmx.hi) * (1.0f + 1e-5f);  // rounded up: conservative
+  // bin range per axis (conservative): floors of values clamped to
+  // [0, nb - 1] first
   int bx0, bx1, by0, by1, bz0, bz1;
   {
-    int l = (int)floorf((chx - hhx - cut) * P.inv_be[0] - 1e-3f);
-    int h = (int)floorf((chx + hhx + cut) * P.inv_be[0] + 1e-3f);
-    bx0 = min(max(l, 0), b.nb[0] - 1);
-    bx1 = min(max(h, 0), b.nb[0] - 1);
-    l = (int)floorf((chy - hhy - cut) * P.inv_be[1] - 1e-3f);
-    h = (int)floorf((chy + hhy + cut) * P.inv_be[1] + 1e-3f);
-    by0 = min(max(l, 0), b.nb[1] - 1);
-    by1 = min(max(h, 0), b.nb[1] - 1);
-    l = (int)floorf((chz - hhz - cut) * P.inv_be[2] - 1e-3f);
-    h = (int)floorf((chz + hhz + cut) * P.inv_be[2] + 1e-3f);
-    bz0 = min(max(l, 0), b.nb[2] - 1);
-    bz1 = min(max(h, 0), b.nb[2] - 1);
+    auto cellof = [&](float t, int a) {
+      int k;
+      floor_small(fminf(fmaxf(t, 0.0f), b.nm1f[a]), &k);
+      return k;
+    };
+    bx0 = cellof((chx - hhx - cut) * P.inv_be[0] - 1e-3f, 0);
+    bx1 = cellof((chx + hhx + cut) * P.inv_be[0] + 1e-3f, 0);
+    by0 = cellof((chy - hhy - cut) * P.inv_be[1] - 1e-3f, 1);
+    by1 = cellof((chy + hhy + cut) * P.inv_be[1] + 1e-3f, 1);
+    bz0 = cellof((chz - hhz - cut) * P.inv_be[2] - 1e-3f, 2);
+    bz1 = cellof((chz + hhz + cut) * P.inv_be[2] + 1e-3f, 2);
   }
   __syncwarp();
 
@@ -396,6 +501,7 @@ k_qcm(MeshDev m, QcmParams P, BinDev b, const int32_t* __restrict__ bin_start,
   // inside it -- has a single call site in the code.
   int nb = 0;  // buffered culled candidates (warp-uniform)
   const int nrx = by1 - by0 + 1, nrows = nrx * (bz1 - bz0 + 1);
+  const float inv_nrx = __fdividef(1.0f, __int_as_float(0x4B000000 + nrx) - 8388608.0f);
   int rb = -32, base = 0, total = 0;  // row batch, chunk start, candidates in the batch
   int my_s0 = 0, my_excl = 0;         // this lane's row: first slot, offset in the batch
   bool more = true;
@@ -411,7 +517,10 @@ k_qcm(MeshDev m, QcmParams P, BinDev b, const int32_t* __restrict__ bin_start,
         int cntr = 0;
         my_s0 = 0;
         if (ri < nrows) {
-          int by = by0 + ri % nrx, bz = bz0 + ri / nrx;
+          int by, bz;
+          row_split(ri, nrx, inv_nrx, &by, &bz);
+          by += by0;
+          bz += bz0;
           int64_t row = (int64_t)b.nb[0] * (by + (int64_t)b.nb[1] * bz);
           my_s0 = bin_start[row + bx0];
           cntr = bin_start[row + bx1 + 1] - my_s0;
@@ -465,7 +574,7 @@ k_qcm(MeshDev m, QcmParams P, BinDev b, const int32_t* __restrict__ bin_start,
     if (nb == 0) break;
     __syncwarp();
     const int cnt = nb < 32 ? nb : 32;
-    qcm_group<K>(sm, w, P, cnt, xs64, xs32, perm);
+    qcm_group<K>(sm, w, P, cnt, xs64, xs32, perm, nb_count, nb_idsum);
     int rest = nb - cnt;
     float4 tb = make_float4(0.f, 0.f, 0.f, 0.f);
     int ts = 0;
@@ -483,14 +592,18 @@ k_qcm(MeshDev m, QcmParams P, BinDev b, const int32_t* __restrict__ bin_start,
   }
   __syncwarp();
 
-  // outputs
-  const int64_t o = e * Q;
-  for (int q = lane; q < Q; q += 32) {
-    df64 a = sm.accdf[wp][q];
-    if (eps64) eps64[o + q] = 1.0 - ((double)a.hi + (double)a.lo) * P.inv_vr;
-    if (nb_count) nb_count[o + q] = sm.cnt[wp][q];
-    if (nb_idsum) nb_idsum[o + q] = sm.ids[wp][q];
-  }
+  // outputs: a point's lane sums, in units of (pi / 12) / V_R
+  if (eps64)
+    for (int q = lane; q < Q; q += 32) {
+      const int ps = q / G::kPts, l0 = (q - ps * G::kPts) * G::kLanes;
+      df64 a(0.f, 0.f);
+#pragma unroll
+      for (int t = 0; t < G::kLanes; ++t) {
+        const float2 v = sm.acc[wp][ps][l0 + t];
+        a += df64(v.x, v.y);
+      }
+      eps64[o + q] = fma(-double_from_df_int(a), P.inv_vr12, 1.0);
+    }
 }
 
 // ----------------------------------------------------------------------------
@@ -550,9 +663,9 @@ k_qcm_pts(MeshDev m, QcmParams P, BinDev b, const int32_t* __restrict__ bin_star
   const int64_t e = blockIdx.x * (int64_t)kQcmWarps + wp;
   if (e >= m.E) return;  // whole warp leaves together
   const int e32 = (int)e, exy = m.ne[0] * m.ne[1];  // E < 2^31
-  const int ez = e32 / exy;
+  const int ez = P.by_exy.div(e32);
   const int rxy = e32 - ez * exy;
-  const int ey = rxy / m.ne[0];
+  const int ey = P.by_ex.div(rxy);
   const int ex = rxy - ey * m.ne[0];
   const bool want_ids = nb_idsum != nullptr;
   const bool want_counts = nb_count != nullptr || want_ids;
@@ -609,6 +722,7 @@ k_qcm_pts(MeshDev m, QcmParams P, BinDev b, const int32_t* __restrict__ bin_star
   // across rows, as in k_qcm); every 32 kept ones are tested
   int nb = 0;
   const int nrx = by1 - by0 + 1, nrows = nrx * (bz1 - bz0 + 1);
+  const float inv_nrx = __fdividef(1.0f, __int_as_float(0x4B000000 + nrx) - 8388608.0f);
   int rb = -32, base = 0, total = 0;
   int my_s0 = 0, my_excl = 0;
   bool more = true;
@@ -624,7 +738,10 @@ k_qcm_pts(MeshDev m, QcmParams P, BinDev b, const int32_t* __restrict__ bin_star
         int cntr = 0;
         my_s0 = 0;
         if (ri < nrows) {
-          const int by = by0 + ri % nrx, bz = bz0 + ri / nrx;
+          int by, bz;
+          row_split(ri, nrx, inv_nrx, &by, &bz);
+          by += by0;
+          bz += bz0;
           const int64_t row = (int64_t)b.nb[0] * (by + (int64_t)b.nb[1] * bz);
           my_s0 = bin_start[row + bx0];
           cntr = bin_start[row + bx1 + 1] - my_s0;
@@ -892,8 +1009,8 @@ cudaError_t launch_qcm(const MeshDev& m, const Tables& t, const BinDev& b, int p
   P.cw = nullptr;
   P.R = R;
   P.R32 = (float)R;
-  P.inv_vr = 1.0 / (4.0 / 3.0 * kPi * R * R * R);
-  P.inv_vr32 = (float)P.inv_vr;
+  P.inv_vr12 = 1.0 / (16.0 * R * R * R);
+  P.inv_vr32 = (float)(1.0 / (4.0 / 3.0 * kPi * R * R * R));
   P.hx = (float)m.h[0];
   P.hy = (float)m.h[1];
   P.hz = (float)m.h[2];
@@ -933,6 +1050,18 @@ cudaError_t launch_qcm(const MeshDev& m, const Tables& t, const BinDev& b, int p
   if (delta < 1.0 / 4096.0) delta = 1.0 / 4096.0;
   if (delta > 0.25) delta = 0.25;
   P.delta = (float)delta;
+  // band of the double-float predicate: the relative positions are known to
+  // about 2^-44 of the box, the definition rounds to 2^-51 of box plus origin,
+  // and 1/R of either moves the squared distance by 2 sqrt(3) times as much,
+  // its own arithmetic by 2^-43; 16 times that and more
+  double far = 0.0, off = 0.0;
+  for (int a = 0; a < 3; ++a) {
+    far = m.L[a] > far ? m.L[a] : far;
+    off = fabs(m.x0[a]) > off ? fabs(m.x0[a]) : off;
+  }
+  P.delta_df = (float)((1.0 / 64.0 + (far + off / 64.0) / R) / 274877906944.0);  // 2^-38
+  P.by_exy.set(m.ne[0] * m.ne[1]);
+  P.by_ex.set(m.ne[0]);
   for (int q = 0; q < 64; ++q) {
     int qx = q % nq, qy = (q / nq) % nq, qz = q / (nq * nq);
     double wq = q < nq * nq * nq ? t.w[qx] * t.w[qy] * t.w[qz] : 0.0;
@@ -957,11 +1086,11 @@ cudaError_t launch_qcm(const MeshDev& m, const Tables& t, const BinDev& b, int p
     count_launches(1);
     P.cw = cw;
   }
-  dim3 grid((unsigned)((m.E + kQcmWarps - 1) / kQcmWarps));
-  dim3 block(kQcmWarps * 32);
   bool fp64 = precision == 0;
 #define CFDEM_QCM(KK)                                                                     \
   if (m.k == KK) {                                                                        \
+    const int wb = fp64 ? QcmGeom<KK>::kWarps : kQcmWarps;                                \
+    const dim3 grid((unsigned)((m.E + wb - 1) / wb)), block(wb * 32);                     \
     if (fp64)                                                                             \
       k_qcm<KK><<<grid, block, 0, s>>>(m, P, b, bin_start, perm, xs64, xs32, st, eps_q64, \
                                        nb_count, nb_idsum);                               \
