@@ -278,8 +278,9 @@ __device__ __noinline__ bool in_band(const QcmSmem<K>& sm, int wp, int j, float 
 // once per group -- and 30 for its sum.  100,000 spheres, Q2 32x32x128: 354 us
 // with everything formed per hit and a segmented warp scan of double-floats
 // per 32 hits, 300 us with the tables and the lane sums, 242 us with the FP64
-// and conversion instructions out of the per-element code; Q3 (23,000
-// spheres) 97 -> 64 us, Q1 (9,000) 17 -> 11 us.
+// and conversion instructions out of the per-element code, 238 us with idle
+// lanes as NaN candidates instead of a predicate in every test; Q3 (23,000
+// spheres) 97 -> 62 us, Q1 (9,000) 17 -> 11 us.
 template <int K>
 __device__ __forceinline__ void qcm_group(QcmSmem<K>& sm, const QcmWarp& w,
                                           const QcmParams& P, int cnt,
@@ -292,10 +293,10 @@ __device__ __forceinline__ void qcm_group(QcmSmem<K>& sm, const QcmWarp& w,
   constexpr int NQ = G::NQ;
   const unsigned FULL = 0xffffffffu;
   const int lane = w.lane, wp = w.warp;
-  const bool valid = lane < cnt;
-  float4 my = make_float4(0.f, 0.f, 0.f, 0.f);
+  // a lane without a candidate: a NaN, which no comparison lets through
+  float4 my = make_float4(__int_as_float(0x7fffffff), 0.f, 0.f, 0.f);
   int myslot = 0;
-  if (valid) {
+  if (lane < cnt) {
     my = sm.buf[wp][lane];
     myslot = sm.bslot[wp][lane];
     const float4* ff = reinterpret_cast<const float4*>(xs32) + 2 * (int64_t)myslot;
@@ -345,10 +346,9 @@ __device__ __forceinline__ void qcm_group(QcmSmem<K>& sm, const QcmWarp& w,
 #pragma unroll
         for (int a = 0; a < NQ; ++a) {
           float d2 = sx[a] + syz;
-          bool hit = valid && d2 < c2_in;
-          if (valid && d2 >= c2_in && d2 <= c2_out) {  // inside the band: exact FP64 predicate
+          bool hit = d2 < c2_in;
+          if (!hit && d2 <= c2_out)  // inside the band
             hit = in_band<K>(sm, wp, lane, P.delta_df, xs64, myslot, a | (b << 2) | (cz << 4));
-          }
           unsigned mask = __ballot_sync(FULL, hit);
           if (hit)
             sm.queue[wp][qn + __popc(mask & w.lt_mask)] =
