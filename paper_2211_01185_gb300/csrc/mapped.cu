@@ -32,10 +32,13 @@
 // (no quick convergence, iterates far out, a Jacobian that changes much) to
 // the FP64 iteration from the centre.  polish_in finishes an accepted start
 // with double-float residuals and the FP32 inverse Jacobian: each step gains
-// about five digits, so two residuals reach the 1e-13.  120,000 points on a
+// about five digits, so two residuals reach the 1e-13, and one more with the
+// residual in FP64 (fp64_step) takes the double-float rounding out: without it
+// 0.225 ms below, but up to twice the plain iteration's error on some meshes.
+// 120,000 points on a
 // Q2 cylinder of 5,280 elements: locate and interpolate a 3-vector 13.6 ms
-// with plain FP64 Newton, 0.225 ms now
-// (locate 175 us: scattered loads of control points, 16 warps an SM).
+// with plain FP64 Newton, 0.328 ms now
+// (scattered loads of control points at 16 warps an SM, the FP64 step).
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -423,6 +426,45 @@ __device__ __forceinline__ void bernstein_df(df64 t, df64* l) {
   }
 }
 
+// One step with the map's residual in FP64 and the FP32 inverse Jacobian, so
+// that a polished xi carries the rounding of the FP64 definition and not the
+// double-float one
+template <int K>
+__device__ __forceinline__ void fp64_step(const MappedDev& md, const Tables& tb, int64_t e,
+                                          const double p[3], const float Ji[3][3], float inv,
+                                          double xi[3]) {
+  constexpr int NQ = K + 1, NL = NQ * NQ * NQ;
+  const int32_t* cn = md.conn + e * NL;
+  double l[3][NQ], dl[3][NQ];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) cfdem::lagrange<K, double>(tb.z, tb.lw, xi[a], l[a], dl[a]);
+  double X[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+  for (int c = 0; c < NQ; ++c) {
+    double u[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int b = 0; b < NQ; ++b) {
+      double v[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+      for (int a = 0; a < NQ; ++a) {
+        const double* P = md.nodes + 3 * (int64_t)cn[a + NQ * (b + NQ * c)];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) v[i] += l[0][a] * __ldg(P + i);
+      }
+#pragma unroll
+      for (int i = 0; i < 3; ++i) u[i] += l[1][b] * v[i];
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) X[i] += l[2][c] * u[i];
+  }
+  float r[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) r[i] = (float)(X[i] - p[i]) * inv;
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+    xi[a] -= (double)(Ji[a][0] * r[0] + Ji[a][1] * r[1] + Ji[a][2] * r[2]);
+}
+
 // Finishes a start of the screen: X_e(xi) = p with residuals in double-float
 // (the element's control points relative to its centre carry 2^-48 of its
 // size, more than FP64 keeps of coordinates 32 element sizes away) and the
@@ -434,7 +476,8 @@ __device__ __forceinline__ void bernstein_df(df64 t, df64* l) {
 // in the cube, 0 when xi lies outside it, -1 when the steps do not shrink
 // fast.
 template <int K>
-__device__ __forceinline__ int polish_in(const MappedDev& md, int64_t e, const double p[3],
+__device__ __forceinline__ int polish_in(const MappedDev& md, const Tables& tb, int64_t e,
+                                         const double p[3],
                                          const float start[3], const float Ji[3][3],
                                          double xi_out[3]) {
   constexpr int NQ = K + 1, NL = NQ * NQ * NQ;
@@ -494,6 +537,10 @@ __device__ __forceinline__ int polish_in(const MappedDev& md, int64_t e, const d
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
         xi_out[a] = (double)xi[a].hi + (double)xi[a].lo;
+      }
+      fp64_step<K>(md, tb, e, p, Ji, (float)inv, xi_out);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
         if (!(xi_out[a] >= -1e-10 && xi_out[a] <= 1.0 + 1e-10)) return 0;
       }
 #pragma unroll
@@ -658,7 +705,7 @@ k_locate_mapped(MappedDev md, Tables tb, int64_t n, const double* __restrict__ x
     __syncwarp();
     if (!done && sc != kOutside) {
       int in = -1;
-      if (sc == kStart) in = polish_in<K>(md, e, p, start, Ji, xo);
+      if (sc == kStart) in = polish_in<K>(md, tb, e, p, start, Ji, xo);
       if (in < 0) in = newton_in<K>(md, tb, e, p, xo) ? 1 : 0;
       if (in) {
         found = e;
