@@ -47,12 +47,7 @@ struct Interp<double> {
 template <>
 struct Interp<float> {
   using V = df64;
-  struct Sum : DfDotAcc {
-    __device__ __forceinline__ void first(V b, V x) {
-      s = b.hi * x.hi;
-      c = fmaf(b.lo, x.hi, fmaf(b.hi, x.lo, fmaf(b.hi, x.hi, -s)));
-    }
-  };
+  using Sum = DfDotAcc;
   static __device__ __forceinline__ double wide(V v) { return double_from_df_int(v); }
 };
 

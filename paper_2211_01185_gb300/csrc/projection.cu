@@ -369,13 +369,7 @@ struct Acc {
 // residuals accurate to ~1e-14 on the FP32 pipes, which on this part have 61
 // times the FP64 throughput.
 template <>
-struct Acc<df64> : DfDotAcc {
-  // the first term needs no two-sum: 4 instructions instead of 12
-  __device__ __forceinline__ void first(df64 b, df64 x) {
-    s = b.hi * x.hi;
-    c = fmaf(b.lo, x.hi, fmaf(b.hi, x.lo, fmaf(b.hi, x.hi, -s)));
-  }
-};
+struct Acc<df64> : DfDotAcc {};
 
 // --- load and epilogue policies of the tile operator -----------------------
 // Plain: x_eff = x[g]

@@ -93,8 +93,8 @@ struct QcmParams {
 
 __device__ __forceinline__ float ff_two_prod_sum(float a, float b_hi, float b_lo, float* lo) {
   // a * (b_hi + b_lo) as a float-float; a is an exact small integer + 0.5
-  float p = a * b_hi;
-  float e = fmaf(a, b_hi, -p);
+  float e;
+  const float p = two_prod(a, b_hi, &e);
   *lo = e + a * b_lo;
   return p;
 }
@@ -176,8 +176,8 @@ __device__ __forceinline__ df64 lens_df(df64 R, df64 r, df64 D, df64 c43, df64 c
 }
 
 __device__ __forceinline__ df64 df_sq(df64 a) {
-  const float p = a.hi * a.hi;
-  const float e = fmaf(a.hi, a.hi, -p);
+  float e;
+  const float p = two_prod(a.hi, a.hi, &e);
   return df_renorm(p, fmaf(a.hi + a.hi, a.lo, e));
 }
 // (s, e) += v, e the sum of the rounding errors and low parts
@@ -194,23 +194,26 @@ __device__ __forceinline__ void df_gather(float& s, float& e, float v) {
 __device__ __forceinline__ df64 lens_hit(df64 D, float4 rad, float2 full) {
   if (df_le(D, df64(rad.z, rad.w))) return df64(full.x, full.y);
   const float y = rsqrtf(D.hi);
-  const float x0 = D.hi * y;
-  const float sq = x0 * x0;
-  const float r0 = (D.hi - sq) + (D.lo - fmaf(x0, x0, -sq));  // D - x0^2
+  const float x0 = __fmul_rn(D.hi, y);
+  float sq_e;
+  const float sq = two_prod(x0, x0, &sq_e);
+  const float r0 = (D.hi - sq) + (D.lo - sq_e);  // D - x0^2
   const df64 d = df_renorm(x0, r0 * (0.5f * y));
   const df64 S(rad.x, rad.y);
   const df64 sd = S - d;
   // D + 2 d S - 3 (R - r)^2, the three high parts and all errors apart
   const df64 dS = d * S;
-  const float p3 = 3.0f * rad.z;
+  float p3_e;
+  const float p3 = two_prod(3.0f, rad.z, &p3_e);
   float hi = D.hi, lo = D.lo + 2.0f * dS.lo;
-  lo -= fmaf(3.0f, rad.w, fmaf(3.0f, rad.z, -p3));
+  lo -= fmaf(3.0f, rad.w, p3_e);
   df_gather(hi, lo, 2.0f * dS.hi);
   df_gather(hi, lo, -p3);
   const df64 num = df_renorm(hi, lo);
   const float y1 = fmaf(y, fmaf(-d.hi, y, 1.0f), y);
-  const float pe = d.hi * y1;
-  const float re = (1.0f - pe) - fmaf(d.lo, y1, fmaf(d.hi, y1, -pe));
+  float pe_e;
+  const float pe = two_prod(d.hi, y1, &pe_e);
+  const float re = (1.0f - pe) - fmaf(d.lo, y1, pe_e);
   return df_sq(sd) * (num * df_renorm(y1, y1 * re));
 }
 
