@@ -90,6 +90,7 @@ struct CgScalars {
   unsigned int ticket;  // last-block counter
   int loops;       // bodies of a device-driven CG loop run so far
   float alpha_hi, alpha_lo;  // double-float split of alpha (mixed solve)
+  int split;        // 1 while the FP64 solve takes its operator in double-float
   int xnz;          // 1 if the start vector has a nonzero entry (else A x0 = 0 is skipped)
   double* x;        // iterate of the FP64 solve, where its loop is not given it (a graph)
   // kept over the resets between solves (kCgReset): 1 once a solve whose

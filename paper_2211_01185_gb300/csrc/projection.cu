@@ -456,15 +456,18 @@ struct EpiStoreDf {
     return __ldcg(reinterpret_cast<const float*>(p + g)) * acc.hi;
   }
 };
-// df64 image of an FP64 direction, stored in FP64; the dot product in df64
+// df64 image of an FP64 direction, stored in FP64; the dot product in FP64:
+// its terms are of the size of b times the square of what the residual has
+// dropped by, far outside FP32's exponents for ordinary right-hand sides
 struct EpiStoreSplit {
-  using acc_t = df64;
+  using acc_t = double;
   static constexpr bool kXE = false;
   double* y;
   const double* p;  // the direction, written by this block's load phase
-  __device__ __forceinline__ df64 operator()(int64_t g, df64 acc, df64) const {
-    y[g] = double_from_df_int(acc);
-    return df_from_double_int(__ldcg(p + g)) * acc;
+  __device__ __forceinline__ double operator()(int64_t g, df64 acc, df64) const {
+    const double v = double_from_df_int(acc);
+    y[g] = v;
+    return __ldcg(p + g) * v;
   }
 };
 // residual r = b - A x in df64; r32 = high part (input of the FP32
@@ -751,11 +754,18 @@ k_cg_apply(MeshDev m, const T* __restrict__ bands, Coefs<T> cf, const T* __restr
 // |b| the direction is of that size too, and the 2^-47 of the double-float
 // image are 1e-18 of b -- a hundredth of an FP64 rounding of what the first
 // directions added, so the solution keeps its FP64 accuracy, at less than half
-// the time (Q2 65 x 65 x 257: 106 -> 60 us).  Both kernels are
-// queued and one of them returns at once.
-__device__ __forceinline__ bool small_residual(const CgScalars* sc) {
-  const volatile CgScalars* v = sc;
-  return v->rr <= 1e-8 * v->bb;
+// the time (Q2 65 x 65 x 257: 106 -> 60 us).  Double-float has FP32's
+// exponents: where the residual, or the direction, which is the residual over
+// the elements' volume, is below 1e-25 or above 1e25, the operator stays in
+// FP64 (a double-float image of 1e-25 still keeps 1e-45, which is 1e-24 of
+// b).  Both kernels are queued and one of them returns at once;
+// k_cg_update64 decides for the iterations that follow.
+struct SplitRange {
+  double lo, hi;  // of r . r
+};
+static SplitRange split_range(const MeshDev& m) {
+  const double v2 = m.Ve * m.Ve;
+  return {1e-50 * (v2 > 1.0 ? v2 : 1.0), 1e50 * (v2 < 1.0 ? v2 : 1.0)};
 }
 
 // p = z + beta p_old ; Ap = A p ; alpha = rz / (p . Ap)
@@ -765,7 +775,7 @@ k_cg_apply64(MeshDev m, const double* __restrict__ bands, Coefs<double> cf,
              const float* __restrict__ z, const double* __restrict__ p_old,
              double* __restrict__ p_new, double* __restrict__ Ap, double* partials, CgScalars* sc,
              int first) {
-  if (((volatile CgScalars*)sc)->done || (!first && small_residual(sc))) return;
+  if (((volatile CgScalars*)sc)->done || (!first && ((volatile CgScalars*)sc)->split)) return;
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ double red[32];
   LoadDir64 ld{z, p_old, p_new, first ? 0.0 : sc->beta, first != 0};
@@ -786,13 +796,13 @@ k_cg_apply64_split(MeshDev m, const df64* __restrict__ bands, Coefs<df64> cf,
                    const float* __restrict__ z, const double* __restrict__ p_old,
                    double* __restrict__ p_new, double* __restrict__ Ap, double* partials,
                    CgScalars* sc) {
-  if (((volatile CgScalars*)sc)->done || !small_residual(sc)) return;
+  if (((volatile CgScalars*)sc)->done || !((volatile CgScalars*)sc)->split) return;
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ double red[32];
   LoadDirSplit ld{z, p_old, p_new, df_from_double(sc->beta)};
   EpiStoreSplit ep{Ap, p_new};
-  const df64 d = apply_tile<K, S, df64>(m, bands, cf, ld, ep, reinterpret_cast<df64*>(smraw));
-  double vals[1] = {block_sum(double_from_df_int(d), red)};
+  const double d = apply_tile<K, S, df64>(m, bands, cf, ld, ep, reinterpret_cast<df64*>(smraw));
+  double vals[1] = {block_sum(d, red)};
   double out[1];
   if (last_block_reduce(partials, 1, vals, &sc->ticket, out, red) && threadIdx.x == 0) {
     sc->pAp = out[0];
@@ -875,7 +885,7 @@ k_cg_start(int64_t n, const TB* __restrict__ b, const T* __restrict__ Ax, T* __r
 __global__ void __launch_bounds__(256)
 k_cg_update64(int64_t n, double* __restrict__ r, const double* __restrict__ p,
               const double* __restrict__ Ap, float* __restrict__ rf, double* partials,
-              CgScalars* sc, int maxit) {
+              CgScalars* sc, int maxit, SplitRange range) {
   if (((volatile CgScalars*)sc)->done) return;
   __shared__ double red[256];
   const double alpha = sc->alpha;
@@ -892,9 +902,11 @@ k_cg_update64(int64_t n, double* __restrict__ r, const double* __restrict__ p,
   double vals[1] = {block_sum256(rr, red)};
   double out[1];
   if (last_block_reduce(partials, 1, vals, &sc->ticket, out, red) && threadIdx.x == 0) {
-    sc->rr = out[0];
+    const double r2 = out[0];
+    sc->rr = r2;
+    sc->split = r2 <= 1e-8 * sc->bb && r2 >= range.lo && r2 <= range.hi;
     sc->it += 1;
-    if (out[0] <= sc->tol2 || sc->it >= maxit) sc->done = 1;
+    if (r2 <= sc->tol2 || sc->it >= maxit) sc->done = 1;
   }
 }
 
@@ -1611,7 +1623,8 @@ static cudaError_t cg_solve64(const MeshDev& m, const double* bands, const doubl
       k_cg_apply64_split<K, S><<<g, kApplyThreads, apply_smem<K, S, df64>(), st>>>(
           m, w.bands_df, cfd, zc, pc, pn, w.Ap, w.partials, sc);
     if (tm) tm->end(kStageOp64, st);
-    k_cg_update64<<<vb, 256, 0, st>>>(n, w.r, pn, w.Ap, w.r32, w.partials, sc, maxit);
+    k_cg_update64<<<vb, 256, 0, st>>>(n, w.r, pn, w.Ap, w.r32, w.partials, sc, maxit,
+                                       split_range(m));
     count_launches(first ? 2 : 3);
     cudaError_t ee = cudaGetLastError();
     if (ee != cudaSuccess) return ee;
