@@ -219,8 +219,10 @@ cfdem_status cfdem_apply(cfdem_t ctx, const double *x_dev, double *y_dev);
  * above cg_rtol is reported by the next cfdem_synchronize either way.
  * While the context's stream is being captured into a CUDA graph the CG
  * loop becomes a conditional (while) node of that graph that iterates on the
- * device until convergence or cg_maxit; the statistics of a replay are read
- * by the next cfdem_synchronize / cfdem_get_stats.  Capture requires the
+ * device until convergence or cg_maxit; the statistics of the last replay
+ * are read by the next cfdem_synchronize / cfdem_get_stats, and a solve that
+ * stopped above cg_rtol is reported there even if later solves or replays
+ * have followed it.  Capture requires the
  * stage timers off and, for the mixed path, the fast-diagonalisation
  * preconditioner (else CFDEM_ESTATE). */
 cfdem_status cfdem_project(cfdem_t ctx, const double *eps_q_dev, double *eps_nodal_dev);

@@ -490,22 +490,27 @@ cfdem_status alloc_mesh_arena(cfdem_t c) {
   return CFDEM_OK;
 }
 
-// statistics of a solve that ran inside a graph, from the device scalars
-// (the stream has been synchronised)
+// statistics of a solve whose outcome the host has not read, from the device
+// scalars (the stream has been synchronised); a failure is read once
 cudaError_t read_pending_stats(cfdem_t c) {
-  if (!c->stats_pending || !c->cg.sc) return cudaSuccess;
+  if (!(c->stats_pending || c->captured_solves) || !c->cg.sc) return cudaSuccess;
   CgScalars hs;
   cudaError_t e = cudaMemcpy(&hs, c->cg.sc, sizeof hs, cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return e;
-  double bb = hs.bb > 0 ? hs.bb : 1.0;
-  c->last_iters = hs.it;
-  c->last_outer = c->prm.precision == 1 ? hs.it : 0;
-  c->last_relres = std::sqrt(hs.rr / bb);
-  c->last_converged = c->last_relres <= c->prm.cg_rtol;
-  if (!c->last_converged || hs.failed) c->pending_not_converged = 1;
-  if (hs.failed) {
-    const int zero = 0;
-    e = cudaMemcpy(&c->cg.sc->failed, &zero, sizeof zero, cudaMemcpyHostToDevice);
+  bool failed = hs.failed != 0;
+  if (hs.unread) {
+    double bb = hs.bb > 0 ? hs.bb : 1.0;
+    c->last_iters = hs.it;
+    c->last_outer = c->prm.precision == 1 ? hs.it : 0;
+    c->last_relres = std::sqrt(hs.rr / bb);
+    c->last_converged = hs.rr <= hs.tol2;  // the tolerance it ran with
+    failed = failed || !c->last_converged;
+  }
+  if (failed) {
+    c->pending_not_converged = 1;
+    static_assert(offsetof(CgScalars, failed) == offsetof(CgScalars, unread) + sizeof(int), "");
+    const int zero[2] = {0, 0};
+    e = cudaMemcpy(&c->cg.sc->unread, zero, sizeof zero, cudaMemcpyHostToDevice);
   }
   c->stats_pending = false;
   return e;
@@ -513,7 +518,7 @@ cudaError_t read_pending_stats(cfdem_t c) {
 
 // read a finished solve's outcome before what it depends on changes
 cfdem_status settle_stats(cfdem_t c) {
-  if (!c->stats_pending) return CFDEM_OK;
+  if (!(c->stats_pending || c->captured_solves)) return CFDEM_OK;
   CK(c->stream ? cudaStreamSynchronize(c->stream) : cudaDeviceSynchronize(), "status");
   CK(read_pending_stats(c), "status");
   return CFDEM_OK;
@@ -592,8 +597,7 @@ cfdem_status solve_graphed(cfdem_t c, const double* b, double* x, bool* done) {
       return CFDEM_OK;
     }
   }
-  // a solve whose outcome nobody has read yet: remember a failure
-  if (c->stats_pending) CK(launch_cg_keep(c->cg.sc, c->stream), "solve");
+  c->cg.unread = 1;
   CK(solve_part(c, kSolveStart, b, x, c->stream, &it, &outer, &rel, &conv), "solve");
   CK(cudaGraphLaunch(c->loop_exec, c->stream), "solve");
   CK(solve_part(c, kSolveFinish, b, x, c->stream, &it, &outer, &rel, &conv), "solve");
@@ -619,10 +623,9 @@ cfdem_status solve(cfdem_t c, const double* b, double* x, const char* what) {
     bool done = false;
     const cfdem_status st = solve_graphed(c, b, x, &done);
     if (st != CFDEM_OK || done) return st;
-    const cfdem_status ss = settle_stats(c);  // the scalars are about to be overwritten
-    if (ss != CFDEM_OK) return ss;
   }
   c->cg.loop = captured ? c->loop_stream : nullptr;
+  c->cg.unread = captured;
   c->cg.timer = c->timer.on ? &c->timer : nullptr;
   c->timer.begin(kStageSolve, c->stream);
   e = solve_part(c, kSolveAll, b, x, c->stream, &it, &outer, &rel, &conv);
@@ -633,10 +636,10 @@ cfdem_status solve(cfdem_t c, const double* b, double* x, const char* what) {
   if (e != cudaSuccess) return cuda_fail(c, e, what);
   c->timer.end(kStageSolve, c->stream);
   if (captured) {
-    c->stats_pending = true;
+    c->stats_pending = c->captured_solves = true;
     return CFDEM_OK;
   }
-  c->stats_pending = false;
+  // (stats_pending stays: a solve before this one may have failed unread)
   c->last_iters = it;
   c->last_outer = outer;
   c->last_relres = rel;
@@ -955,6 +958,7 @@ cfdem_status cfdem_set_mesh(cfdem_t c, const double origin[3], const double exte
   if (c->stream) cudaStreamSynchronize(c->stream);
   drop_loop(c);
   free_mesh_arena(c);
+  c->captured_solves = false;  // such graphs end with the arena
   c->mesh = m;
   c->have_mesh = true;
   s = alloc_mesh_arena(c);

@@ -71,10 +71,12 @@ struct cfdem_ctx {
   int last_iters = 0, last_outer = 0, last_converged = 1;
   double last_relres = 0.0;
   int pending_not_converged = 0;
-  // set when the last solve ran inside a captured graph: its iteration count
-  // and residual are read from the device scalars at the next synchronising
-  // call
-  bool stats_pending = false;
+  // set while a solve's outcome may lie unread in the device scalars (its
+  // iteration count, its residual, and whether it or an unread one before it
+  // failed): read at the next synchronising call.  captured_solves: a graph
+  // of the caller's holds a solve of this context, whose replays the host
+  // does not see
+  bool stats_pending = false, captured_solves = false;
   cudaStream_t loop_stream = nullptr;  // capture stream of device-driven CG loops
   // the CG loop of eager solves as a graph (see solve()): captured on
   // cap_stream at the second solve of a configuration (gen, tile shape)

@@ -2,7 +2,6 @@
 // coupling library.  Nothing here is part of the public C ABI (cfdem.h).
 #pragma once
 
-#include <cstddef>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -93,11 +92,11 @@ struct CgScalars {
   int split;        // 1 while the FP64 solve takes its operator in double-float
   int xnz;          // 1 if the start vector has a nonzero entry (else A x0 = 0 is skipped)
   double* x;        // iterate of the FP64 solve, where its loop is not given it (a graph)
-  // kept over the resets between solves (kCgReset): 1 once a solve whose
-  // statistics the host had not read yet stopped above its tolerance
-  int failed;
+  // kept over the resets between solves (k_cg_reset): unread = 1 while the
+  // host has not seen the outcome of the solve (it does not wait for it),
+  // failed = 1 once such a solve stopped above its tolerance
+  int unread, failed;
 };
-constexpr size_t kCgReset = offsetof(CgScalars, failed);
 
 // The parts of a solve.  All queues it whole.  Start, Loop and Finish are the
 // same launches split so that Loop, which touches the solver's own vectors
@@ -297,9 +296,8 @@ struct CgWork {
   // on which the body of the device-driven CG loop is captured
   cudaStream_t loop;
   SolvePart part;     // what run_cg64 / run_cg_mixed queue (kSolveAll = 0)
+  int unread;         // 1: the host leaves the outcome in the scalars for later
 };
-// folds the last solve's outcome into CgScalars::failed
-cudaError_t launch_cg_keep(CgScalars* sc, cudaStream_t s);
 // true when s is a stream under active capture
 bool stream_capturing(cudaStream_t s);
 int cg_blocks(const MeshDev& m);

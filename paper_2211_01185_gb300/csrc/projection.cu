@@ -1433,12 +1433,18 @@ static cudaError_t loop_close(cudaStream_t ls, cudaGraphConditionalHandle h, CgS
   return body_status != cudaSuccess ? body_status : e;
 }
 
-__global__ void k_cg_keep(CgScalars* sc) {
-  if (!(sc->rr <= sc->tol2)) sc->failed = 1;
+// The scalars of a new solve.  A kernel in place of a memset (also in captured
+// solves, whose replays the host does not see): an outcome that nobody has
+// read yet is folded into `failed` before it is overwritten.
+__global__ void k_cg_reset(CgScalars* sc, int unread) {
+  const int failed = sc->failed || (sc->unread && !(sc->rr <= sc->tol2));
+  *sc = CgScalars{};
+  sc->unread = unread;
+  sc->failed = failed;
 }
 
-cudaError_t launch_cg_keep(CgScalars* sc, cudaStream_t s) {
-  k_cg_keep<<<1, 1, 0, s>>>(sc);
+static cudaError_t cg_reset(const CgWork& w, cudaStream_t s) {
+  k_cg_reset<<<1, 1, 0, s>>>(w.sc, w.unread);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -1577,7 +1583,7 @@ static cudaError_t cg_solve64(const MeshDev& m, const double* bands, const doubl
   CgScalars* sc = w.sc;
   if ((e = set_smem64<K, S>()) != cudaSuccess) return e;
   if (w.part != kSolveLoop) {
-    if ((e = cudaMemsetAsync(sc, 0, kCgReset, s)) != cudaSuccess) return e;
+    if ((e = cg_reset(w, s)) != cudaSuccess) return e;
     // the operator is skipped on the device when x0 has no nonzero entry
     k_flag_nonzero<double><<<vb, 256, 0, s>>>(n, x, &sc->xnz);
     count_launches(1);
@@ -1698,7 +1704,7 @@ static cudaError_t cg_solve_df(const MeshDev& m, const df64* bands, const double
     return cudaGetLastError();
   }
   if (w.part != kSolveLoop) {
-    if ((e = cudaMemsetAsync(w.sc, 0, kCgReset, s)) != cudaSuccess) return e;
+    if ((e = cg_reset(w, s)) != cudaSuccess) return e;
     k_split_df<<<vb, 256, 0, s>>>(n, b, x, w.x_df, w.r_df, w.r32, w.partials, w.sc);
     k_residual_df<K, S><<<g, kApplyThreads, sm, s>>>(m, bands, cf, w.x_df, b, w.r_df, w.r32,
                                                      w.partials, w.sc, rtol);
@@ -1807,7 +1813,7 @@ cudaError_t run_cg64(const MeshDev& m, const double* bands, const double* coef,
     *converged = *relres_host <= rtol;
     return cudaSuccess;
   }
-  if ((e = cudaMemsetAsync(w.sc, 0, kCgReset, s)) != cudaSuccess) return e;
+  if ((e = cg_reset(w, s)) != cudaSuccess) return e;
   if ((e = make_dinv<double>(m, bands, coef, w.dinv, s)) != cudaSuccess) return e;
   e = cg_solve<double, double, double>(m, bands, coef, b, x, x, rtol, maxit, w.r, w.z, w.p0,
                                        w.p1, w.Ap, w.dinv, w.partials, w.sc, s, iters_host,
@@ -1855,7 +1861,7 @@ cudaError_t run_cg_mixed(const MeshDev& m, const double* bands64, const float* b
     if (w.timer) w.timer->begin(kStageOp64, s);
     if ((e = apply_t<double>(m, bands64, coef, x, w.Ap, s)) != cudaSuccess) return e;
     if (w.timer) w.timer->end(kStageOp64, s);
-    if ((e = cudaMemsetAsync(w.sc, 0, kCgReset, s)) != cudaSuccess) return e;
+    if ((e = cg_reset(w, s)) != cudaSuccess) return e;
     k_residual<double><<<vb, 256, 0, s>>>(n, b, w.Ap, w.r, w.partials, w.sc);
     count_launches(1);
     if ((e = cudaMemcpyAsync(&hs, w.sc, sizeof(CgScalars), cudaMemcpyDeviceToHost, s)) !=
@@ -1870,7 +1876,7 @@ cudaError_t run_cg_mixed(const MeshDev& m, const double* bands64, const float* b
     double scale = rn > 0 ? 1.0 / rn : 1.0;
     k_to_f32<<<vb, 256, 0, s>>>(n, w.r, scale, w.rin32, w.d32);
     count_launches(1);
-    if ((e = cudaMemsetAsync(w.sc, 0, kCgReset, s)) != cudaSuccess) return e;
+    if ((e = cg_reset(w, s)) != cudaSuccess) return e;
     int it = 0;
     double rr = 0;
     e = cg_solve<float, float, float>(m, bands32, coef, w.rin32, w.d32, w.d32, inner_rtol,
