@@ -35,7 +35,10 @@
 // about five digits, so two residuals reach the 1e-13, and one more with the
 // residual in FP64 (fp64_step) takes the double-float rounding out: without it
 // 0.225 ms below, but up to twice the plain iteration's error on some meshes.
-// 120,000 points on a
+// Far from the origin rounding decides where the plain iteration ends; there,
+// and on meshes of sizes beyond FP32's exponents, the candidates take it as it
+// is defined, operation by operation (is_far, newton_in), and the elements are
+// the definition's at any distance.  120,000 points on a
 // Q2 cylinder of 5,280 elements: locate and interpolate a 3-vector 13.6 ms
 // with plain FP64 Newton, 0.328 ms now
 // (scattered loads of control points at 16 warps an SM, the FP64 step).
@@ -204,7 +207,9 @@ __device__ __forceinline__ void bernstein(float t, float* l, float* dl) {
 // image X_0 and the Jacobian's determinant.  The ranges are widened by what
 // FP32 loses in J_a . q for coordinates below ten and by the 1e-10 by which
 // xi may pass the cube.  frame[5]: (J_0, lo_0), (J_1, lo_1), (J_2, lo_2),
-// (hi, det), (X_0, 0); det = 0 marks an element too flat for FP32.
+// (hi, det), (X_0, 1 / half edge); det = 0 marks an element that FP32 does not
+// serve: too flat, or of a size near the ends of its exponents (1e-20 and
+// 1e20 leave room for the residuals of the last FP64 step).
 template <int K>
 __global__ void k_frames(int64_t E, const double* __restrict__ ref,
                          const float4* __restrict__ rel, float4* __restrict__ frame) {
@@ -250,7 +255,8 @@ __global__ void k_frames(int64_t E, const double* __restrict__ ref,
     nrm *= sqrt(J[0][i] * J[0][i] + J[1][i] * J[1][i] + J[2][i] * J[2][i]);
   }
   const double det = J[0][0] * A[0][0] + J[0][1] * A[1][0] + J[0][2] * A[2][0];
-  bool ok = ref[4 * e + 3] > 0.0 && fabs(det) >= 1e-3 * nrm && nrm > 1e-12;
+  const double inv = ref[4 * e + 3];
+  bool ok = inv >= 1e-20 && inv <= 1e20 && fabs(det) >= 1e-3 * nrm && nrm > 1e-12;
   float4 f[5];
   float hi[3] = {0.f, 0.f, 0.f};
 #pragma unroll
@@ -274,18 +280,31 @@ __global__ void k_frames(int64_t E, const double* __restrict__ ref,
     hi[a] = (float)up + m;
   }
   f[3] = make_float4(hi[0], hi[1], hi[2], ok ? (float)det : 0.0f);
-  f[4] = make_float4((float)X[0], (float)X[1], (float)X[2], 0.0f);
+  f[4] = make_float4((float)X[0], (float)X[1], (float)X[2], (float)inv);
   for (int q = 0; q < 5; ++q) frame[5 * e + q] = f[q];
 }
 
 enum Screen { kOutside, kStart, kUnsure };
 
-// The hull test of candidate e at p; kStart: not excluded, and xi is the
-// first Newton iterate from the centre, `step` its step and det0 the
-// centre's determinant.  kUnsure: no FP32 screen for this element.
+// How far rounding of coordinates of the size of p (|p| in half edges, a)
+// moves xi, in units of 2^-53: the largest row of |J^-1| a.  The definition's
+// iteration stops at a step of 1e-13, which its roundings can keep it from
+// where this is above 150 (of 200,000 interior points of bent and flat Q1 to
+// Q3 elements the first one missed lies at 152, one in 5,000 is missed at
+// 128 to 256, one in 400 at 256 to 512).  Above kFar the definition's own
+// iteration decides.
+constexpr float kFar = 64.0f;
+__device__ __forceinline__ bool is_far(const float row[3], const float a[3]) {
+  return !(fabsf(row[0]) * a[0] + fabsf(row[1]) * a[1] + fabsf(row[2]) * a[2] <= kFar);
+}
+
+// The hull test of candidate e at p (pf: p in FP32); kStart: not excluded, and
+// xi is the first Newton iterate from the centre, `step` its step and det0 the
+// centre's determinant.  kUnsure: no FP32 screen for this element or this far
+// from the origin.
 __device__ __forceinline__ Screen screen_hull(const MappedDev& md, int64_t e, const double p[3],
-                                              float q[3], float xi[3], float* step,
-                                              float* det0) {
+                                              const float pf[3], float q[3], float xi[3],
+                                              float* step, float* det0) {
   const float4* f = md.frame + 5 * e;
   const double* rf = md.ref + 4 * e;
   const float4 h = __ldg(f + 3);
@@ -295,12 +314,15 @@ __device__ __forceinline__ Screen screen_hull(const MappedDev& md, int64_t e, co
   for (int i = 0; i < 3; ++i) q[i] = (float)((p[i] - rf[i]) * inv);
   const float4 X0 = __ldg(f + 4);
   const float up[3] = {h.x, h.y, h.z};
+  const float size[3] = {fabsf(pf[0]) * X0.w, fabsf(pf[1]) * X0.w, fabsf(pf[2]) * X0.w};
   const float d0[3] = {X0.x - q[0], X0.y - q[1], X0.z - q[2]};
   float big = 0.0f;
-  bool out = false;
+  bool out = false, far = false;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     const float4 r = __ldg(f + a);
+    const float row[3] = {r.x, r.y, r.z};
+    far = far || is_far(row, size);
     const float t = fmaf(r.z, q[2], fmaf(r.y, q[1], r.x * q[0]));
     out = out || t < r.w || t > up[a];
     const float d = fmaf(r.z, d0[2], fmaf(r.y, d0[1], r.x * d0[0]));
@@ -309,7 +331,7 @@ __device__ __forceinline__ Screen screen_hull(const MappedDev& md, int64_t e, co
   }
   *step = big;
   *det0 = h.w;
-  return out ? kOutside : kStart;
+  return far ? kUnsure : (out ? kOutside : kStart);
 }
 
 // The FP32 Newton screen (see the file comment), from the hull test's first
@@ -470,11 +492,10 @@ __device__ __forceinline__ void fp64_step(const MappedDev& md, const Tables& tb,
 // size, more than FP64 keeps of coordinates 32 element sizes away) and the
 // FP32 inverse Jacobian.  A linear iteration with ratio rho ~ 1e-5: done when
 // the step is at most 1e-13, or the step that would follow it (step * rho,
-// rho from the last two) at most 1e-15 -- the latter only where coordinates
-// of this size resolve xi that far (far from the origin the FP64 iteration
-// from the centre decides whether 1e-13 can be reached).  Returns 1 with xi
-// in the cube, 0 when xi lies outside it, -1 when the steps do not shrink
-// fast.
+// rho from the last two) at most 1e-15.  Returns 1 with xi in the cube, 0 when
+// xi lies outside it, -1 when the steps do not shrink fast or coordinates of
+// this size do not resolve xi that far (the FP64 iteration from the centre
+// decides then, is_far).
 template <int K>
 __device__ __forceinline__ int polish_in(const MappedDev& md, const Tables& tb, int64_t e,
                                          const double p[3],
@@ -485,7 +506,14 @@ __device__ __forceinline__ int polish_in(const MappedDev& md, const Tables& tb, 
   const float4* Pl = md.rel_lo + e * NL;
   const double* rf = md.ref + 4 * e;
   const double inv = rf[3];
-  const bool near = fmax(fmax(fabs(p[0]), fabs(p[1])), fabs(p[2])) * inv <= 256.0;
+  {
+    const float invf = (float)inv;
+    const float size[3] = {fabsf((float)p[0]) * invf, fabsf((float)p[1]) * invf,
+                           fabsf((float)p[2]) * invf};
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+      if (is_far(Ji[a], size)) return -1;
+  }
   df64 xi[3], q[3];
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
@@ -533,7 +561,7 @@ __device__ __forceinline__ int polish_in(const MappedDev& md, const Tables& tb, 
       big = fmaxf(big, fabsf(d));
     }
     if (!(big <= 0.1f * prev || big <= 1e-13f)) return -1;  // also NaN
-    if (big <= 1e-13f || (near && it > 0 && big * (big / prev) <= 1e-15f)) {
+    if (big <= 1e-13f || (it > 0 && big * (big / prev) <= 1e-15f)) {
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
         xi_out[a] = (double)xi[a].hi + (double)xi[a].lo;
@@ -552,8 +580,22 @@ __device__ __forceinline__ int polish_in(const MappedDev& md, const Tables& tb, 
   return -1;
 }
 
-// Newton inversion of the map of element e at p (see the file comment);
-// returns true with xi in the cube, else false
+// determinant by cofactors of the first row, each operation rounded
+__device__ __forceinline__ double det3_rn(const double M[3][3]) {
+  double m[3];
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    const int p = j == 0 ? 1 : 0, q = j == 2 ? 1 : 2;
+    m[j] = __dmul_rn(M[0][j], __dsub_rn(__dmul_rn(M[1][p], M[2][q]), __dmul_rn(M[1][q], M[2][p])));
+  }
+  return __dadd_rn(__dsub_rn(m[0], m[1]), m[2]);
+}
+
+// Newton inversion of the map of element e at p (see the file comment), every
+// operation rounded as the definition states it (node by node, no contraction
+// into FMA): far from the origin, where coordinates do not resolve xi to
+// 1e-13, the roundings decide whether a step of 1e-13 is ever taken, and they
+// have to be the definition's.  Returns true with xi in the cube, else false.
 template <int K>
 __device__ __noinline__ bool newton_in(const MappedDev& md, const Tables& tb, int64_t e,
                                        const double p[3], double xi_out[3]) {
@@ -563,46 +605,46 @@ __device__ __noinline__ bool newton_in(const MappedDev& md, const Tables& tb, in
   for (int it = 0; it < 50; ++it) {
     double l[3][NQ], dl[3][NQ];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) cfdem::lagrange<K, double>(tb.z, tb.lw, xi[a], l[a], dl[a]);
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+      for (int j = 0; j < NQ; ++j) {
+        double v = 1.0, dv = 0.0;
+#pragma unroll
+        for (int b = 0; b < NQ; ++b) {
+          if (b == j) continue;
+          const double den = __dsub_rn(tb.z[j], tb.z[b]), t = __dsub_rn(xi[a], tb.z[b]);
+          dv = __dadd_rn(__ddiv_rn(__dmul_rn(dv, t), den), __ddiv_rn(v, den));
+          v = __ddiv_rn(__dmul_rn(v, t), den);
+        }
+        l[a][j] = v;
+        dl[a][j] = dv;
+      }
     double X[3] = {0.0, 0.0, 0.0}, J[3][3] = {{0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}};
-    // sum factorised: x, then y, then z
 #pragma unroll
-    for (int c = 0; c < NQ; ++c) {
-      double u[3] = {0.0, 0.0, 0.0}, u0[3] = {0.0, 0.0, 0.0}, u1[3] = {0.0, 0.0, 0.0};
+    for (int c = 0; c < NQ; ++c)
 #pragma unroll
-      for (int b = 0; b < NQ; ++b) {
-        double v[3] = {0.0, 0.0, 0.0}, v0[3] = {0.0, 0.0, 0.0};
+      for (int b = 0; b < NQ; ++b)
 #pragma unroll
         for (int a = 0; a < NQ; ++a) {
-          const double* P = md.nodes + 3 * (int64_t)cn[a + NQ * (b + NQ * c)];
+          const double* P = md.nodes + 3 * (int64_t)__ldg(cn + a + NQ * (b + NQ * c));
+          const double w = __dmul_rn(__dmul_rn(l[0][a], l[1][b]), l[2][c]);
+          const double w0 = __dmul_rn(__dmul_rn(dl[0][a], l[1][b]), l[2][c]);
+          const double w1 = __dmul_rn(__dmul_rn(l[0][a], dl[1][b]), l[2][c]);
+          const double w2 = __dmul_rn(__dmul_rn(l[0][a], l[1][b]), dl[2][c]);
 #pragma unroll
           for (int i = 0; i < 3; ++i) {
             const double Pi = __ldg(P + i);
-            v[i] += l[0][a] * Pi;
-            v0[i] += dl[0][a] * Pi;
+            X[i] = __dadd_rn(X[i], __dmul_rn(w, Pi));
+            J[i][0] = __dadd_rn(J[i][0], __dmul_rn(w0, Pi));
+            J[i][1] = __dadd_rn(J[i][1], __dmul_rn(w1, Pi));
+            J[i][2] = __dadd_rn(J[i][2], __dmul_rn(w2, Pi));
           }
         }
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-          u[i] += l[1][b] * v[i];
-          u0[i] += l[1][b] * v0[i];
-          u1[i] += dl[1][b] * v[i];
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        X[i] += l[2][c] * u[i];
-        J[i][0] += l[2][c] * u0[i];
-        J[i][1] += l[2][c] * u1[i];
-        J[i][2] += dl[2][c] * u[i];
-      }
-    }
-    const double r[3] = {X[0] - p[0], X[1] - p[1], X[2] - p[2]};
-    const double det = J[0][0] * (J[1][1] * J[2][2] - J[1][2] * J[2][1]) -
-                       J[0][1] * (J[1][0] * J[2][2] - J[1][2] * J[2][0]) +
-                       J[0][2] * (J[1][0] * J[2][1] - J[1][1] * J[2][0]);
+    const double r[3] = {__dsub_rn(X[0], p[0]), __dsub_rn(X[1], p[1]), __dsub_rn(X[2], p[2])};
+    const double det = det3_rn(J);
     if (!(fabs(det) > 0.0)) return false;
-    double d[3];
+    double big = 0.0;
+    bool inside = true;
 #pragma unroll
     for (int col = 0; col < 3; ++col) {  // Cramer's rule
       double M[3][3];
@@ -610,18 +652,10 @@ __device__ __noinline__ bool newton_in(const MappedDev& md, const Tables& tb, in
       for (int i = 0; i < 3; ++i)
 #pragma unroll
         for (int j = 0; j < 3; ++j) M[i][j] = j == col ? r[i] : J[i][j];
-      const double dm = M[0][0] * (M[1][1] * M[2][2] - M[1][2] * M[2][1]) -
-                        M[0][1] * (M[1][0] * M[2][2] - M[1][2] * M[2][0]) +
-                        M[0][2] * (M[1][0] * M[2][1] - M[1][1] * M[2][0]);
-      d[col] = dm / det;
-    }
-    double big = 0.0;
-    bool inside = true;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      xi[a] -= d[a];
-      big = fmax(big, fabs(d[a]));
-      inside = inside && xi[a] >= -3.0 && xi[a] <= 4.0;
+      const double d = __ddiv_rn(det3_rn(M), det);
+      xi[col] = __dsub_rn(xi[col], d);
+      big = fmax(big, fabs(d));
+      inside = inside && xi[col] >= -3.0 && xi[col] <= 4.0;
     }
     if (!inside) return false;
     if (big <= 1e-13) {
@@ -697,7 +731,7 @@ k_locate_mapped(MappedDev md, Tables tb, int64_t n, const double* __restrict__ x
     float q[3], start[3], Ji[3][3], step = 0.0f, det0 = 0.0f;
     if (!done)
       while ((e = next()) >= 0 &&
-             (sc = screen_hull(md, e, p, q, start, &step, &det0)) == kOutside) {
+             (sc = screen_hull(md, e, p, pf, q, start, &step, &det0)) == kOutside) {
       }
     __syncwarp();
     done = done || e < 0;
