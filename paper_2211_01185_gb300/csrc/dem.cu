@@ -34,15 +34,18 @@
 // One thread per particle (the form before) left every lane to its own
 // serial chain of 6 to 12 contacts of ~300 dependent operations, and a bed of
 // 5,000 spheres 157 warps for 152 SMs.  Per sub-step, 100,000 spheres on the
-// mixed path 154 -> 90 us (contact kernel 120 -> 63 us, now bound by the
-// latency of its gathers at 64 % of the warps), 5,003 spheres in FP64 190 ->
-// 60 us (181 -> 43 us, bound by the FP64 pipe).
+// mixed path 154 -> 96 us (contact kernel 120 -> 71 us, bound by the latency
+// of its gathers at 64 % of the warps and by the FP64 pipe), 5,003 spheres in
+// FP64 190 -> 60 us (181 -> 43 us, bound by the FP64 pipe).
 //
 // Each particle keeps its own copy of a pair's d_t (the partner's is its
 // negative), so i and j never write the same word.  The state is FP64; the
-// contact arithmetic is FP64 or, on the mixed path, FP32 on differences of
-// double-float positions and velocities (FP64 instructions, conversions
-// among them, issue at 1/64 of the FP32 rate here).
+// contact arithmetic is FP64 or, on the mixed path, FP32 on FP64 differences of
+// positions and velocities and an FP64 contact test: eleven FP64 instructions a
+// contact, their results made FP32 by moves of bit fields (FP64 instructions,
+// conversions among them, issue at 1/64 of the FP32 rate here).  Double-float
+// copies in their place take 63 us, but lose the overlap's digits in large
+// boxes (dem_pair).
 #include <algorithm>
 #include <cmath>
 #include <cstdarg>
@@ -67,19 +70,20 @@ struct DemDev {
   double rmax;
   int nc[3];                            // cells per axis
   float inv_ce[3];                      // 1 / cell edge
-  df64 ext[3];                          // hi - lo
   int cap;                              // contacts per particle
 };
 
 // The constants of a kind of contact (particle-particle, particle-wall):
-// effective Young's and shear moduli, -2 sqrt(5/6) beta(e) sqrt(2 Y_e) and
-// ... sqrt(8 G_e), so that eta_n and eta_t share one root, the friction
-// coefficients, and the mass of a particle of radius 1.  Kept in the type of
+// effective Young's and shear moduli, -2 sqrt(5/6) beta(e) sqrt(2 Y_e m) and
+// ... sqrt(8 G_e m), so that eta_n and eta_t share one root, the friction
+// coefficients, and the relative mass of a particle of radius 1.  Masses are
+// taken relative to the mass m of a particle of the largest radius: products
+// of masses in kg leave FP32's exponents for particles of nanometres.  Kept in the type of
 // the arithmetic: converting a kernel argument from FP64 is an FP64-pipe
 // instruction of its own.
 template <typename R>
 struct Contact {
-  R Ye, Ge, en, et, mus, mur, mass1;
+  R Ye, Ge, en, et, mus, mur, cube;
 };
 
 // One contact's force F and torque Tq on particle i, advancing the carried
@@ -141,8 +145,9 @@ __device__ __forceinline__ int cell_axis(double x, double lo, float inv_ce, int 
   return t >= 1.0f ? (t < (float)nc ? (int)t : nc - 1) : 0;  // NaN to 0
 }
 
-// The Velocity Verlet updates, with explicit FMAs so that the forces' kernel
-// and the one below give the same bits.
+// The Velocity Verlet updates, with explicit FMAs so that the opening half
+// kick and drift give the same bits at the start of a call (k_dem_begin) and
+// between two sub-steps (k_dem_advance).
 __device__ __forceinline__ void half_kick(double hdt, double a, double& v) { v = fma(hdt, a, v); }
 
 // cell of a position (cell_axis per axis)
@@ -248,17 +253,31 @@ k_dem_ranges(int ncells, int tile, const int32_t* __restrict__ count, int32_t* _
 }
 
 // The state in cell order, for the contacts.  xs: FP32 position (offset from
-// the box's low corner) and radius, for the screen and as the high parts on
-// the mixed path.
+// the box's low corner) and radius, for the screen.
 struct DemCells {
   float4* xs;
   int32_t* perm;   // particle at each place
   int32_t* cell;   // and its cell
-  // mixed: low parts of position and radius, high and low parts of the
-  // velocity, angular velocity; FP64: position and radius, v, w
-  float4 *xl, *vh, *vl, *wf;
-  double2 *xr, *vw;  // [n][2], [n][3]
+  double2* xr;     // [n][2] position and radius
+  double2* vw;     // FP64: [n][3] v, w; mixed: [n][2] v
+  float4* wf;      // mixed: w
 };
+
+// v in FP32 by moves of bit fields (a conversion is an FP64-pipe instruction):
+// half a unit of the 24th significand bit added (a carry moves into the
+// exponent as it should; ties round away), the leading bits moved down, and the
+// exponent's bias changed by 896 -- 3 x 256, which the move drops, and 128, the
+// flip of its top bit.  Zero, and values whose float is not normal, take the
+// conversion, as a real call.
+static __device__ __noinline__ float f32_convert(double v) { return (float)v; }
+__device__ __forceinline__ float f32_of(double v) {
+  unsigned lo, hi;
+  double_halves(v, &lo, &hi);
+  if ((hi & 0x7fffffffu) - 0x38100000u >= 0x0fd00000u) return f32_convert(v);
+  const unsigned l = lo + 0x10000000u, h = hi + (l < lo ? 1u : 0u);
+  const unsigned m = __funnelshift_l(l, h, 3);
+  return __uint_as_float((hi & 0x80000000u) | ((m & 0x7fffffffu) ^ 0x40000000u));
+}
 
 template <typename R>
 __global__ void k_dem_cell_scatter(int64_t n, DemDev p, const double* __restrict__ x,
@@ -279,28 +298,18 @@ __global__ void k_dem_cell_scatter(int64_t n, DemDev p, const double* __restrict
   const double vd[3] = {v[3 * i], v[3 * i + 1], v[3 * i + 2]};
   const double wd[3] = {w[3 * i], w[3 * i + 1], w[3 * i + 2]};
   const double rd = r[i];
+  cs.xr[2 * (int64_t)s] = make_double2(xd[0], xd[1]);
+  cs.xr[2 * (int64_t)s + 1] = make_double2(xd[2], rd);
+  cs.xs[s] = make_float4((float)(xd[0] - p.lo[0]), (float)(xd[1] - p.lo[1]),
+                         (float)(xd[2] - p.lo[2]), (float)rd);
   if (std::is_same<R, double>::value) {
-    cs.xs[s] = make_float4((float)(xd[0] - p.lo[0]), (float)(xd[1] - p.lo[1]),
-                           (float)(xd[2] - p.lo[2]), (float)rd);
-    cs.xr[2 * (int64_t)s] = make_double2(xd[0], xd[1]);
-    cs.xr[2 * (int64_t)s + 1] = make_double2(xd[2], rd);
     cs.vw[3 * (int64_t)s] = make_double2(vd[0], vd[1]);
     cs.vw[3 * (int64_t)s + 1] = make_double2(vd[2], wd[0]);
     cs.vw[3 * (int64_t)s + 2] = make_double2(wd[1], wd[2]);
   } else {
-    df64 q[4], u[3], om[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      q[a] = df_from_double_int(xd[a] - p.lo[a]);
-      u[a] = df_from_double_int(vd[a]);
-      om[a] = df_from_double_int(wd[a]);
-    }
-    q[3] = df_from_double_int(rd);
-    cs.xs[s] = make_float4(q[0].hi, q[1].hi, q[2].hi, q[3].hi);
-    cs.xl[s] = make_float4(q[0].lo, q[1].lo, q[2].lo, q[3].lo);
-    cs.vh[s] = make_float4(u[0].hi, u[1].hi, u[2].hi, 0.0f);
-    cs.vl[s] = make_float4(u[0].lo, u[1].lo, u[2].lo, 0.0f);
-    cs.wf[s] = make_float4(om[0].hi + om[0].lo, om[1].hi + om[1].lo, om[2].hi + om[2].lo, 0.0f);
+    cs.vw[2 * (int64_t)s] = make_double2(vd[0], vd[1]);
+    cs.vw[2 * (int64_t)s + 1] = make_double2(vd[2], 0.0);
+    cs.wf[s] = make_float4((float)wd[0], (float)wd[1], (float)wd[2], 0.0f);
   }
 }
 
@@ -310,10 +319,7 @@ __device__ __forceinline__ float abs_max3(float4 q) {
 }
 
 // a particle at a place of the cell order, as the contacts use it
-template <typename R>
-struct Body;
-template <>
-struct Body<double> {
+struct Body {
   double x[3], r;
   __device__ __forceinline__ void load(const DemCells& cs, int64_t s) {
     const double2 a = __ldg(cs.xr + 2 * s), b = __ldg(cs.xr + 2 * s + 1);
@@ -322,25 +328,27 @@ struct Body<double> {
     x[2] = b.x;
     r = b.y;
   }
-};
-template <>
-struct Body<float> {
-  df64 x[3], r;
-  __device__ __forceinline__ void load(const DemCells& cs, int64_t s) {
-    const float4 h = __ldg(cs.xs + s), l = __ldg(cs.xl + s);
-    x[0] = df64(h.x, l.x);
-    x[1] = df64(h.y, l.y);
-    x[2] = df64(h.z, l.z);
-    r = df64(h.w, l.w);
+  // the radius in the type of the contact's arithmetic
+  __device__ __forceinline__ double radius(const DemCells&, int64_t, double) const { return r; }
+  __device__ __forceinline__ float radius(const DemCells& cs, int64_t s, float) const {
+    return __ldg(&cs.xs[s].w);
   }
 };
 
+// v > 0 by its bits, without an FP64 compare (false for NaN)
+__device__ __forceinline__ bool above_zero(double v) {
+  unsigned lo, hi;
+  double_halves(v, &lo, &hi);
+  return (int)hi >= 0 && (hi | lo) != 0u && (hi < 0x7ff00000u || (hi == 0x7ff00000u && lo == 0u));
+}
+
 // The contact test of a pair: n from i to j and the overlap.  FP64: |d| > 0
 // and |d| < r_i + r_j on the root.  Mixed: the overlap is (rs^2 - d^2) /
-// (rs + d) with the difference of squares in double-float, so the small
-// overlap keeps its digits.
-__device__ __forceinline__ bool dem_pair(const Body<double>& a, const Body<double>& b, double* nrm,
-                                         double* dn) {
+// (rs + d) with the positions' differences and the difference of squares in
+// FP64, so that the small overlap keeps its digits however large the box is
+// (eight FP64 instructions a pair; from double-float copies of the positions
+// an overlap of 1e-6 r in a box of 2,000 r was off by up to 7e-5).
+__device__ __forceinline__ bool dem_pair(const Body& a, const Body& b, double* nrm, double* dn) {
   const double d[3] = {b.x[0] - a.x[0], b.x[1] - a.x[1], b.x[2] - a.x[2]};
   const double dist = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
   const double rs = a.r + b.r;
@@ -351,18 +359,17 @@ __device__ __forceinline__ bool dem_pair(const Body<double>& a, const Body<doubl
   *dn = rs - dist;
   return true;
 }
-__device__ __forceinline__ bool dem_pair(const Body<float>& a, const Body<float>& b, float* nrm,
-                                         float* dn) {
-  const df64 d[3] = {b.x[0] - a.x[0], b.x[1] - a.x[1], b.x[2] - a.x[2]};
-  const df64 d2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-  const df64 rs = a.r + b.r;
-  const df64 over = rs * rs - d2;
-  if (!((over.hi > 0.0f || (over.hi == 0.0f && over.lo > 0.0f)) && d2.hi > 0.0f)) return false;
-  const float dist = sqrtf(d2.hi);
+__device__ __forceinline__ bool dem_pair(const Body& a, const Body& b, float* nrm, float* dn) {
+  const double d[3] = {b.x[0] - a.x[0], b.x[1] - a.x[1], b.x[2] - a.x[2]};
+  const double d2 = fma(d[2], d[2], fma(d[1], d[1], d[0] * d[0]));
+  const double rs = a.r + b.r;
+  const float over = f32_of(fma(rs, rs, -d2)), d2f = f32_of(d2);
+  if (!(over > 0.0f && d2f > 0.0f)) return false;
+  const float dist = sqrtf(d2f);
   const float inv = 1.0f / dist;
 #pragma unroll
-  for (int c = 0; c < 3; ++c) nrm[c] = d[c].hi * inv;
-  *dn = over.hi / (rs.hi + dist);
+  for (int c = 0; c < 3; ++c) nrm[c] = f32_of(d[c]) * inv;
+  *dn = over / (f32_of(rs) + dist);
   return true;
 }
 
@@ -384,19 +391,21 @@ __device__ __forceinline__ void dem_relative(const DemCells& cs, int64_t s, int6
 #pragma unroll
   for (int a = 0; a < 3; ++a) dv[a] = vi[a] - vj[a];
 }
+// mixed: the difference in FP64, then FP32
+__device__ __forceinline__ void dem_spin(const DemCells& cs, int64_t s, float* w) {
+  const float4 a = __ldg(cs.wf + s);
+  w[0] = a.x;
+  w[1] = a.y;
+  w[2] = a.z;
+}
 __device__ __forceinline__ void dem_relative(const DemCells& cs, int64_t s, int64_t q, float* dv,
                                              float* wi, float* wj) {
-  const float4 hi = __ldg(cs.vh + s), li = __ldg(cs.vl + s), hj = __ldg(cs.vh + q),
-               lj = __ldg(cs.vl + q), a = __ldg(cs.wf + s), b = __ldg(cs.wf + q);
-  dv[0] = (hi.x - hj.x) + (li.x - lj.x);
-  dv[1] = (hi.y - hj.y) + (li.y - lj.y);
-  dv[2] = (hi.z - hj.z) + (li.z - lj.z);
-  wi[0] = a.x;
-  wi[1] = a.y;
-  wi[2] = a.z;
-  wj[0] = b.x;
-  wj[1] = b.y;
-  wj[2] = b.z;
+  const double2 a = __ldg(cs.vw + 2 * s), b = __ldg(cs.vw + 2 * q);
+  dv[0] = f32_of(a.x - b.x);
+  dv[1] = f32_of(a.y - b.y);
+  dv[2] = f32_of(__ldg(&cs.vw[2 * s + 1].x) - __ldg(&cs.vw[2 * q + 1].x));
+  dem_spin(cs, s, wi);
+  dem_spin(cs, q, wj);
 }
 // own velocity and angular velocity, and the overlap with wall `wl` (x-, x+,
 // y-, ...; positive in contact)
@@ -404,27 +413,24 @@ __device__ __forceinline__ void dem_own(const DemCells& cs, int64_t s, double* v
   dem_motion(cs, s, v, w);
 }
 __device__ __forceinline__ void dem_own(const DemCells& cs, int64_t s, float* v, float* w) {
-  const float4 h = __ldg(cs.vh + s), l = __ldg(cs.vl + s), a = __ldg(cs.wf + s);
-  v[0] = h.x + l.x;
-  v[1] = h.y + l.y;
-  v[2] = h.z + l.z;
-  w[0] = a.x;
-  w[1] = a.y;
-  w[2] = a.z;
+  const double2 a = __ldg(cs.vw + 2 * s);
+  v[0] = f32_of(a.x);
+  v[1] = f32_of(a.y);
+  v[2] = f32_of(__ldg(&cs.vw[2 * s + 1].x));
+  dem_spin(cs, s, w);
 }
-__device__ __forceinline__ double wall_overlap(const DemDev& p, const Body<double>& b, int wl) {
+__device__ __forceinline__ double wall_overlap(const DemDev& p, const Body& b, int wl) {
   const double xa = wl < 2 ? b.x[0] : (wl < 4 ? b.x[1] : b.x[2]);
   const double lo = wl < 2 ? p.lo[0] : (wl < 4 ? p.lo[1] : p.lo[2]);
   const double hi = wl < 2 ? p.hi[0] : (wl < 4 ? p.hi[1] : p.hi[2]);
-  return wl & 1 ? b.r - (hi - xa) : b.r - (xa - lo);
+  return b.r - (wl & 1 ? hi - xa : xa - lo);
 }
-__device__ __forceinline__ float wall_overlap(const DemDev& p, const Body<float>& b, int wl) {
-  const df64 xa = wl < 2 ? b.x[0] : (wl < 4 ? b.x[1] : b.x[2]);  // from the low corner
-  const df64 ext = wl < 2 ? p.ext[0] : (wl < 4 ? p.ext[1] : p.ext[2]);
-  return (wl & 1 ? b.r - (ext - xa) : b.r - xa).hi;
-}
-__device__ __forceinline__ double body_radius(const Body<double>& b) { return b.r; }
-__device__ __forceinline__ float body_radius(const Body<float>& b) { return b.r.hi + b.r.lo; }
+template <typename R>
+__device__ __forceinline__ R in_type(double v);
+template <>
+__device__ __forceinline__ double in_type<double>(double v) { return v; }
+template <>
+__device__ __forceinline__ float in_type<float>(double v) { return f32_of(v); }
 
 // contact lists of the last and of this evaluation: partners ascending, one -1
 // behind the last (C per particle), and their tangential displacements; the
@@ -484,8 +490,9 @@ k_dem_forces(int64_t n, DemDev p, Contact<R> k, Contact<R> kw, R dt,
   const float4 qi = __ldg(cs.xs + at);
   const float Mi = abs_max3(qi);
   constexpr float kScreen = 3.814697265625e-06f;  // 2^-18
-  Body<R> me_b;
+  Body me_b;
   me_b.load(cs, at);
+  const R rir = me_b.radius(cs, at, (R)0);
   const int cell = cs.cell[at];
   const int cyz = cell / p.nc[0], cx = cell - cyz * p.nc[0];
   const int cz = cyz / p.nc[1], cy = cyz - cz * p.nc[1];
@@ -511,7 +518,7 @@ k_dem_forces(int64_t n, DemDev p, Contact<R> k, Contact<R> kw, R dt,
   auto visit = [&](int s, bool exact) {
     if (s == (int)at || !screen(s)) return;
     if (exact) {
-      Body<R> o;
+      Body o;
       R nr[3], dn;
       o.load(cs, s);
       if (!dem_pair(me_b, o, nr, &dn)) return;
@@ -557,8 +564,7 @@ k_dem_forces(int64_t n, DemDev p, Contact<R> k, Contact<R> kw, R dt,
   __syncwarp();
 
   // ---- contacts, eight at a time; lanes 0..5 add the six components up
-  const R rir = body_radius(me_b);
-  const R mir = k.mass1 * rir * rir * rir;
+  const R mir = k.cube * rir * rir * rir;
   R sum = 0;
   int m = 0;  // contacts kept
   const int rounds = __reduce_max_sync(0xffffffffu, (unsigned)nc);
@@ -567,13 +573,14 @@ k_dem_forces(int64_t n, DemDev p, Contact<R> k, Contact<R> kw, R dt,
     bool on = c < nc;
     int32_t j = 0;
     int64_t q = 0;
-    R nrm[3], dn = 0;
-    Body<R> o;
+    R nrm[3], dn = 0, rj = 0;
+    Body o;
     if (on) {
       const int l = s_ord[grp][c];
       j = s_j[grp][l];
       q = s_at[grp][l];
       o.load(cs, q);
+      rj = o.radius(cs, q, (R)0);
       on = dem_pair(me_b, o, nrm, &dn);
     }
     const unsigned b = (__ballot_sync(0xffffffffu, on) >> base) & 0xffu;
@@ -595,8 +602,7 @@ k_dem_forces(int64_t n, DemDev p, Contact<R> k, Contact<R> kw, R dt,
         for (int a = 0; a < 3; ++a) th[a] = h.t_old[(i * C + old) * 3 + a];
       R wi[3], wj[3], vrel[3];
       dem_relative(cs, at, q, vrel, wi, wj);
-      const R rj = body_radius(o);
-      const R mj = k.mass1 * rj * rj * rj;
+      const R mj = k.cube * rj * rj * rj;
       const R me = mir * mj / (mir + mj);
       const R Re = rir * rj / (rir + rj);
       const R ws[3] = {rir * wi[0] + rj * wj[0], rir * wi[1] + rj * wj[1],
@@ -626,8 +632,8 @@ k_dem_forces(int64_t n, DemDev p, Contact<R> k, Contact<R> kw, R dt,
   if (live && lane == 0 && m < C) h.j_new[i * C + m] = -1;
 
   // ---- walls x-, x+, y-, y+, z-, z+: a lane each
-  const R dnw = lane < 6 ? wall_overlap(p, me_b, lane) : (R)-1;
-  const bool on = live && dnw > (R)0;
+  const double over = lane < 6 ? wall_overlap(p, me_b, lane) : -1.0;
+  const bool on = live && above_zero(over);
   const unsigned all = __ballot_sync(0xffffffffu, on);
   if (all) {
     const unsigned b = (all >> base) & 0xffu, had = live ? h.wmask[i] : 0u;
@@ -647,7 +653,7 @@ k_dem_forces(int64_t n, DemDev p, Contact<R> k, Contact<R> kw, R dt,
       if (had >> lane & 1u)
 #pragma unroll
         for (int a = 0; a < 3; ++a) th[a] = tw[a];
-      dem_contact<R>(nrm, dnw, vrel, wi, rir, mir, rir, kw, dt, th, F, Tq);
+      dem_contact<R>(nrm, in_type<R>(over), vrel, wi, rir, mir, rir, kw, dt, th, F, Tq);
 #pragma unroll
       for (int a = 0; a < 3; ++a) tw[a] = th[a];
     }
@@ -770,7 +776,7 @@ cfdem_status dcuda(cfdem_dem_t d, cudaError_t e, const char* where) {
 
 Contact<float> in_float(const Contact<double>& k) {
   return Contact<float>{(float)k.Ye, (float)k.Ge, (float)k.en, (float)k.et, (float)k.mus,
-                        (float)k.mur, (float)k.mass1};
+                        (float)k.mur, (float)k.cube};
 }
 
 #define DCK(expr, where)                                  \
@@ -879,16 +885,20 @@ cfdem_status cfdem_dem_set_params(cfdem_dem_t d, const cfdem_dem_params* p) {
     return -2.0 * std::sqrt(5.0 / 6.0) * (le / std::sqrt(le * le + kPi * kPi));
   };
   const double nu = p->poisson, nuw = p->wall_poisson;
+  // the radius of relative mass 1, and its mass
+  const double r1 = std::min(std::max(p->max_radius, 1e-10), 1e10);
+  const double cube = 1.0 / (r1 * r1 * r1);
+  const double mass = p->rho_p * (4.0 / 3.0 * kPi) * (r1 * r1 * r1);
   auto contact = [&](double Y2, double nu2, double e, double mus, double mur) {
     Contact<double> k{};
     k.Ye = 1.0 / ((1.0 - nu * nu) / p->youngs + (1.0 - nu2 * nu2) / Y2);
     k.Ge = 1.0 / (2.0 * (2.0 - nu) * (1.0 + nu) / p->youngs +
                   2.0 * (2.0 - nu2) * (1.0 + nu2) / Y2);
-    k.en = c56(e) * std::sqrt(2.0 * k.Ye);
-    k.et = c56(e) * std::sqrt(8.0 * k.Ge);
+    k.en = c56(e) * std::sqrt(2.0 * k.Ye * mass);
+    k.et = c56(e) * std::sqrt(8.0 * k.Ge * mass);
     k.mus = mus;
     k.mur = mur;
-    k.mass1 = p->rho_p * (4.0 / 3.0 * kPi);
+    k.cube = cube;
     return k;
   };
   d->pp = contact(p->youngs, nu, p->restitution, p->friction, p->rolling_friction);
@@ -900,7 +910,6 @@ cfdem_status cfdem_dem_set_params(cfdem_dem_t d, const cfdem_dem_params* p) {
     q.lo[a] = p->lo[a];
     q.hi[a] = p->hi[a];
     const double ext = p->hi[a] - p->lo[a];
-    q.ext[a] = df64((float)ext, (float)(ext - (double)(float)ext));
     double f = std::floor(ext / (2.0 * p->max_radius * (1.0 + 1.0 / 512.0)));
     int nc = f < 1.0 ? 1 : (f > 4096.0 ? 4096 : (int)f);
     q.nc[a] = nc;
@@ -998,12 +1007,9 @@ cfdem_status cfdem_dem_step(cfdem_dem_t d, int64_t n, double* x, double* v, doub
   cs.xs = d->xs;
   cs.perm = d->perm;
   cs.cell = d->pcell;
-  cs.xl = d->body;
-  cs.vh = d->body + d->cap_n;
-  cs.vl = d->body + 2 * d->cap_n;
-  cs.wf = d->body + 3 * d->cap_n;
   cs.xr = reinterpret_cast<double2*>(d->body);
   cs.vw = reinterpret_cast<double2*>(d->body + 2 * d->cap_n);
+  cs.wf = d->body + 4 * d->cap_n;
   int32_t* total = d->count;
   int32_t* cells[2] = {d->count + 1, d->count + 1 + ncells};
   int set = 0;
