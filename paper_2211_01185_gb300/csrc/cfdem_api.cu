@@ -1132,12 +1132,13 @@ namespace {
 // mixed path with many particles per node (large elements, dense beds):
 // split the nodal velocity and void fraction into double-float pairs once
 // per node instead of once per particle that reads them (the same split,
-// so the same bits); the buffer is allocated outside a stream capture
+// so the same bits); the buffer is allocated outside a stream capture.  The
+// kernels with the shear force take the FP64 values
 cfdem_status split_nodal(cfdem_t c, int64_t n, const double* u_nodal, const double* eps_nodal,
-                         ForceParams* fp) {
+                         bool shear, ForceParams* fp) {
   const MeshDev& m = c->mesh;
   const int64_t nq = (int64_t)(m.k + 1) * (m.k + 1) * (m.k + 1);
-  if (c->prm.precision != 1 || n * nq < 8 * m.n_nodes) return CFDEM_OK;
+  if (c->prm.precision != 1 || shear || n * nq < 8 * m.n_nodes) return CFDEM_OK;
   if (!c->nodal_df && !stream_capturing(c->stream))
     CK(grow(&c->nodal_df, 2 * (size_t)m.n_nodes), "forces");
   if (!c->nodal_df) return CFDEM_OK;
@@ -1167,7 +1168,7 @@ cfdem_status forces_with_event(cfdem_t c, int64_t n, const double* x, const doub
     CK(cudaMemsetAsync(c->src_max, 0, 3 * sizeof(unsigned long long), c->stream), "forces");
   c->timer.begin(kStageForces, c->stream);
   ForceParams fp = force_params(c);
-  s = split_nodal(c, n, u_nodal, eps_nodal, &fp);
+  s = split_nodal(c, n, u_nodal, eps_nodal, fp.shear, &fp);
   if (s != CFDEM_OK) return s;
   CK(launch_forces(m, c->tab, c->prm.precision, fp, n, x, r, u_p, u_nodal, p_nodal, eps_nodal,
                    f, f_drag, ps, c->st, c->stream),
@@ -1262,7 +1263,7 @@ cfdem_status cfdem_adjoint(cfdem_t c, int64_t n, const double* x, const double* 
     CK(cudaMemsetAsync(c->adj_geps, 0, sizeof(double) * m.n_nodes, c->stream), "adjoint");
   if (dJ_du) CK(cudaMemsetAsync(dJ_du, 0, sizeof(double) * 3 * m.n_nodes, c->stream), "adjoint");
   ForceParams fp = force_params(c);
-  s = split_nodal(c, n, u_nodal, eps_nodal, &fp);
+  s = split_nodal(c, n, u_nodal, eps_nodal, fp.shear && g_f, &fp);
   if (s != CFDEM_OK) return s;
   CK(launch_adj_forces(m, c->tab, c->prm.precision, fp, n, x, r, u_p, u_nodal,
                        p_nodal, eps_nodal, g_f, g_fdrag, dJ_dx, dJ_du, c->adj_geps, c->st,
