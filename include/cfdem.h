@@ -129,7 +129,10 @@ typedef struct {
     double stage_ms[8];
     int64_t stage_calls[8];
     int32_t timer_overflow;       /* 1 if more than 1024 pairs per stage were asked */
-    int64_t kernel_launches;      /* kernels launched by the library since set_timing */
+    int64_t kernel_launches;      /* kernels launched by the library since set_timing, those
+                                     of a solve's graph included; replays of a caller's or a
+                                     batch's graph and iterations that a solve's graph repeats
+                                     on the device are not counted */
     int32_t precond;              /* preconditioner in use: 0 Jacobi, 1 FDM */
     int32_t tile_shape;           /* operator tile in use, nodes: 0 16x8x8 (Q3 16x9x6), 1 22x13x4
                                      (Q2 22x14x4, Q3 19x15x6), 2 25x15x4 (Q2 25x10x6, Q3 25x15x3) */

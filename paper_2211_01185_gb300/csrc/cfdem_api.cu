@@ -24,7 +24,11 @@ using namespace cfdem;
 namespace cfdem {
 
 static std::atomic<long long> g_launches{0};
-void count_launches(int n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
+static thread_local long long t_launches = 0;  // of this thread
+void count_launches(int n) {
+  g_launches.fetch_add(n, std::memory_order_relaxed);
+  t_launches += n;
+}
 long long launches_total() { return g_launches.load(std::memory_order_relaxed); }
 
 void Timer::create() {
@@ -557,6 +561,21 @@ cudaError_t solve_part(cfdem_t c, SolvePart part, const double* b, double* x, cu
   return e;
 }
 
+// kernels of a graph, those of conditional bodies left out
+int kernel_nodes(cudaGraph_t g) {
+  size_t n = 0;
+  if (cudaGraphGetNodes(g, nullptr, &n) != cudaSuccess) return 0;
+  std::vector<cudaGraphNode_t> nodes(n);
+  if (cudaGraphGetNodes(g, nodes.data(), &n) != cudaSuccess) return 0;
+  int kernels = 0;
+  for (size_t i = 0; i < n; ++i) {
+    cudaGraphNodeType t;
+    if (cudaGraphNodeGetType(nodes[i], &t) == cudaSuccess && t == cudaGraphNodeTypeKernel)
+      ++kernels;
+  }
+  return kernels;
+}
+
 // The CG loop of an eager solve as a graph: the same launches as a captured
 // solve, with the device deciding how often to iterate, so that the host
 // neither waits for the convergence flag (two round trips of ~20 us with the
@@ -582,12 +601,15 @@ cfdem_status solve_graphed(cfdem_t c, const double* b, double* x, bool* done) {
     if (e == cudaSuccess) e = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeRelaxed);
     if (e == cudaSuccess) {
       c->cg.loop = c->loop_stream;
+      const long long before = t_launches;
       e = solve_part(c, kSolveLoop, b, x, c->cap_stream, &it, &outer, &rel, &conv);
       c->cg.loop = nullptr;
       cudaGraph_t g = nullptr;
       const cudaError_t ee = cudaStreamEndCapture(c->cap_stream, &g);
       if (e == cudaSuccess) e = ee;
+      count_launches((int)(before - t_launches));  // recorded, not launched
       if (e == cudaSuccess) e = cudaGraphInstantiate(&c->loop_exec, g, 0);
+      if (e == cudaSuccess) c->loop_kernels = kernel_nodes(g);
       if (g) cudaGraphDestroy(g);
     }
     if (e != cudaSuccess) {
@@ -600,6 +622,7 @@ cfdem_status solve_graphed(cfdem_t c, const double* b, double* x, bool* done) {
   c->cg.unread = 1;
   CK(solve_part(c, kSolveStart, b, x, c->stream, &it, &outer, &rel, &conv), "solve");
   CK(cudaGraphLaunch(c->loop_exec, c->stream), "solve");
+  count_launches(c->loop_kernels);
   CK(solve_part(c, kSolveFinish, b, x, c->stream, &it, &outer, &rel, &conv), "solve");
   c->stats_pending = true;
   *done = true;

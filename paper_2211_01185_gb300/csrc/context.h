@@ -84,6 +84,7 @@ struct cfdem_ctx {
   cudaGraphExec_t loop_exec = nullptr;
   unsigned loop_gen = 0;
   int loop_shape = -1;
+  int loop_kernels = 0;      // kernels it launches, bodies of its loop left out
   int loop_solves = 0;       // eager solves of this configuration so far
   bool loop_failed = false;  // the capture failed: this configuration stays eager
   unsigned gen = 0;                    // bumped by every change of mesh, parameters or timing
