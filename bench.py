@@ -10,13 +10,14 @@ fraction of ~0.53 in the lower 40 % (synthetic, seeded).
 The headline `value` is the mixed path (FP32 work, FP64 refinement of the
 projection) replayed as one CUDA graph per step, in particle-coupling updates
 per second; the FP64 path is timed the same way beside it, with the error of
-the mixed results against it.  The default run also reports, under
-`workloads`, the Q1 8x8x32 bed of 2,000 spheres, the Q3 24x24x96 bed of
-1,000,000 spheres, the 64-bed ensemble, the adjoint workload and the DEM
-step (fewer timed steps each).
+the mixed results against it.  The default run also times the Q1 8x8x32 bed of
+2,000 spheres, the Q3 24x24x96 bed of 1,000,000 spheres, the 64-bed ensemble,
+the adjoint workload and the DEM step (fewer timed steps each).  The printed
+line holds the headline and each other workload's time; --detail FILE writes
+stage times, rooflines and everything else that was measured.
 
 Usage: python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
-                       [--workload NAME] [--quick]
+                       [--workload NAME] [--quick] [--detail FILE]
 Under torchrun each rank runs an independent replica of the step on its own
 GPU (the step has no exchange between beds); value = all particles / max time.
 """
@@ -949,8 +950,37 @@ def run_profile(args):
     return 0
 
 
+# what the printed line carries (--detail writes everything)
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step",
+             "ms_per_step_median", "higher_is_better", "scaling", "vs_baseline", "dtype", "data",
+             "config", "run", "gpu_launches", "clocks", "e2e", "mixed_speedup_over_fp64",
+             "err_mixed_vs_fp64", "cpu_baseline")
+LINE_ROOFLINE = ("bound", "kernel", "achieved", "peak", "unit", "frac", "traffic",
+                 "ms_per_launch", "launches_per_step")
+LINE_MAX = 2600
+
+
+def headline(res):
+    """The one line of a run: the headline's keys, short enough to be kept whole
+    where only the end of a program's output is."""
+    d = {k: res[k] for k in LINE_KEYS if k in res}
+    if "roofline" in res:
+        d["roofline"] = {k: res["roofline"][k] for k in LINE_ROOFLINE if k in res["roofline"]}
+    wl = {k: v.get("ms_per_step", v.get("mixed", {}).get("ms_per_step"))
+          for k, v in res.get("workloads", {}).items()}
+    if wl:
+        d["workloads_ms_per_step"] = wl
+    line = json.dumps(d)
+    for k in ("cpu_baseline", "run", "workloads_ms_per_step", "roofline"):   # the least first
+        if len(line) <= LINE_MAX:
+            break
+        d.pop(k, None)
+        line = json.dumps(d)
+    return line
+
+
 def _summary(r):
-    """The keys of a secondary workload that the bench line carries."""
+    """The keys of a secondary workload that the detail carries."""
     keep = ("workload", "mesh", "particles", "nodes", "value", "ms_per_step", "steps",
             "mixed", "fp64", "mixed_speedup_over_fp64", "err_mixed_vs_fp64", "roofline",
             "step_hbm", "cpu_baseline", "solo_sequential", "solo_graphs", "graph_replayed",
@@ -968,6 +998,9 @@ def main():
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-e2e", action="store_true")
+    ap.add_argument("--detail", metavar="FILE",
+                    help="write everything measured to FILE (JSON): stage times, rooflines, "
+                         "both precisions and the other workloads")
     ap.add_argument("--quick", action="store_true",
                     help="the headline bed only (no secondary workloads)")
     ap.add_argument("--workload", default=WORKLOAD,
@@ -1044,7 +1077,10 @@ def main():
     if env.dist is not None:
         env.dist.barrier()
     if env.rank == 0:
-        print(json.dumps(res), flush=True)
+        if args.detail:
+            with open(args.detail, "w") as fh:
+                json.dump(res, fh, indent=1)
+        print(headline(res), flush=True)
     if env.dist is not None:
         env.dist.destroy_process_group()
     return 0
