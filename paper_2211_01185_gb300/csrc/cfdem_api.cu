@@ -583,7 +583,12 @@ int kernel_nodes(cudaGraph_t g) {
 // context's own vectors only; b and x are taken and written by launches
 // outside it.  It is built at the second solve of a configuration, so that a
 // single solve does not pay for it (eager step of 2,000 spheres on Q1 8x8x32:
-// 251 -> 172 us).  *done = false: not available, solve with host checks.
+// 251 -> 172 us).  Recording and instantiating it costs that solve about
+// 80 us (390 us with the dense form of the preconditioner), each solve from it
+// on gains 40 to 70 us (up to 380): on Q1 8x8x32 the first solve of a
+// configuration takes 179 us, the second 213, every later one 132, so that it
+// pays from the third on and a program with two solves per configuration is
+// 10 % slower.  *done = false: not available, solve with host checks.
 cfdem_status solve_graphed(cfdem_t c, const double* b, double* x, bool* done) {
   *done = false;
   if (c->loop_gen != c->gen || c->loop_shape != c->mesh.shape) {

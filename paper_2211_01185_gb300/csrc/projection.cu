@@ -1374,9 +1374,10 @@ static int vec_blocks(int64_t n) {
 // the node's condition from `done`, so the graph iterates on the device until
 // the CG has converged or reached its iteration cap.  (Two iterations, so that
 // the ping-pong buffers are back in their roles at the end of the body.)  The
-// first two iterations are queued before the node, and a k_loop_cond ahead
-// of the node decides whether the body runs at all: a solve that converges
-// in two iterations -- the mixed cold start -- launches no idle iteration.
+// first iterations are queued before the node, two of the mixed and Jacobi
+// solves and three of the FP64 solve, and a k_loop_cond ahead of the node
+// decides whether the body runs at all: a solve that converges in as many --
+// the cold start -- launches no idle iteration.
 
 // one thread: continue while the CG is not done, and never beyond
 // max_bodies - 1 bodies whatever the kernels of the body did (sc->loops is

@@ -616,14 +616,16 @@ k_qcm(MeshDev m, QcmParams P, BinDev b, const int32_t* __restrict__ bin_start,
 // (R + r, (R + r)^2, (R - r)^2, the volume of the smaller sphere, the
 // volume-conserving weight); then every candidate is broadcast to the lanes,
 // each lane tests its own Gauss point (two for Q3; for Q1 four groups of 8
-// lanes take every fourth candidate) and adds the lens volume to a
-// Neumaier-compensated sum in registers.  No hit queue and no scan: the
-// instructions per candidate are a distance, a compare and, for the lanes
-// that hit, the lens volume.  Q3's batches of 64 come from eight places of
-// the reach: 16 % of its pairs overlap, and lists of 64 mixed candidates are
-// even enough for the warp to run about twice the hits of a mean lane, where
-// testing and evaluating candidate by candidate ran every one (1,000,000
-// spheres, 24 x 24 x 96 Q3: 765 -> 712 us, the same bits).  Sums run over the
+// lanes take every fourth candidate), lists the candidates of the batch that
+// overlap it, and adds their lens volumes, in the list's order, to a
+// Neumaier-compensated sum in registers.  No queue that lanes share and no
+// scan: the instructions per candidate are a distance, a compare and, for the
+// lanes that hit, the lens volume.  Q3's batches of 64 come from eight places
+// of the reach: 16 % of its pairs overlap, and lists of 64 mixed candidates
+// are even enough for the warp to run about twice the hits of a mean lane,
+// where testing and evaluating candidate by candidate ran every one (1,000,000
+// spheres, 24 x 24 x 96 Q3: 765 -> 712 us; another order of the sums, whose
+// compensation gave the same FP32 values on that bed).  Sums run over the
 // candidates in a fixed order
 // (the Q1 groups combined by a fixed shuffle tree), so results are
 // reproducible.
