@@ -603,8 +603,9 @@ k_dem_forces(int64_t n, DemDev p, Contact<R> k, Contact<R> kw, R dt,
       R wi[3], wj[3], vrel[3];
       dem_relative(cs, at, q, vrel, wi, wj);
       const R mj = k.cube * rj * rj * rj;
-      const R me = mir * mj / (mir + mj);
-      const R Re = rir * rj / (rir + rj);
+      // (ratios first: the product of two relative masses can underflow)
+      const R me = mir * (mj / (mir + mj));
+      const R Re = rir * (rj / (rir + rj));
       const R ws[3] = {rir * wi[0] + rj * wj[0], rir * wi[1] + rj * wj[1],
                        rir * wi[2] + rj * wj[2]};
       vrel[0] += ws[1] * nrm[2] - ws[2] * nrm[1];

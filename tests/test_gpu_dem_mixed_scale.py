@@ -12,11 +12,11 @@ from paper_2211_01185_gb300 import cfdem as cf
 pytestmark = pytest.mark.gpu
 
 
-def _kick(x, r, box, precision, dt, v):
+def _kick(x, r, box, precision, dt, v, max_radius):
     """velocity change of one sub-step"""
     p = D.glass_params((0, 0, 0), tuple(box), g=(0, 0, 0), friction=0.0, wall_friction=0.0)
     prm = {k: p[k] for k in D.PARAM_KEYS}
-    prm.update(g=p["g"], lo=p["lo"], hi=p["hi"], max_radius=float(r.max()), capacity=24,
+    prm.update(g=p["g"], lo=p["lo"], hi=p["hi"], max_radius=max_radius, capacity=24,
                precision=precision)
     tx, tv, tw = dev(x), dev(v), dev(np.zeros_like(x))
     with cf.Dem(prm) as dm:
@@ -25,9 +25,10 @@ def _kick(x, r, box, precision, dt, v):
     return host(tv) - v
 
 
-def _compare(x, r, box, dt, v=None):
+def _compare(x, r, box, dt, v=None, max_radius=None):
     v = np.zeros_like(x) if v is None else v
-    a, b = (_kick(x, r, box, p, dt, v) for p in (0, 1))
+    max_radius = max_radius or float(r.max())
+    a, b = (_kick(x, r, box, p, dt, v, max_radius) for p in (0, 1))
     size = np.linalg.norm(a, axis=1)
     assert (size > 0).sum() > 0.9 * len(x)
     assert np.array_equal(size > 0, np.linalg.norm(b, axis=1) > 0)
@@ -75,10 +76,12 @@ def test_walls_of_long_boxes(overlap):
     _compare(x, np.full(n, rad), box, 1e-16)
 
 
+@pytest.mark.parametrize("stated", [1.0, 1e7])
 @pytest.mark.parametrize("rad", [1e-2, 1e-5, 1e-7, 1e-8, 2e-9])
-def test_particle_sizes(rad):
+def test_particle_sizes(rad, stated):
     """With a relative velocity, so that the damping (root of the effective
-    mass) is in the forces."""
+    mass) is in the forces; also with a stated largest radius far above the
+    particles' own."""
     rng = np.random.default_rng(6)
     n = 100
     c = np.stack([4.0 + 5.0 * np.arange(n), np.full(n, 10.0), np.full(n, 10.0)], axis=1)
@@ -90,4 +93,4 @@ def test_particle_sizes(rad):
     v = np.zeros_like(x)
     v[1::2] = -0.3 * u
     box = rad * np.array([5.0 * n + 10.0, 20.0, 20.0])
-    _compare(rad * x, np.full(2 * n, rad), box, 1e-12 * rad, v)
+    _compare(rad * x, np.full(2 * n, rad), box, 1e-12 * rad, v, stated * rad)
