@@ -37,7 +37,7 @@
 // 0.225 ms below, but up to twice the plain iteration's error on some meshes.
 // Far from the origin rounding decides where the plain iteration ends; there,
 // and on meshes of sizes beyond FP32's exponents, the candidates take it as it
-// is defined, operation by operation (is_far, newton_in), and the elements are
+// is defined, operation by operation (is_far, newton_far), and the elements are
 // the definition's at any distance.  120,000 points on a
 // Q2 cylinder of 5,280 elements: locate and interpolate a 3-vector 13.6 ms
 // with plain FP64 Newton, 0.328 ms now
@@ -284,7 +284,8 @@ __global__ void k_frames(int64_t E, const double* __restrict__ ref,
   for (int q = 0; q < 5; ++q) frame[5 * e + q] = f[q];
 }
 
-enum Screen { kOutside, kStart, kUnsure };
+// kUnsure: the FP64 iteration decides; kDefinition: as the definition states it
+enum Screen { kOutside, kStart, kUnsure, kDefinition };
 
 // How far rounding of coordinates of the size of p (|p| in half edges, a)
 // moves xi, in units of 2^-53: the largest row of |J^-1| a.  The definition's
@@ -300,15 +301,15 @@ __device__ __forceinline__ bool is_far(const float row[3], const float a[3]) {
 
 // The hull test of candidate e at p (pf: p in FP32); kStart: not excluded, and
 // xi is the first Newton iterate from the centre, `step` its step and det0 the
-// centre's determinant.  kUnsure: no FP32 screen for this element or this far
-// from the origin.
+// centre's determinant.  kDefinition: no FP32 screen for this element (flat or
+// of extreme size) or this far from the origin.
 __device__ __forceinline__ Screen screen_hull(const MappedDev& md, int64_t e, const double p[3],
                                               const float pf[3], float q[3], float xi[3],
                                               float* step, float* det0) {
   const float4* f = md.frame + 5 * e;
   const double* rf = md.ref + 4 * e;
   const float4 h = __ldg(f + 3);
-  if (h.w == 0.0f) return kUnsure;
+  if (h.w == 0.0f) return kDefinition;
   const double inv = rf[3];
 #pragma unroll
   for (int i = 0; i < 3; ++i) q[i] = (float)((p[i] - rf[i]) * inv);
@@ -331,7 +332,7 @@ __device__ __forceinline__ Screen screen_hull(const MappedDev& md, int64_t e, co
   }
   *step = big;
   *det0 = h.w;
-  return far ? kUnsure : (out ? kOutside : kStart);
+  return far ? kDefinition : (out ? kOutside : kStart);
 }
 
 // The FP32 Newton screen (see the file comment), from the hull test's first
@@ -493,9 +494,9 @@ __device__ __forceinline__ void fp64_step(const MappedDev& md, const Tables& tb,
 // FP32 inverse Jacobian.  A linear iteration with ratio rho ~ 1e-5: done when
 // the step is at most 1e-13, or the step that would follow it (step * rho,
 // rho from the last two) at most 1e-15.  Returns 1 with xi in the cube, 0 when
-// xi lies outside it, -1 when the steps do not shrink fast or coordinates of
-// this size do not resolve xi that far (the FP64 iteration from the centre
-// decides then, is_far).
+// xi lies outside it, -1 when the steps do not shrink fast (the FP64 iteration
+// from the centre decides then), -2 when coordinates of this size do not
+// resolve xi that far (the definition's does, is_far).
 template <int K>
 __device__ __forceinline__ int polish_in(const MappedDev& md, const Tables& tb, int64_t e,
                                          const double p[3],
@@ -512,7 +513,7 @@ __device__ __forceinline__ int polish_in(const MappedDev& md, const Tables& tb, 
                            fabsf((float)p[2]) * invf};
 #pragma unroll
     for (int a = 0; a < 3; ++a)
-      if (is_far(Ji[a], size)) return -1;
+      if (is_far(Ji[a], size)) return -2;
   }
   df64 xi[3], q[3];
 #pragma unroll
@@ -580,6 +581,91 @@ __device__ __forceinline__ int polish_in(const MappedDev& md, const Tables& tb, 
   return -1;
 }
 
+// Newton inversion of the map of element e at p (see the file comment), where
+// coordinates resolve xi: sum factorised, a third of the operations of the
+// definition's form below.  Returns true with xi in the cube, else false.
+template <int K>
+__device__ __noinline__ bool newton_in(const MappedDev& md, const Tables& tb, int64_t e,
+                                       const double p[3], double xi_out[3]) {
+  constexpr int NQ = K + 1, NL = NQ * NQ * NQ;
+  double xi[3] = {0.5, 0.5, 0.5};
+  const int32_t* cn = md.conn + e * NL;
+  for (int it = 0; it < 50; ++it) {
+    double l[3][NQ], dl[3][NQ];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) cfdem::lagrange<K, double>(tb.z, tb.lw, xi[a], l[a], dl[a]);
+    double X[3] = {0.0, 0.0, 0.0}, J[3][3] = {{0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}};
+    // sum factorised: x, then y, then z
+#pragma unroll
+    for (int c = 0; c < NQ; ++c) {
+      double u[3] = {0.0, 0.0, 0.0}, u0[3] = {0.0, 0.0, 0.0}, u1[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+      for (int b = 0; b < NQ; ++b) {
+        double v[3] = {0.0, 0.0, 0.0}, v0[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+        for (int a = 0; a < NQ; ++a) {
+          const double* P = md.nodes + 3 * (int64_t)cn[a + NQ * (b + NQ * c)];
+#pragma unroll
+          for (int i = 0; i < 3; ++i) {
+            const double Pi = __ldg(P + i);
+            v[i] += l[0][a] * Pi;
+            v0[i] += dl[0][a] * Pi;
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          u[i] += l[1][b] * v[i];
+          u0[i] += l[1][b] * v0[i];
+          u1[i] += dl[1][b] * v[i];
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        X[i] += l[2][c] * u[i];
+        J[i][0] += l[2][c] * u0[i];
+        J[i][1] += l[2][c] * u1[i];
+        J[i][2] += dl[2][c] * u[i];
+      }
+    }
+    const double r[3] = {X[0] - p[0], X[1] - p[1], X[2] - p[2]};
+    const double det = J[0][0] * (J[1][1] * J[2][2] - J[1][2] * J[2][1]) -
+                       J[0][1] * (J[1][0] * J[2][2] - J[1][2] * J[2][0]) +
+                       J[0][2] * (J[1][0] * J[2][1] - J[1][1] * J[2][0]);
+    if (!(fabs(det) > 0.0)) return false;
+    double d[3];
+#pragma unroll
+    for (int col = 0; col < 3; ++col) {  // Cramer's rule
+      double M[3][3];
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) M[i][j] = j == col ? r[i] : J[i][j];
+      const double dm = M[0][0] * (M[1][1] * M[2][2] - M[1][2] * M[2][1]) -
+                        M[0][1] * (M[1][0] * M[2][2] - M[1][2] * M[2][0]) +
+                        M[0][2] * (M[1][0] * M[2][1] - M[1][1] * M[2][0]);
+      d[col] = dm / det;
+    }
+    double big = 0.0;
+    bool inside = true;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      xi[a] -= d[a];
+      big = fmax(big, fabs(d[a]));
+      inside = inside && xi[a] >= -3.0 && xi[a] <= 4.0;
+    }
+    if (!inside) return false;
+    if (big <= 1e-13) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+        if (!(xi[a] >= -1e-10 && xi[a] <= 1.0 + 1e-10)) return false;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) xi_out[a] = fmin(fmax(xi[a], 0.0), 1.0);
+      return true;
+    }
+  }
+  return false;
+}
+
 // determinant by cofactors of the first row, each operation rounded
 __device__ __forceinline__ double det3_rn(const double M[3][3]) {
   double m[3];
@@ -591,13 +677,15 @@ __device__ __forceinline__ double det3_rn(const double M[3][3]) {
   return __dadd_rn(__dsub_rn(m[0], m[1]), m[2]);
 }
 
-// Newton inversion of the map of element e at p (see the file comment), every
-// operation rounded as the definition states it (node by node, no contraction
-// into FMA): far from the origin, where coordinates do not resolve xi to
-// 1e-13, the roundings decide whether a step of 1e-13 is ever taken, and they
-// have to be the definition's.  Returns true with xi in the cube, else false.
+// The same with every operation rounded as the definition states it (node by
+// node, no contraction into FMA), for candidates far from the origin: where
+// coordinates do not resolve xi to 1e-13, the roundings decide whether a step
+// of 1e-13 is ever taken, and they have to be the definition's.  (Not for all
+// doubtful candidates: a lane in 50 steps without a root holds the kernel, for
+// 7,131 points on a coarse Q3 cylinder 1.37 ms with the form above and 5.1 ms
+// with this one.)
 template <int K>
-__device__ __noinline__ bool newton_in(const MappedDev& md, const Tables& tb, int64_t e,
+__device__ __noinline__ bool newton_far(const MappedDev& md, const Tables& tb, int64_t e,
                                        const double p[3], double xi_out[3]) {
   constexpr int NQ = K + 1, NL = NQ * NQ * NQ;
   double xi[3] = {0.5, 0.5, 0.5};
@@ -738,9 +826,10 @@ k_locate_mapped(MappedDev md, Tables tb, int64_t n, const double* __restrict__ x
     if (!done && sc == kStart) sc = screen_newton<K>(md, e, q, step, det0, start, Ji);
     __syncwarp();
     if (!done && sc != kOutside) {
-      int in = -1;
+      int in = sc == kDefinition ? -2 : -1;
       if (sc == kStart) in = polish_in<K>(md, tb, e, p, start, Ji, xo);
-      if (in < 0) in = newton_in<K>(md, tb, e, p, xo) ? 1 : 0;
+      if (in == -1) in = newton_in<K>(md, tb, e, p, xo) ? 1 : 0;
+      if (in == -2) in = newton_far<K>(md, tb, e, p, xo) ? 1 : 0;
       if (in) {
         found = e;
         done = true;
